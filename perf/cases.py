@@ -292,8 +292,9 @@ def _set_tiling(ctx, tiling):
 def _stack(case, obs):
     """The residual-w stack of an interval: plane fit, moved components, planes and their spacing."""
     s, uvw = obs.sky, obs.uvw.reshape(-1, 3)
-    ab = torch.linalg.lstsq(uvw[:, :2], uvw[:, 2:]).solution[:, 0].cpu()
-    a, b = float(ab[0]), float(ab[1])
+    uu, uv, vv, uw, vw = (float((uvw[:, p] * uvw[:, q]).sum()) for p, q in ((0, 0), (0, 1), (1, 1), (0, 2), (1, 2)))
+    det = uu * vv - uv * uv
+    a, b = (uw * vv - vw * uv) / det, (vw * uu - uw * uv) / det
     l, m, flux = s.lms[:, 0], s.lms[:, 1], s.lms[:, 2]
     nm1 = torch.sqrt(1.0 - l * l - m * m) - 1.0
     lms = torch.stack([l + a * nm1, m + b * nm1, flux], 1)
