@@ -175,10 +175,13 @@ psc_status psc_uvw(int n_ant, const double *ant_enu_m, double lat_rad, double de
  * image zero-padded to Ng x Ng, G[gy][gx] = sum I[row][col]
  * exp(+2 pi i ((gx-Ng/2)(col-N/2) + (gy-Ng/2)(row-N/2)) / Ng).
  * image_dev: device float [N][N]; grid_out: device complex64 [Ng][Ng];
- * stream: cudaStream_t or NULL.  For N % 8 == 0 the two matrix products run
+ * stream: cudaStream_t or NULL.  Computed by FP32 FFTs in the output buffer
+ * wherever the odd part of Ng is at most 512 (or, for N % 8 != 0, at most N),
+ * with a temporary table of up to 8 Ng bytes unless Ng is a power of two.
+ * Other sizes are two matrix products: for N % 8 == 0
  * on the tensor cores in split bfloat16 (each FP32 operand as three bfloat16
  * parts, FP32 accumulation; error at FP32 rounding level; operands staged by
- * TMA) and need a temporary workspace of 6 N K + 24 Ng K bytes, K = N rounded
+ * TMA) with a temporary workspace of 6 N K + 24 Ng K bytes, K = N rounded
  * up to a multiple of 32; otherwise FP32 SIMT with a temporary complex64
  * [N][Ng].  Synchronises the stream before freeing the
  * workspace and returning; PSC_ERR_TIMEOUT if a tensor-core wait ran out. */

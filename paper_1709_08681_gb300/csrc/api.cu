@@ -497,11 +497,12 @@ psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void 
     void *ws = nullptr;
     int *err_dev = nullptr;
     int herr = 0;
-    cudaError_t e = cudaMalloc(&ws, model_grid_ws_bytes(gd->n_img, gd->n_grid));
+    const size_t ws_bytes = model_grid_ws_bytes(gd->n_img, gd->n_grid);
+    cudaError_t e = ws_bytes ? cudaMalloc(&ws, ws_bytes) : cudaSuccess;
     if (e == cudaSuccess) e = launch_model_grid(gd->n_img, gd->n_grid, image_dev, ws, (float2 *)grid_out, &err_dev, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaMemcpy(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaFree(ws);
+    if (e == cudaSuccess && err_dev) e = cudaMemcpy(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost);
+    if (ws) cudaFree(ws);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "psc_model_grid");
     if (herr) return fail(nullptr, PSC_ERR_TIMEOUT, "psc_model_grid: a tensor-core wait timed out");
     return PSC_OK;

@@ -228,8 +228,14 @@ size_t stencil_dyn_smem(int c_group, int max_tab_len, int stage);
 cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *prefix_dev, const FeatPair *pairs_dev,
                                   int n, long long total_blocks, int threads, size_t dyn, int max_bl, int max_ant,
                                   float sigma, cudaStream_t s);
+// Model grid of an image by FFT (grid_fft.cu), for the sizes that
+// model_grid_fft_ok takes; ws: model_grid_fft_ws_bytes(n_grid).
+bool model_grid_fft_ok(int n_img, int n_grid);
+size_t model_grid_fft_ws_bytes(int n_grid);
+cudaError_t model_grid_fft(int n_img, int n_grid, const float *image, void *ws, float2 *grid_out, cudaStream_t s);
 // Workspace (bytes) of launch_model_grid; the model grid goes to grid_out
-// and *err_dev points (inside ws) at a flag set if a tensor-core wait ran out.
+// and *err_dev points (inside ws) at a flag set if a tensor-core wait ran out
+// (nullptr when no tensor-core pass ran).
 size_t model_grid_ws_bytes(int n_img, int n_grid);
 // Model grid of n_comp point components (host [n_comp][stride] = l, m, S, and
 // with stride 4 also n - 1, which gives flux k the phase 2 pi wp (n_k - 1)) on
