@@ -1355,6 +1355,7 @@ struct psc_batch {
     size_t gather_bytes = 0;
     std::vector<size_t> lm_off;
     int total_bl = 0;
+    int max_ant = 0, max_bpb = 0;    // most antennas of a context, most records of a baseline
     int grid = 0;
     int threads = 128;           // fused-kernel block size: the widest context's shape
     bool stacked = false;        // every context reads a residual-w stack (else none does)
@@ -1414,7 +1415,7 @@ psc_status build_tables(psc_batch *b) {
     std::vector<const LMState *> st0(n);
     std::vector<const double *> lm0(n);
     size_t dyn = 0, lmd = 0;
-    int threads = 32;
+    int threads = 32, max_ant = 0, max_bpb = 0;
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
         threads = std::max(threads, eval_threads(c));
@@ -1433,9 +1434,13 @@ psc_status build_tables(psc_batch *b) {
         lm0[k] = c->d_lm0;
         dyn = std::max(dyn, eval_dyn_smem(ch_span(c), tab_stride(c, c->kv)));
         lmd = std::max(lmd, lm_smem_bytes(c->n_ant));
+        max_ant = std::max(max_ant, c->n_ant);
+        max_bpb = std::max(max_bpb, red[k].bpb);
     }
     b->total_bl = blp[n];
     b->threads = threads;
+    b->max_ant = max_ant;
+    b->max_bpb = max_bpb;
     b->eval_dyn = dyn;
     b->lm_dyn = lmd;
     // one fused kernel per persistent launch: the track kernel for all
@@ -1521,8 +1526,8 @@ psc_status enqueue_iteration(psc_batch *b) {
         PSC_BCUDA(b, cudaEventRecord(b->ev_pool[b->ev_used + 1], s));
         b->ev_used += 2;
     }
-    PSC_BCUDA(b, launch_reduce_batch(b->d_red, b->d_bl_prefix, n, b->total_bl, s));
-    PSC_BCUDA(b, launch_lm_update_batch(b->d_lm, n, b->lm_dyn, s));
+    PSC_BCUDA(b, launch_reduce_batch(b->d_red, b->d_bl_prefix, n, b->total_bl, b->max_bpb, b->max_ant, s));
+    PSC_BCUDA(b, launch_lm_update_batch(b->d_lm, n, b->lm_dyn, b->max_ant, s));
     return PSC_OK;
 }
 

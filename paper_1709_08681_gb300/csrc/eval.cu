@@ -527,14 +527,20 @@ __global__ void __launch_bounds__(kMaxThreads, kW ? 4 : 0) eval_kernel(const Eva
     }                                                 // brick loop
 }
 
-// Second stage (a): per-baseline sums over its bricks, one thread per
-// (baseline, sum), the bricks added in order (deterministic).  partials is
-// [kRed][n_bricks] with the bricks of baseline bl at [bl * bpb, (bl + 1) * bpb).
-// Batched form: the global baseline number runs over the baselines of all
-// contexts (bl_prefix).
+// Second stage (a): per-baseline sums over its bricks, kL threads per
+// (baseline, sum).  partials is [kRed][n_bricks] with the bricks of baseline bl
+// at [bl * bpb, (bl + 1) * bpb).  The order of the additions is the same for
+// either kL (eight strided sums, then a tree), so results do not depend on what
+// else a batch holds.  Batched form: the global baseline number runs over the
+// baselines of all contexts (bl_prefix).
+// kL = 8 where a baseline has more than 8 records: its chain of dependent loads
+// is what the pass costs (351 baselines of 300
+// records: 52 us by one thread, 10 us by 8).
+template <int kL>
 __global__ void bl_reduce_kernel(const RedArgs r0, const RedArgs *__restrict__ ra,
                                  const int *__restrict__ bl_prefix, int n_ctx) {
-    const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long gt = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kL;
+    const int l = threadIdx.x % kL;
     const int gb = (int)(gt / kRed), k = (int)(gt - (long long)gb * kRed);
     RedArgs r = r0;
     int bl = gb;
@@ -552,51 +558,84 @@ __global__ void bl_reduce_kernel(const RedArgs r0, const RedArgs *__restrict__ r
     if (r.skip != nullptr && *r.skip) return;
     const size_t nb = (size_t)r.n_bl * r.bpb;
     const double *p = r.partials + (size_t)k * nb + (size_t)bl * r.bpb;
-    double sum = 0.0;
-    for (int b = 0; b < r.bpb; ++b) sum += p[b];
-    r.blsum[(size_t)bl * kRed + k] = sum;
+    double sum;
+    if constexpr (kL == 8) {
+        sum = 0.0;
+        for (int b = l; b < r.bpb; b += 8) sum += p[b];
+        const unsigned group = 0xffu << (threadIdx.x & 24);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(group, sum, o);
+    } else if (r.bpb == 1) {
+        sum = p[0];
+    } else {
+        double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int b0 = 0; b0 < r.bpb; b0 += 8)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (b0 + j < r.bpb) s[j] += p[b0 + j];
+        sum = ((s[0] + s[4]) + (s[2] + s[6])) + ((s[1] + s[5]) + (s[3] + s[7]));
+    }
+    if (l == 0) r.blsum[(size_t)bl * kRed + k] = sum;
 }
 
 // Second stage (b): chi^2, per-antenna gradient and diagonal blocks, cross
-// blocks; ev = chi2 | g[2n] | H[3n] | X[4 nbl].  One block per context
-// (blockIdx.x indexes ra when batched), fixed order.
-__global__ void ev_kernel(const RedArgs r0, const RedArgs *__restrict__ ra) {
+// blocks; ev = chi2 | g[2n] | H[3n] | X[4 nbl].  blockIdx.x indexes ra when
+// batched; blockIdx.y = 0 sums chi^2, the other blocks take a warp per antenna
+// (its lanes over the partners, then a butterfly) and share the cross blocks.
+// Fixed order.  One block per context, a thread per antenna, took 199 us at 197
+// antennas and 17 us at 27: 15 and 6 now.
+constexpr int kEvWarps = 8;
+__global__ void __launch_bounds__(32 * kEvWarps) ev_kernel(const RedArgs r0, const RedArgs *__restrict__ ra) {
     const RedArgs r = ra != nullptr ? ra[blockIdx.x] : r0;
     if (r.skip != nullptr && *r.skip) return;
-    __shared__ double s_chi[kMaxThreads];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_ant = r.n_ant, n_bl = r.n_bl;
-    double chi = 0.0;
-    for (int bl = tid; bl < n_bl; bl += blockDim.x) {
+    if (blockIdx.y == 0) {
+        __shared__ double s_chi[32 * kEvWarps];
+        double chi = 0.0;
+#pragma unroll 4
+        for (int bl = tid; bl < n_bl; bl += 32 * kEvWarps) chi += r.blsum[(size_t)bl * kRed];
+        s_chi[tid] = chi;
+        __syncthreads();
+        for (int o = 16 * kEvWarps; o > 0; o >>= 1) {
+            if (tid < o) s_chi[tid] += s_chi[tid + o];
+            __syncthreads();
+        }
+        if (tid == 0) r.ev[0] = s_chi[0];
+        return;
+    }
+    // as many blocks as this context's antennas fill, whatever else the batch holds
+    const int by = blockIdx.y - 1, nby = (n_ant + kEvWarps - 1) / kEvWarps;
+    if (by >= nby) return;
+    for (int bl = by * 32 * kEvWarps + tid; bl < n_bl; bl += nby * 32 * kEvWarps) {
         const double *sb = r.blsum + (size_t)bl * kRed;
-        chi += sb[0];
         double *x = r.ev + 1 + 5 * (size_t)n_ant + 4 * (size_t)bl;
         x[0] = sb[11]; x[1] = sb[12]; x[2] = sb[13]; x[3] = sb[14];
     }
-    s_chi[tid] = chi;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (tid < o) s_chi[tid] += s_chi[tid + o];
-        __syncthreads();
+    const int an = by * kEvWarps + warp;
+    if (an >= n_ant) return;
+    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int o = lane; o < n_ant; o += 32) {
+        if (o == an) continue;
+        const int i = min(an, o), j = max(an, o);
+        const int bl = i * (2 * n_ant - i - 1) / 2 + (j - i - 1);
+        const double *sb = r.blsum + (size_t)bl * kRed + (an == i ? 0 : 2);
+        v[0] += sb[1];
+        v[1] += sb[2];
+        sb += an == i ? 0 : 1;
+        v[2] += sb[5];
+        v[3] += sb[6];
+        v[4] += sb[7];
     }
-    if (tid == 0) r.ev[0] = s_chi[0];
-    for (int an = tid; an < n_ant; an += blockDim.x) {
-        double g0 = 0, g1 = 0, h0 = 0, h1 = 0, h2 = 0;
-        for (int o = 0; o < n_ant; ++o) {
-            if (o == an) continue;
-            const int i = min(an, o), j = max(an, o);
-            const int bl = i * (2 * n_ant - i - 1) / 2 + (j - i - 1);
-            const double *sb = r.blsum + (size_t)bl * kRed;
-            if (an == i) {
-                g0 += sb[1]; g1 += sb[2]; h0 += sb[5]; h1 += sb[6]; h2 += sb[7];
-            } else {
-                g0 += sb[3]; g1 += sb[4]; h0 += sb[8]; h1 += sb[9]; h2 += sb[10];
-            }
-        }
-        r.ev[1 + 2 * an] = g0;
-        r.ev[2 + 2 * an] = g1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane == 0) {
+        r.ev[1 + 2 * an] = v[0];
+        r.ev[2 + 2 * an] = v[1];
         double *h = r.ev + 1 + 2 * (size_t)n_ant + 3 * (size_t)an;
-        h[0] = h0; h[1] = h1; h[2] = h2;
+        h[0] = v[2]; h[1] = v[3]; h[2] = v[4];
     }
 }
 
@@ -719,24 +758,29 @@ cudaError_t set_eval_smem(size_t dyn) {
     return cudaSuccess;
 }
 
-cudaError_t launch_reduce(const RedArgs &r, cudaStream_t s) {
-    const long long threads = (long long)r.n_bl * kRed;
-    bl_reduce_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(r, nullptr, nullptr, 0);
+namespace {
+cudaError_t reduce_launches(const RedArgs &r, const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl,
+                            int max_bpb, int max_ant, cudaStream_t s) {
+    const long long sums = (long long)total_bl * kRed;
+    if (max_bpb > 8)
+        bl_reduce_kernel<8><<<(unsigned)((8 * sums + 255) / 256), 256, 0, s>>>(r, ra_dev, bl_prefix_dev, n_ctx);
+    else
+        bl_reduce_kernel<1><<<(unsigned)((sums + 255) / 256), 256, 0, s>>>(r, ra_dev, bl_prefix_dev, n_ctx);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    ev_kernel<<<1, kMaxThreads, 0, s>>>(r, nullptr);
+    ev_kernel<<<dim3(n_ctx, 1 + (max_ant + kEvWarps - 1) / kEvWarps), 32 * kEvWarps, 0, s>>>(r, ra_dev);
     return cudaGetLastError();
 }
+}  // namespace
 
-cudaError_t launch_reduce_batch(const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl,
-                                cudaStream_t s) {
-    const long long threads = (long long)total_bl * kRed;
+cudaError_t launch_reduce(const RedArgs &r, cudaStream_t s) {
+    return reduce_launches(r, nullptr, nullptr, 1, r.n_bl, r.bpb, r.n_ant, s);
+}
+
+cudaError_t launch_reduce_batch(const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl, int max_bpb,
+                                int max_ant, cudaStream_t s) {
     RedArgs none{};
-    bl_reduce_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(none, ra_dev, bl_prefix_dev, n_ctx);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    ev_kernel<<<n_ctx, kMaxThreads, 0, s>>>(none, ra_dev);
-    return cudaGetLastError();
+    return reduce_launches(none, ra_dev, bl_prefix_dev, n_ctx, total_bl, max_bpb, max_ant, s);
 }
 
 }  // namespace psc

@@ -138,7 +138,7 @@ struct LMArgs {
     double *lm_trial;          // [n_ant][2] offsets of the next evaluation (EvalArgs::lm)
     const double *ev;          // evaluation at lm_trial: chi2 | g[2n] | H[3n] | X[4 nbl]
     double *cur;               // same layout, accepted evaluation
-    double *mat;               // [2n][2n] scratch for the damped full system (large systems)
+    double *mat;               // [2n][2n] scratch: L^-1 in FP32 and vectors (large systems), the FP64 matrix (fallback)
     float *mat32;              // [2n][2n] FP32 factor (large systems)
     double *rhs;               // [2n] scratch
     const int2 *pairs;
@@ -180,8 +180,8 @@ cudaError_t launch_eval_batch(const EvalArgs *args_dev, const long long *prefix_
                               cudaStream_t s);
 cudaError_t eval_batch_occupancy(int threads, size_t dyn, bool stacked, int *blocks_per_sm);
 cudaError_t launch_reduce(const RedArgs &r, cudaStream_t s);
-cudaError_t launch_reduce_batch(const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl,
-                                cudaStream_t s);
+cudaError_t launch_reduce_batch(const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl, int max_bpb,
+                                int max_ant, cudaStream_t s);
 // A° tables of every channel (ap_table_dev: the caller's table on the device
 // for PSC_AP_TABLE, else unused).
 cudaError_t launch_tables(const psc_aperture &ap, const double *ap_table_dev, const double *freq_dev, int nc,
@@ -194,8 +194,8 @@ inline double aperture_reach(int kind, double dl, double du, int support) {
 // Argument check of an aperture description (message in *why).
 bool aperture_ok(const psc_aperture *ap, const char **why);
 cudaError_t launch_lm_update(const LMArgs &a, cudaStream_t s);
-// Batched forms: one block per context (device arrays of LMArgs).
-cudaError_t launch_lm_update_batch(const LMArgs *la_dev, int n_ctx, size_t dyn, cudaStream_t s);
+// Batched forms (device arrays of LMArgs; max_ant: the most antennas of a context).
+cudaError_t launch_lm_update_batch(const LMArgs *la_dev, int n_ctx, size_t dyn, int max_ant, cudaStream_t s);
 cudaError_t launch_lm_restart_batch(const LMArgs *la_dev, const LMState *const *st0_dev,
                                     const double *const *lm0_dev, int n_ctx, cudaStream_t s);
 size_t lm_smem_bytes(int n_ant);
