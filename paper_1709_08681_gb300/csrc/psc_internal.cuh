@@ -94,6 +94,7 @@ struct StencilArgs {
     const float *w;
     float w_scale;
     double *partials;          // [56][n_bricks]
+    double *direct;            // nullptr, or [n_bl][56] written instead (one brick a baseline)
     int n_bl, nt, nc, ng, support, ov;
     float du;
     int t_tile, c_group, n_tt, n_cg, time_stride;   // n_tt counts the kept (strided) time steps
@@ -102,7 +103,8 @@ struct StencilArgs {
     int stage;                 // 1: stage the grid cells of a brick in shared memory when they fit
     long long n_bricks;
     float sigma;               // stencil spacing (rad)
-    int wpb;                   // 1: one brick per block; 4: bricks of one warp, four per block (shared tables)
+    int ring;                  // cells of a lane's ring row (features.cu); 0: taps read the grid
+    int wpb;                   // 1: one brick per block; 8: bricks of one warp, eight per block (shared tables)
 };
 
 // Per-pair outputs of a batched feature pass (psc_features_batch).
@@ -221,13 +223,15 @@ cudaError_t launch_step_max(const double *uvw, int nt, int n_bl, unsigned *out_b
 // Records msg as the context-free last error (psc_last_error(NULL)); returns st.
 psc_status set_global_error(psc_status st, const char *msg);
 cudaError_t launch_features(const StencilArgs &a, double *blsum, int n_ant, float *feat, cudaStream_t s);
-// Dynamic shared memory of one stencil block.
-size_t stencil_dyn_smem(int c_group, int max_tab_len, int stage);
+// Cells of a stencil block's ring rows (StencilArgs::ring) and its dynamic shared memory.
+int stencil_ring(const StencilArgs &a, int threads);
+size_t stencil_dyn_smem(const StencilArgs &a, int threads);
 // The stencil pass, per-baseline sums and features of n pairs in three launches
-// (device tables of StencilArgs, first-brick prefixes [n + 1] and FeatPair).
+// (device tables of StencilArgs, first-brick prefixes [n + 1] and FeatPair);
+// direct: every pair's pass writes the per-baseline sums itself.
 cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *prefix_dev, const FeatPair *pairs_dev,
                                   int n, long long total_blocks, int threads, size_t dyn, int max_bl, int max_ant,
-                                  float sigma, cudaStream_t s);
+                                  bool direct, float sigma, cudaStream_t s);
 // Model grid of an image by FFT (grid_fft.cu), for the sizes that
 // model_grid_fft_ok takes; ws: model_grid_fft_ws_bytes(n_grid).
 bool model_grid_fft_ok(int n_img, int n_grid);
