@@ -224,34 +224,134 @@ __global__ void split_dft_matrix_kernel(const double2 *__restrict__ W, int n, in
 // Component operands of the grid G[gy][gx] = sum_k S_k exp(2 pi i (u_gx l_k + v_gy m_k)),
 // u_g = v_g = (g - Ng/2) du, as the second tensor-core pass with
 // A[gx][k] = S_k exp(2 pi i u_gx l_k) and B[gy][k] = exp(2 pi i v_gy m_k): split planes
-// [3][Ng][kp] of the real and imaginary parts, phases from FP64 sincospi,
+// [3][rows][kp] of the real and imaginary parts, Ng rows of A and b_rows of B,
 // columns k >= n_comp zero (kp = n_comp rounded up to a multiple of the K chunk).
-__global__ void split_comp_kernel(const double *__restrict__ comp, int n_comp, int stride, double wp, int kp, int ng,
-                                  double du, bf16 *__restrict__ Ar, bf16 *__restrict__ Ai, bf16 *__restrict__ Br,
-                                  bf16 *__restrict__ Bi) {
-    const long long total = (long long)ng * kp;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const int g = (int)(e / kp), k = (int)(e % kp);
-        double ar = 0.0, ai = 0.0, br = 0.0, bi = 0.0;
-        if (k < n_comp) {
-            const double x = (double)(g - ng / 2) * du;
-            const double *ck = comp + (size_t)stride * k;
-            // flux phase of a w-plane: 2 pi wp (n - 1), folded into the u factor
-            const double wph = stride == 4 ? wp * ck[3] : 0.0;
-            double sn, cs;
-            sincospi(2.0 * (x * ck[0] + wph), &sn, &cs);
-            ar = ck[2] * cs;
-            ai = ck[2] * sn;
-            sincospi(2.0 * x * ck[1], &sn, &cs);
-            br = cs;
-            bi = sn;
-        }
-        bf16 h, m, l;
-        split3d(ar, h, m, l); Ar[e] = h; Ar[total + e] = m; Ar[2 * total + e] = l;
-        split3d(ai, h, m, l); Ai[e] = h; Ai[total + e] = m; Ai[2 * total + e] = l;
-        split3d(br, h, m, l); Br[e] = h; Br[total + e] = m; Br[2 * total + e] = l;
-        split3d(bi, h, m, l); Bi[e] = h; Bi[total + e] = m; Bi[2 * total + e] = l;
+//
+// FP64 sincospi per element bound this kernel (664 us of the 1755 us that 2000
+// components on a 2048^2 grid took).  With g - Ng/2 = kQ h + q + g_0 a phasor is the
+// product of one of kQ and one of Ng / kQ others, which a block evaluates once in
+// FP64 for its kKb components and multiplies as pairs of FP32 (error below 2^-44,
+// against the split's 2^-24): 104 us.
+constexpr int kKb = 16;                              // components of a block
+constexpr int kQ = 64;                               // fine steps
+
+struct C2 { float rh, ih, rl, il; };                 // a complex number as two FP32 parts
+
+__device__ __forceinline__ C2 c2_phasor(double turns, double amp) {
+    double sn, cs;
+    sincospi(2.0 * turns, &sn, &cs);
+    cs *= amp;
+    sn *= amp;
+    C2 r;
+    r.rh = (float)cs;
+    r.ih = (float)sn;
+    r.rl = (float)(cs - (double)r.rh);
+    r.il = (float)(sn - (double)r.ih);
+    return r;
+}
+
+// a b + c d (products and sum with their rounding errors) as hi + lo.
+__device__ __forceinline__ void c2_dot(float ah, float al, float bh, float bl, float ch, float cl, float dh, float dl,
+                                       float &hi, float &lo) {
+    const float p = __fmul_rn(ah, bh), q = __fmul_rn(ch, dh);
+    float e = fmaf(ah, bh, -p) + fmaf(ch, dh, -q);
+    e = fmaf(ah, bl, fmaf(al, bh, e));
+    e = fmaf(ch, dl, fmaf(cl, dh, e));
+    const float t = __fadd_rn(p, q), bb = __fsub_rn(t, p);
+    e += __fadd_rn(__fsub_rn(p, __fsub_rn(t, bb)), __fsub_rn(q, bb));
+    hi = __fadd_rn(t, e);
+    lo = __fsub_rn(e, __fsub_rn(hi, t));
+}
+
+__device__ __forceinline__ void split3p(float hi, float lo, bf16 &h, bf16 &m, bf16 &l) {
+    h = __float2bfloat16_rn(hi);
+    const float r = (hi - __bfloat162float(h)) + lo;
+    m = __float2bfloat16_rn(r);
+    l = __float2bfloat16_rn(r - __bfloat162float(m));
+}
+
+__global__ void __launch_bounds__(256) split_comp_kernel(const double *__restrict__ comp, int n_comp, int stride, double wp,
+                                                         int kp, int ng, int b_rows, double du, bf16 *__restrict__ Ar,
+                                                         bf16 *__restrict__ Ai, bf16 *__restrict__ Br, bf16 *__restrict__ Bi) {
+    __shared__ C2 s_q[2][kQ][kKb];                   // fine steps of u l and v m
+    __shared__ C2 s_h[2][kKb];                       // this group of kQ rows
+    const int k0 = blockIdx.x * kKb, tid = threadIdx.x;
+    for (int e = tid; e < 2 * kQ * kKb; e += blockDim.x) {
+        const int d = e / (kQ * kKb), q = e / kKb % kQ, k = k0 + e % kKb;
+        s_q[d][q][e % kKb] = k < n_comp ? c2_phasor((double)q * du * comp[(size_t)stride * k + d], 1.0) : C2{0.f, 0.f, 0.f, 0.f};
     }
+    const int n_grp = (ng + kQ - 1) / kQ;
+    for (int grp = blockIdx.y; grp < n_grp; grp += gridDim.y) {
+        __syncthreads();
+        if (tid < 2 * kKb) {
+            const int d = tid / kKb, k = k0 + tid % kKb;
+            C2 v{0.f, 0.f, 0.f, 0.f};
+            if (k < n_comp) {
+                const double *ck = comp + (size_t)stride * k;
+                // flux phase of a w-plane: 2 pi wp (n - 1), folded into the u factor
+                const double wph = d == 0 && stride == 4 ? wp * ck[3] : 0.0;
+                v = c2_phasor((double)(grp * kQ - ng / 2) * du * ck[d] + wph, d == 0 ? ck[2] : 1.0);
+            }
+            s_h[d][tid % kKb] = v;
+        }
+        __syncthreads();
+        // two neighbouring components a thread: four-byte stores
+        for (int e = tid; e < 2 * kQ * (kKb / 2); e += blockDim.x) {
+            const int d = e / (kQ * (kKb / 2)), q = e / (kKb / 2) % kQ, kk = e % (kKb / 2) * 2;
+            const int g = grp * kQ + q, rows = d == 0 ? ng : b_rows;
+            if (g >= rows || k0 + kk >= kp) continue;
+            bf16 re[2][3], im[2][3];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const C2 x = s_h[d][kk + j], y = s_q[d][q][kk + j];
+                float hi, lo;
+                c2_dot(x.rh, x.rl, y.rh, y.rl, -x.ih, -x.il, y.ih, y.il, hi, lo);
+                split3p(hi, lo, re[j][0], re[j][1], re[j][2]);
+                c2_dot(x.rh, x.rl, y.ih, y.il, x.ih, x.il, y.rh, y.rl, hi, lo);
+                split3p(hi, lo, im[j][0], im[j][1], im[j][2]);
+            }
+            const size_t plane = (size_t)rows * kp, o = (size_t)g * kp + k0 + kk;
+            bf16 *R = d == 0 ? Ar : Br, *I = d == 0 ? Ai : Bi;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                *reinterpret_cast<__nv_bfloat162 *>(R + p * plane + o) = __nv_bfloat162(re[0][p], re[1][p]);
+                *reinterpret_cast<__nv_bfloat162 *>(I + p * plane + o) = __nv_bfloat162(im[0][p], im[1][p]);
+            }
+        }
+    }
+}
+
+// What the half-plane pass leaves of a Hermitian component grid (B's rows end at
+// Ng/2): row v = 0, the sums of A's rows, and column gx = 0 for v > 0, the sums of
+// A[0] conj(B[Ng - gy]).  A warp per cell.
+__global__ void comp_edge_kernel(const bf16 *__restrict__ Ar, const bf16 *__restrict__ Ai, const bf16 *__restrict__ Br,
+                                 const bf16 *__restrict__ Bi, int ng, int kp, float2 *__restrict__ G) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int half = ng / 2;
+    if (w >= ng + half - 1) return;
+    const bool row = w < ng;
+    const int gx = row ? w : 0, gy = row ? half : half + 1 + (w - ng);
+    const size_t pa = (size_t)ng * kp, pb = (size_t)half * kp;
+    const size_t oa = (size_t)gx * kp, ob = (size_t)(ng - gy) * kp;
+    auto sum3 = [](const bf16 *p, size_t plane, size_t at) {
+        return (__bfloat162float(p[at]) + __bfloat162float(p[plane + at])) + __bfloat162float(p[2 * plane + at]);
+    };
+    float re = 0.f, im = 0.f;
+    for (int k = lane; k < kp; k += 32) {
+        const float ar = sum3(Ar, pa, oa + k), ai = sum3(Ai, pa, oa + k);
+        float br = 1.f, bi = 0.f;
+        if (!row) {
+            br = sum3(Br, pb, ob + k);
+            bi = -sum3(Bi, pb, ob + k);
+        }
+        re += ar * br - ai * bi;
+        im += ar * bi + ai * br;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane == 0) G[(size_t)gy * ng + gx] = make_float2(re, im);
 }
 
 __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t k_stride) {
@@ -300,6 +400,7 @@ struct TcPassArgs {
     int a_rows, b_rows, k;  // rows of the A and B operands, depth (= N, also the plane pitch)
     bf16 *Tr, *Ti;          // pass 1 output planes [3][Ng][N]
     float2 *G;              // pass 2 output [Ng][Ng]
+    int hermitian;          // pass 2: every cell (gy, gx) past the first row and column is also, conjugated, (Ng - gy, Ng - gx)
     int ng;
     int *err;
 };
@@ -485,6 +586,8 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
                     g.Ti[o] = h; g.Ti[plane_t + o] = mm; g.Ti[2 * plane_t + o] = l;
                 } else {
                     g.G[(size_t)col * g.ng + m] = make_float2(sum_re[j], sum_im[j]);
+                    if (g.hermitian && col > 0 && m > 0)
+                        g.G[(size_t)(g.ng - col) * g.ng + g.ng - m] = make_float2(sum_re[j], -sum_im[j]);
                 }
             }
         }
@@ -629,34 +732,49 @@ cudaError_t launch_model_grid(int n_img, int n_grid, const float *image, void *w
     return launch_tc_pass<2>(a2, s);
 }
 
+namespace {
+// Real fluxes make the grid Hermitian: the matrix product then covers the rows v < 0
+// and writes their mirror images too (with a w-plane's complex fluxes it covers all):
+// 429 us of tensor-core pass for 2000 components on 2048^2, 842 without.
+int comp_b_rows(int stride, int n_grid) { return stride == 3 ? n_grid / 2 : n_grid; }
+}  // namespace
+
 size_t model_grid_comp_ws_bytes(int n_comp, int n_grid, int stride) {
-    const size_t kp = (size_t)comp_depth(n_comp), ng = (size_t)n_grid;
-    return al256((size_t)n_comp * stride * sizeof(double)) + 4 * al256(3 * ng * kp * 2) + 256;
+    const size_t kp = (size_t)comp_depth(n_comp), ng = (size_t)n_grid, nb = (size_t)comp_b_rows(stride, n_grid);
+    return al256((size_t)n_comp * stride * sizeof(double)) + 2 * al256(3 * ng * kp * 2) + 2 * al256(3 * nb * kp * 2) + 256;
 }
 
 cudaError_t launch_model_grid_comp(int n_comp, const double *comp_host, int stride, double wp, int n_grid, double du,
                                    void *ws, float2 *grid_out, int **err_dev, cudaStream_t s) {
     const int kp = comp_depth(n_comp);
-    const size_t ng = (size_t)n_grid;
+    const int b_rows = comp_b_rows(stride, n_grid);
+    const size_t ng = (size_t)n_grid, nb = (size_t)b_rows;
     unsigned char *p = (unsigned char *)ws;
     double *comp = (double *)p; p += al256((size_t)n_comp * stride * sizeof(double));
     bf16 *Ar = (bf16 *)p; p += al256(3 * ng * kp * 2);
     bf16 *Ai = (bf16 *)p; p += al256(3 * ng * kp * 2);
-    bf16 *Br = (bf16 *)p; p += al256(3 * ng * kp * 2);
-    bf16 *Bi = (bf16 *)p; p += al256(3 * ng * kp * 2);
+    bf16 *Br = (bf16 *)p; p += al256(3 * nb * kp * 2);
+    bf16 *Bi = (bf16 *)p; p += al256(3 * nb * kp * 2);
     *err_dev = (int *)p;
     cudaError_t e = cudaMemsetAsync(*err_dev, 0, sizeof(int), s);
     if (e == cudaSuccess && n_comp > 0)
         e = cudaMemcpyAsync(comp, comp_host, (size_t)n_comp * stride * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
-    split_comp_kernel<<<(int)std::min<size_t>((ng * kp + 255) / 256, 8192), 256, 0, s>>>(
-        comp, n_comp, stride, wp, kp, n_grid, du, Ar, Ai, Br, Bi);
+    // blocks of kKb components; their groups of rows shared out until the chip is full
+    const int kblocks = (kp + kKb - 1) / kKb, groups = (n_grid + kQ - 1) / kQ;
+    const int split = std::max(1, std::min(groups, (2 * 152 + kblocks - 1) / kblocks));
+    split_comp_kernel<<<dim3(kblocks, split), 256, 0, s>>>(comp, n_comp, stride, wp, kp, n_grid, b_rows, du, Ar, Ai, Br, Bi);
     TcPassArgs a2{};
     a2.A[0] = Ar; a2.A[1] = Ai; a2.n_a = 2;
     a2.B[0] = Br; a2.B[1] = Bi;
-    a2.a_rows = n_grid; a2.b_rows = n_grid; a2.k = kp;
+    a2.a_rows = n_grid; a2.b_rows = b_rows; a2.k = kp;
     a2.G = grid_out; a2.ng = n_grid; a2.err = *err_dev;
-    return launch_tc_pass<2>(a2, s);
+    a2.hermitian = b_rows < n_grid;
+    e = launch_tc_pass<2>(a2, s);
+    if (e != cudaSuccess || !a2.hermitian) return e;
+    const int cells = n_grid + n_grid / 2 - 1;
+    comp_edge_kernel<<<(cells * 32 + 255) / 256, 256, 0, s>>>(Ar, Ai, Br, Bi, n_grid, kp, grid_out);
+    return cudaGetLastError();
 }
 
 }  // namespace psc
