@@ -378,8 +378,8 @@ psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread);
  * (TwoSum) per lane and across the warp, then in FP64.  Predictions
  * (psc_predict) keep the brick kernel.  0 switches back to the brick kernel;
  * so do psc_set_tiling, psc_set_flat_tiling, psc_set_kernel_model,
- * psc_set_grid_precision(PSC_GRID_BF16) and psc_set_wstack.  The first call
- * with vis_per_lane > 0 builds the tensor maps of the grid and per-channel
+ * psc_set_grid_precision(PSC_GRID_BF16) and psc_set_wstack.  psc_create (where
+ * it picks this kernel by size) or the first call with vis_per_lane > 0 builds the tensor maps of the grid and per-channel
  * tables (a few KB; synchronises the stream).  Errors: PSC_ERR_ARG when the
  * context uses the exact kernel, a residual-w stack or the BF16 grid copy, a
  * grid not 16-byte aligned, an aperture reaching outside the S x S window,

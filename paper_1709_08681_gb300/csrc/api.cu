@@ -45,10 +45,13 @@ struct psc_ctx {
     bool begun = false;
     int *d_done = nullptr;       // points at d_state->done
     int max_tab_len = 0;
+    bool auto_shape = true;      // no tiling set: brick_shape() picks one from the sizes
+    // the tiling set by the caller or the autotuner (auto_shape false)
     int t_tile = 32, c_group = 4;
     int kv = 1;                  // visibilities per thread at consecutive times
     int flat = 0;                // > 0: bricks of `flat` consecutive (channel, time-group) items
     int no_stage = 0;            // PSC_STAGE_NEVER: taps read the grid from global memory
+    bool trk_set = false;        // a tiling or the track kernel was chosen: trk_kv holds (else auto_track() picks)
     int trk_kv = 0;              // > 0: reduce-mode evaluations run the track kernel, trk_kv visibilities per lane
     float2 *d_tabcs = nullptr;   // track kernel: per-channel (intercept, slope) tables [nc][trk_stride]
     int trk_stride = 0;
@@ -66,6 +69,7 @@ struct psc_ctx {
     double wp_w0 = 0.0, wp_dw = 0.0, wp_a = 0.0, wp_b = 0.0;
     std::vector<double> h_freq;  // channel frequencies (Hz)
     std::vector<int> h_tab_off, h_tab_len;   // radial table layout per channel
+    double rho_top = 0.0;        // aperture radius at the top channel (cells)
     double step_cells = 0.0;     // largest move of a baseline between time steps (cells, top channel)
     bool multi_ok = false;       // kv > 1 allowed: every channel's aperture fits inside the S x S window
     LMState h_state{};
@@ -162,8 +166,6 @@ void free_ctx(psc_ctx *c) {
     delete c;
 }
 
-int n_tt(const psc_ctx *c) { return (c->nt + c->t_tile * c->kv - 1) / (c->t_tile * c->kv); }
-
 // Largest visibility separation within one thread's kv time steps (cells).
 double kv_spread(const psc_ctx *c, int kv) { return (kv - 1) * c->step_cells; }
 
@@ -182,10 +184,6 @@ int tab_stride(const psc_ctx *c, int kv) {
     if (kv == 1) return c->max_tab_len + 2;
     return c->max_tab_len + (int)std::ceil(c->gd.oversample * (kv_spread(c, kv) + 1.0)) + 2;
 }
-int n_cg(const psc_ctx *c) { return (c->nc + c->c_group - 1) / c->c_group; }
-// Track kernel: time chunks of 32 lanes x trk_kv steps per baseline, and the
-// staged tile capacity of one buffer (cells).
-int trk_chunks(const psc_ctx *c) { return (c->nt + 32 * c->trk_kv - 1) / (32 * c->trk_kv); }
 constexpr int kTrkCap = 512;
 // Zero table entries the track kernel's tap pattern can reach past a
 // channel's table with kv visibilities per lane: its taps lie within
@@ -193,25 +191,122 @@ constexpr int kTrkCap = 512;
 int trk_pad(const psc_ctx *c, int kv) {
     return (int)std::ceil(c->gd.oversample * (2.0 * kv_spread(c, kv) + 1.5)) + 2;
 }
-// Flat bricks: groups of kv consecutive time steps per channel, the bricks
-// per baseline, and the most channels one brick's items can span.
-int n_tp(const psc_ctx *c) { return (c->nt + c->kv - 1) / c->kv; }
-long long bricks_per_bl(const psc_ctx *c) {
-    if (c->trk_kv > 0) return trk_chunks(c);
-    if (c->flat > 0) return ((long long)c->nc * n_tp(c) + c->flat - 1) / c->flat;
-    return (long long)n_cg(c) * n_tt(c);
-}
-int ch_span(const psc_ctx *c) {
-    return c->flat > 0 ? std::min(c->nc, (c->flat + n_tp(c) - 2) / n_tp(c) + 1) : c->c_group;
-}
-// Block width of the fused kernel for this context's bricks.
-int eval_threads(const psc_ctx *c) {
-    if (c->trk_kv > 0) return kTrkThreads;
-    return ((c->flat > 0 ? c->flat : c->t_tile * c->c_group) + 31) / 32 * 32;
+// Why the track kernel cannot serve this context with kv visibilities per
+// lane (empty: it can).
+std::string trk_refusal(const psc_ctx *c, int kv) {
+    if (kv != 1 && kv != 2) return "vis_per_lane must be 1 or 2";
+    if (c->kernel_model != PSC_KERNEL_GAUSS) return "the track kernel uses the Gaussian kernel model";
+    if (c->wp_n > 0) return "the track kernel does not read a residual-w stack";
+    if (c->d_grid_bf16) return "the track kernel reads the FP32 grid";
+    if ((uintptr_t)c->grid % 16) return "the track kernel needs a 16-byte aligned grid";
+    if (!c->multi_ok) return "the track kernel needs every channel's aperture inside the S x S window";
+    if (!kv_allowed(c, kv)) return "vis_per_lane 2 needs consecutive time steps within 4 cells";
+    return "";
 }
 
-psc_status ensure_partials(psc_ctx *c) {
-    const size_t need = (size_t)c->n_bl * bricks_per_bl(c);
+// A fused launch's shape: the brick kernel's (rectangular, with `split` lanes per
+// visibility, or flat > 0) or, with trk_kv > 0, the track kernel's.
+struct Shape {
+    int t_tile = 32, c_group = 4, kv = 1, flat = 0, split = 1, trk_kv = 0;
+};
+
+// Channels that one flat brick of `flat` items can span.
+int flat_span(const psc_ctx *c, int flat, int kv) {
+    const int tp = (c->nt + kv - 1) / kv;
+    return std::min(c->nc, (flat + tp - 2) / tp + 1);
+}
+
+// The brick kernel's shape where none was set, by size (us per launch):
+//   from 2e6 visibilities on, flat bricks of 256 items, of two visibilities if they
+//     move less than half a cell a step: 27 antennas, 150 x 64: 731 against 997 for
+//     rectangles of 32 x 4 (one visibility each: 843); 64 antennas at 1.8 cells a
+//     step, 173 x 16: 1413 (two: 1499) against 1734;
+//   below, the rectangles, in whose sums a solve's stop rule and so its last digits
+//     depend on every bit, with the rows of a visibility shared among up to 16 lanes
+//     while the chip would not be full otherwise (at most one lane per two rows, at
+//     least 4): the same sums, see eval.cu.
+// Stacks of grids take flat bricks of 128 from the same size on.  A brick spans at most
+// 8 channels (its tables' shared memory), else the rectangle.
+constexpr double kLargeVis = 2e6;
+// Whether split_taps' arrays fit a block beside four channels' tables (wide apertures' may not).
+bool split_fits(const psc_ctx *c, int split) {
+    return eval_dyn_smem(4, tab_stride(c, 1)) + eval_split_smem(split, c->gd.support) <= (size_t)128 * 1024;
+}
+Shape brick_shape(const psc_ctx *c) {
+    Shape s;
+    if (!c->auto_shape) {
+        s.t_tile = c->t_tile;
+        s.c_group = c->c_group;
+        s.kv = c->kv;
+        s.flat = c->flat;
+        return s;
+    }
+    if (c->kernel_model != PSC_KERNEL_GAUSS) return s;
+    const double n_vis = (double)c->nt * c->n_bl * c->nc;
+    if (n_vis >= kLargeVis) {
+        if (c->wp_n == 0 && c->step_cells <= 0.5 && kv_allowed(c, 2) && flat_span(c, 256, 2) <= 8) {
+            s.flat = 256;
+            s.kv = 2;
+        } else if (flat_span(c, c->wp_n > 0 ? 128 : 256, 1) <= 8) {
+            s.flat = c->wp_n > 0 ? 128 : 256;
+        }
+        return s;
+    }
+    if (c->wp_n > 0) return s;
+    while (s.split < 16 && 2.0 * s.split * n_vis <= 5e5 && 2 * s.split <= c->rho_top + 1.0) s.split *= 2;
+    if (s.split < 4 || !split_fits(c, s.split)) s.split = 1;
+    return s;
+}
+
+// The track kernel's visibilities per lane where no tiling was set, 0 for the brick
+// kernel: small apertures whose baselines move little between steps (their boxes
+// fit), given warps enough (an item is a baseline and 32 steps a lane's visibility);
+// 197 antennas, 60 x 128: 4515 us with two per lane against 10299 for the best
+// brick, 8 x 64: 1660 with one against 3784; but 30 antennas, 20 x 16 (435 items):
+// 46 against 33.  Fast-moving baselines fall back to reading taps from the grid,
+// where the track kernel wins only in large arrays (197 antennas, 77 x 16: 2184
+// against 2918; 60 antennas: 346 against 299).
+int want_track(const psc_ctx *c) {
+    if (c->rho_top > 4.5 || (double)c->nt * c->n_bl * c->nc < kLargeVis) return 0;
+    const int kv = c->nt > 32 && c->step_cells <= 0.5 ? 2 : 1;
+    const long long items = (long long)c->n_bl * ((c->nt + 32 * kv - 1) / (32 * kv));
+    if (items < (c->step_cells <= 0.5 ? 1000 : 20000)) return 0;
+    return trk_refusal(c, kv).empty() ? kv : 0;
+}
+// The same where psc_create has set the track kernel up and nothing else was chosen since.
+int auto_track(const psc_ctx *c) { return c->trk_set || !c->d_tmap ? 0 : want_track(c); }
+
+// The shape of a reduce-mode launch of this context on its own.
+Shape eval_shape(const psc_ctx *c) {
+    Shape s = brick_shape(c);
+    s.trk_kv = c->trk_set ? c->trk_kv : auto_track(c);
+    return s;
+}
+
+int trk_chunks(const psc_ctx *c, const Shape &s) { return (c->nt + 32 * s.trk_kv - 1) / (32 * s.trk_kv); }
+int n_tt(const psc_ctx *c, const Shape &s) { return (c->nt + s.t_tile * s.kv - 1) / (s.t_tile * s.kv); }
+int n_cg(const psc_ctx *c, const Shape &s) { return (c->nc + s.c_group - 1) / s.c_group; }
+// Flat bricks: groups of kv consecutive time steps per channel, the bricks
+// per baseline, and the most channels one brick's items can span.
+int n_tp(const psc_ctx *c, const Shape &s) { return (c->nt + s.kv - 1) / s.kv; }
+long long bricks_per_bl(const psc_ctx *c, const Shape &s) {
+    if (s.trk_kv > 0) return trk_chunks(c, s);
+    if (s.flat > 0) return ((long long)c->nc * n_tp(c, s) + s.flat - 1) / s.flat;
+    return (long long)n_cg(c, s) * n_tt(c, s);
+}
+int ch_span(const psc_ctx *c, const Shape &s) { return s.flat > 0 ? flat_span(c, s.flat, s.kv) : s.c_group; }
+// Block width of the fused kernel for this context's bricks.
+int eval_threads(const Shape &s) {
+    if (s.trk_kv > 0) return kTrkThreads;
+    if (s.split > 1) return kMaxThreads;
+    return ((s.flat > 0 ? s.flat : s.t_tile * s.c_group) + 31) / 32 * 32;
+}
+
+psc_status ensure_partials(psc_ctx *c, const Shape &s) {
+    size_t need = (size_t)c->n_bl * bricks_per_bl(c, s);
+    // room for the other kernel too where the choice depends on the rest of a
+    // batch: another batch's tables must not lose the records they point at
+    if (!c->trk_set) need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, brick_shape(c)));
     if (need <= c->partials_cap) return PSC_OK;
     cudaFree(c->d_partials);
     c->d_partials = nullptr;
@@ -221,7 +316,7 @@ psc_status ensure_partials(psc_ctx *c) {
     return PSC_OK;
 }
 
-EvalArgs eval_args(const psc_ctx *c, const double *lm_dev) {
+EvalArgs eval_args(const psc_ctx *c, const Shape &s, const double *lm_dev) {
     EvalArgs a{};
     a.uvw = c->uvw;
     a.uvs = c->d_uvs;
@@ -240,31 +335,32 @@ EvalArgs eval_args(const psc_ctx *c, const double *lm_dev) {
     a.support = c->gd.support;
     a.ov = c->gd.oversample;
     a.du = (float)c->du;
-    a.t_tile = c->t_tile;
-    a.c_group = c->c_group;
-    a.kv = c->kv;
+    a.t_tile = s.t_tile;
+    a.c_group = s.c_group;
+    a.kv = s.kv;
     a.no_stage = c->no_stage;
-    a.n_tt = n_tt(c);
-    a.n_cg = n_cg(c);
+    a.n_tt = n_tt(c, s);
+    a.n_cg = n_cg(c, s);
     a.decorrelation = c->ap.decorrelation;
     a.max_tab_len = c->max_tab_len;
-    a.tab_stride = tab_stride(c, c->kv);
-    a.n_bricks = (long long)c->n_bl * bricks_per_bl(c);
-    a.flat = c->flat;
-    a.n_tp = n_tp(c);
-    a.bpb = (int)bricks_per_bl(c);
-    a.ch_span = ch_span(c);
+    a.tab_stride = tab_stride(c, s.kv);
+    a.n_bricks = (long long)c->n_bl * bricks_per_bl(c, s);
+    a.flat = s.flat;
+    a.split = s.split;
+    a.n_tp = n_tp(c, s);
+    a.bpb = (int)bricks_per_bl(c, s);
+    a.ch_span = ch_span(c, s);
     a.exact = c->kernel_model == PSC_KERNEL_EXACT_DISK;
     a.bl_order = c->brick_order == PSC_ORDER_UV ? c->d_bl_order : nullptr;
     a.kmom = c->d_kmom;
     a.err = c->d_err;
     a.wait_limit = wait_limit();
-    if (c->trk_kv > 0) {
-        a.trk_kv = c->trk_kv;
-        a.trk_chunks = trk_chunks(c);
+    if (s.trk_kv > 0) {
+        a.trk_kv = s.trk_kv;
+        a.trk_chunks = trk_chunks(c, s);
         a.trk_cap = kTrkCap;
         a.trk_stride = c->trk_stride;
-        a.trk_pad = trk_pad(c, c->trk_kv);
+        a.trk_pad = trk_pad(c, s.trk_kv);
         // the longest table a channel copies with this tiling's pad (the stride
         // is sized for two visibilities per lane)
         a.trk_tabc = (std::min(c->trk_stride, (c->max_tab_len + a.trk_pad + 1) & ~1) + 15) / 16 * 16;
@@ -284,14 +380,14 @@ EvalArgs eval_args(const psc_ctx *c, const double *lm_dev) {
     return a;
 }
 
-RedArgs red_args(const psc_ctx *c, double *ev_out, const int *skip) {
+RedArgs red_args(const psc_ctx *c, const Shape &s, double *ev_out, const int *skip) {
     RedArgs r{};
     r.partials = c->d_partials;
     r.blsum = c->d_blsum;
     r.ev = ev_out;
     r.skip = skip;
     r.n_bl = c->n_bl;
-    r.bpb = (int)bricks_per_bl(c);
+    r.bpb = (int)bricks_per_bl(c, s);
     r.n_ant = c->n_ant;
     return r;
 }
@@ -323,11 +419,15 @@ bool check_grid_desc(const psc_grid_desc *gd, std::string *why) {
     return true;
 }
 
+psc_status trk_prepare(psc_ctx *c);
+
 psc_status eval_reduce(psc_ctx *c, const double *lm_dev, const void *vis_obs, const float *w, double w_scale,
                        double *ev_out, const int *skip) {
-    psc_status st = ensure_partials(c);
+    const Shape shape = eval_shape(c);
+    psc_status st = ensure_partials(c, shape);
+    if (st == PSC_OK && shape.trk_kv > 0) st = trk_prepare(c);
     if (st != PSC_OK) return st;
-    EvalArgs a = eval_args(c, lm_dev);
+    EvalArgs a = eval_args(c, shape, lm_dev);
     a.vis_obs = (const float2 *)vis_obs;
     a.w = w;
     a.w_scale = (float)w_scale;
@@ -345,7 +445,7 @@ psc_status eval_reduce(psc_ctx *c, const double *lm_dev, const void *vis_obs, co
         PSC_CUDA(c, cudaEventRecord(c->ev_pool[c->ev_used + 1], c->stream));
         c->ev_used += 2;
     }
-    PSC_CUDA(c, launch_reduce(red_args(c, ev_out, skip), c->stream));
+    PSC_CUDA(c, launch_reduce(red_args(c, shape, ev_out, skip), c->stream));
     return PSC_OK;
 }
 
@@ -412,19 +512,6 @@ psc_status trk_prepare(psc_ctx *c) {
     c->trk_stride = stride;
     c->d_tmap = maps;
     return PSC_OK;
-}
-
-// Why the track kernel cannot serve this context with kv visibilities per
-// lane (empty: it can).
-std::string trk_refusal(const psc_ctx *c, int kv) {
-    if (kv != 1 && kv != 2) return "vis_per_lane must be 1 or 2";
-    if (c->kernel_model != PSC_KERNEL_GAUSS) return "the track kernel uses the Gaussian kernel model";
-    if (c->wp_n > 0) return "the track kernel does not read a residual-w stack";
-    if (c->d_grid_bf16) return "the track kernel reads the FP32 grid";
-    if ((uintptr_t)c->grid % 16) return "the track kernel needs a 16-byte aligned grid";
-    if (!c->multi_ok) return "the track kernel needs every channel's aperture inside the S x S window";
-    if (!kv_allowed(c, kv)) return "vis_per_lane 2 needs consecutive time steps within 4 cells";
-    return "";
 }
 
 // The evaluation's bounded waits ran out (a kernel set *d_err): clears the flag.
@@ -819,6 +906,7 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
             rho_top = std::max(rho_top, (double)(len[k] - 1) / ov);
         }
         c->step_cells = (double)step_m * sc_max;
+        c->rho_top = rho_top;
         c->multi_ok = std::isfinite(c->step_cells) && rho_top <= 0.5 * gd->support - 1.0;
     }
     // room for the tables of the widest channel group, and the LM layouts
@@ -826,6 +914,7 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
     if (kv_allowed(c, 2)) stride_max = std::max(stride_max, tab_stride(c, 2));
     e = set_eval_smem(eval_dyn_smem(8, stride_max));
     if (e == cudaSuccess) e = lm_prepare(c->n_ant);
+    if (e == cudaSuccess && want_track(c)) (void)trk_prepare(c);      // without it the brick kernel runs
     if (e != cudaSuccess) { psc_status st = cuda_fail(nullptr, e, "psc_create: shared memory"); free_ctx(c); return st; }
     *out = c;
     return PSC_OK;
@@ -837,7 +926,7 @@ psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thr
     if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
     const int tt = t_tile ? t_tile : ctx->t_tile;
     const int cg = c_group ? c_group : ctx->c_group;
-    const int kv = vis_per_thread ? vis_per_thread : ctx->kv;
+    const int kv = vis_per_thread ? vis_per_thread : ctx->kv;       // (32, 4, 1) where none was set
     if (!(kv == 1 || kv == 2)) return fail(ctx, PSC_ERR_ARG, "vis_per_thread must be 1 or 2");
     if (kv != 1 && ctx->kernel_model == PSC_KERNEL_EXACT_DISK)
         return fail(ctx, PSC_ERR_ARG, "the exact disk kernel takes one visibility per thread");
@@ -852,6 +941,8 @@ psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thr
     ctx->kv = kv;
     ctx->flat = 0;
     ctx->trk_kv = 0;
+    ctx->trk_set = true;
+    ctx->auto_shape = false;
     return PSC_OK;
 }
 
@@ -864,22 +955,21 @@ psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread) {
     if (!kv_allowed(ctx, vis_per_thread))
         return fail(ctx, PSC_ERR_ARG, "vis_per_thread 2 needs the aperture inside the S x S window and "
                                       "consecutive time steps within 4 cells");
-    const int old_kv = ctx->kv, old_flat = ctx->flat;
+    if (flat_span(ctx, items, vis_per_thread) > 8)
+        return fail(ctx, PSC_ERR_ARG, "a brick would span more than 8 channels (too few time steps per channel)");
     ctx->kv = vis_per_thread;
     ctx->flat = items;
-    if (ch_span(ctx) > 8) {
-        ctx->kv = old_kv;
-        ctx->flat = old_flat;
-        return fail(ctx, PSC_ERR_ARG, "a brick would span more than 8 channels (too few time steps per channel)");
-    }
     ctx->trk_kv = 0;
+    ctx->trk_set = true;
+    ctx->auto_shape = false;
     return PSC_OK;
 }
 
 psc_status psc_set_track_tiling(psc_ctx *ctx, int vis_per_lane) {
     if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
-    if (vis_per_lane == 0) {
+    if (vis_per_lane == 0) {                          // the brick kernel, in its own shape
         ctx->trk_kv = 0;
+        ctx->trk_set = true;
         return PSC_OK;
     }
     const std::string why = trk_refusal(ctx, vis_per_lane);
@@ -887,6 +977,7 @@ psc_status psc_set_track_tiling(psc_ctx *ctx, int vis_per_lane) {
     psc_status st = trk_prepare(ctx);
     if (st != PSC_OK) return st;
     ctx->trk_kv = vis_per_lane;
+    ctx->trk_set = true;
     return PSC_OK;
 }
 
@@ -1008,10 +1099,7 @@ psc_status psc_predict(psc_ctx *ctx, const double *lm, void *vis_out, void *dvis
     if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
     if (!lm || !vis_out) return fail(ctx, PSC_ERR_ARG, "lm and vis_out must be non-NULL");
     PSC_CUDA(ctx, cudaMemcpyAsync(ctx->d_lm_trial, lm, sizeof(double) * 2 * ctx->n_ant, cudaMemcpyHostToDevice, ctx->stream));
-    const int trk = ctx->trk_kv;                  // predictions always run the brick kernel
-    ctx->trk_kv = 0;
-    EvalArgs a = eval_args(ctx, ctx->d_lm_trial);
-    ctx->trk_kv = trk;
+    EvalArgs a = eval_args(ctx, brick_shape(ctx), ctx->d_lm_trial);    // predictions always run the brick kernel
     a.vis_out = (float2 *)vis_out;
     a.dvis_out = (float2 *)dvis_out;
     PSC_CUDA(ctx, launch_eval(a, true, ctx->stream));
@@ -1022,10 +1110,7 @@ psc_status psc_predict(psc_ctx *ctx, const double *lm, void *vis_out, void *dvis
 psc_status psc_predict_dev(psc_ctx *ctx, const double *lm_dev, void *vis_out, void *dvis_out) {
     if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
     if (!lm_dev || !vis_out) return fail(ctx, PSC_ERR_ARG, "lm_dev and vis_out must be non-NULL");
-    const int trk = ctx->trk_kv;                  // predictions always run the brick kernel
-    ctx->trk_kv = 0;
-    EvalArgs a = eval_args(ctx, lm_dev);
-    ctx->trk_kv = trk;
+    EvalArgs a = eval_args(ctx, brick_shape(ctx), lm_dev);    // predictions always run the brick kernel
     a.vis_out = (float2 *)vis_out;
     a.dvis_out = (float2 *)dvis_out;
     PSC_CUDA(ctx, launch_eval(a, true, ctx->stream));
@@ -1366,6 +1451,7 @@ struct psc_batch {
     int max_ant = 0, max_bpb = 0;    // most antennas of a context, most records of a baseline
     int grid = 0;
     int threads = 128;           // fused-kernel block size: the widest context's shape
+    bool split = false;          // some context shares its visibilities among lanes
     bool stacked = false;        // every context reads a residual-w stack (else none does)
     int track = 0;               // > 0: the persistent launch runs the track kernel, this many visibilities per lane
     int trk_tabc = 0;            // track kernel: table capacity of a warp buffer (entries)
@@ -1424,23 +1510,35 @@ psc_status build_tables(psc_batch *b) {
     std::vector<const double *> lm0(n);
     size_t dyn = 0, lmd = 0;
     int threads = 32, max_ant = 0, max_bpb = 0;
+    // contexts without a tiling take the track kernel only if all of them would, with
+    // the same visibilities per lane: one fused kernel serves the launch
+    int all_trk = auto_track(b->ctxs[0]);
+    for (psc_ctx *c : b->ctxs)
+        if (auto_track(c) != all_trk) all_trk = 0;
+    bool split = false;
+    std::vector<Shape> shapes(n);
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
-        threads = std::max(threads, eval_threads(c));
-        psc_status st = ensure_partials(c);
+        shapes[k] = brick_shape(c);
+        shapes[k].trk_kv = c->trk_set ? c->trk_kv : all_trk;
+        const Shape &shape = shapes[k];
+        threads = std::max(threads, eval_threads(shape));
+        split = split || (shape.trk_kv == 0 && shape.split > 1);
+        psc_status st = ensure_partials(c, shape);
+        if (st == PSC_OK && shape.trk_kv > 0) st = trk_prepare(c);
         if (st != PSC_OK) return bfail(b, st, c->err);
-        ev[k] = eval_args(c, c->d_lm_trial);
+        ev[k] = eval_args(c, shape, c->d_lm_trial);
         ev[k].vis_obs = (const float2 *)b->vis[k];
         ev[k].w = b->w[k];
         ev[k].w_scale = (float)b->w_scale[k];
         ev[k].skip = c->d_done;
         prefix[k + 1] = prefix[k] + ev[k].n_bricks;
-        red[k] = red_args(c, c->d_ev, c->d_done);
+        red[k] = red_args(c, shape, c->d_ev, c->d_done);
         blp[k + 1] = blp[k] + c->n_bl;
         lm[k] = lm_args(c);
         st0[k] = c->d_state0;
         lm0[k] = c->d_lm0;
-        dyn = std::max(dyn, eval_dyn_smem(ch_span(c), tab_stride(c, c->kv)));
+        dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support));
         lmd = std::max(lmd, lm_smem_bytes(c->n_ant));
         max_ant = std::max(max_ant, c->n_ant);
         max_bpb = std::max(max_bpb, red[k].bpb);
@@ -1455,11 +1553,11 @@ psc_status build_tables(psc_batch *b) {
     // contexts (same visibilities per lane) or for none
     int n_trk = 0, kv_trk = 0, tabc = 0;
     for (int k = 0; k < n; ++k) {
-        const psc_ctx *c = b->ctxs[k];
-        if (c->trk_kv <= 0) continue;
+        const int kv = shapes[k].trk_kv;
+        if (kv <= 0) continue;
         ++n_trk;
-        if (kv_trk && kv_trk != c->trk_kv) kv_trk = -1;
-        else if (kv_trk == 0) kv_trk = c->trk_kv;
+        if (kv_trk && kv_trk != kv) kv_trk = -1;
+        else if (kv_trk == 0) kv_trk = kv;
         tabc = std::max(tabc, ev[k].trk_tabc);
     }
     if (n_trk != 0 && (n_trk != n || kv_trk < 0))
@@ -1468,13 +1566,14 @@ psc_status build_tables(psc_batch *b) {
     b->trk_tabc = tabc;
     int per_sm = 0, dev = 0, n_sm = 0;
     b->stacked = b->ctxs[0]->wp_n > 0;
+    b->split = split;
     if (b->track) {
         const size_t tdyn = track_dyn_smem(kTrkCap, tabc);
         PSC_BCUDA(b, set_track_smem(tdyn));
         PSC_BCUDA(b, track_occupancy(b->track, tdyn, &per_sm));
     } else {
         PSC_BCUDA(b, set_eval_smem(dyn));
-        PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, &per_sm));
+        PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, b->split, &per_sm));
     }
     PSC_BCUDA(b, cudaGetDevice(&dev));
     PSC_BCUDA(b, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
@@ -1511,7 +1610,7 @@ psc_status launch_fused(psc_batch *b) {
         PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->track, kTrkCap, b->trk_tabc, b->grid, s));
     else
         PSC_BCUDA(b, launch_eval_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->threads, b->eval_dyn, b->grid,
-                                       b->stacked, s));
+                                       b->stacked, b->split, s));
     return PSC_OK;
 }
 
@@ -1598,6 +1697,8 @@ int fit_t_tile(int nt, int threads, int cg, int kv) {
 using Tiling = std::array<int, 4>;
 
 void apply_tiling(psc_ctx *c, const Tiling &t) {
+    c->auto_shape = false;
+    c->trk_set = true;
     c->trk_kv = 0;
     if (t[3] > 0) {
         c->flat = t[3];
@@ -1698,10 +1799,11 @@ psc_status psc_batch_autotune(psc_batch *b, int *tiling_out) {
     std::vector<std::vector<std::pair<float, Tiling>>> timed(n);
     std::vector<int> reused(n, -1);
     auto time_eval = [&](psc_ctx *c, int k, float *ms) -> psc_status {
-        psc_status st = ensure_partials(c);
+        const Shape shape = eval_shape(c);
+        psc_status st = ensure_partials(c, shape);
         if (st != PSC_OK) return bfail(b, st, c->err);
-        if (c->trk_kv == 0) PSC_BCUDA(b, set_eval_smem(eval_dyn_smem(ch_span(c), tab_stride(c, c->kv))));
-        EvalArgs a = eval_args(c, c->d_lm_trial);
+        if (shape.trk_kv == 0) PSC_BCUDA(b, set_eval_smem(eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv))));
+        EvalArgs a = eval_args(c, shape, c->d_lm_trial);
         a.vis_obs = (const float2 *)b->vis[k];
         a.w = b->w[k];
         a.w_scale = (float)b->w_scale[k];
@@ -1755,23 +1857,25 @@ psc_status psc_batch_autotune(psc_batch *b, int *tiling_out) {
     // shape is narrower take their fastest timed shape of the widest size
     int width = 32;
     for (int k = 0; k < n; ++k)
-        if (reused[k] < 0) width = std::max(width, eval_threads(b->ctxs[k]));
+        if (reused[k] < 0) width = std::max(width, eval_threads(eval_shape(b->ctxs[k])));
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
         c->trk_kv = 0;
         if (reused[k] >= 0) {
             const psc_ctx *o = b->ctxs[reused[k]];
+            c->auto_shape = false;
+            c->trk_set = true;
             c->no_stage = o->no_stage;
             c->c_group = o->c_group;
             c->kv = kv_allowed(c, o->kv) ? o->kv : 1;
             c->flat = o->flat;
-            if (c->flat > 0 && ch_span(c) > 8) {          // a shorter interval: fall back to the default shape
+            if (c->flat > 0 && flat_span(c, c->flat, c->kv) > 8) {          // a shorter interval: fall back to the default shape
                 c->flat = 0;
                 c->c_group = 4;
             }
             if (c->flat == 0)
-                c->t_tile = fit_t_tile(c->nt, o->flat > 0 ? o->flat : eval_threads(o), c->c_group, c->kv);
-        } else if (eval_threads(c) != width) {
+                c->t_tile = fit_t_tile(c->nt, o->flat > 0 ? o->flat : eval_threads(brick_shape(o)), c->c_group, c->kv);
+        } else if (eval_threads(brick_shape(c)) != width) {
             float best = 1e30f;
             for (const auto &x : timed[k]) {
                 const Tiling &t = x.second;

@@ -69,13 +69,108 @@ struct BlockSharedT {
     int taps;          // taps of the brick's visibilities (pi rho_max^2 each, rounded up)
 };
 
+// The tap sums of a rectangle's visibilities with a.split lanes per visibility:
+// lane g takes rows g, g + split, ..., the row sums go through shared memory, and
+// three of the lanes add them up in row order -- the additions of the one-lane loop
+// in eval_brick, so every sum has the same bits.  For contexts with too few
+// visibilities to fill the chip, where a lane's chain of some 600 taps is what the
+// launch waits for: 21,060 visibilities, 185 us with a lane each, 72 us with 8.  Shared memory s_split: [kMaxThreads] windows, [kMaxThreads][6] sums, then
+// [kMaxThreads / split][support] row sums (P, Q).
+__device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_tab, const BlockSharedT<true> &sh,
+                                           float4 *s_split, int bl, int brick, int c_first, bool staged, int bx0, int by0) {
+    const int tid = threadIdx.x, S = a.support;
+    const int grp = tid / a.split, sub = tid & (a.split - 1), groups = blockDim.x / a.split;
+    const int t_first = (brick % a.n_tt) * a.t_tile;
+    const int n_t = min(a.t_tile, a.nt - t_first), n_c = min(a.c_group, a.nc - c_first);
+    float *sums = reinterpret_cast<float *>(s_split + kMaxThreads);
+    float4 *rows = s_split + kMaxThreads + kMaxThreads * 6 / 4 + grp * S;
+    const float ov = (float)a.ov;
+    for (int i0 = 0; i0 < n_t * n_c; i0 += groups) {
+        const int i = i0 + grp;
+        const bool on = i < n_t * n_c;
+        const int lc = on ? i / n_t : 0, slot = on ? lc * a.t_tile + (i - lc * n_t) : 0;
+        const float4 win = s_split[slot];
+        const int ix0 = __float_as_int(win.x), iy0 = __float_as_int(win.y);
+        const float hx = win.z, hy = win.w;
+        const float rmax = a.chan[c_first + lc].rho_max, rmax2 = __fmul_rn(rmax, rmax);
+        const unsigned tab_adj = (unsigned)__cvta_generic_to_shared(s_tab + lc * a.tab_stride) - (0x4B000000u << 3);
+        int b_lo = max(0, (int)floorf(hy - rmax) + 1), b_hi = min(S - 1, (int)ceilf(hy + rmax) - 1);
+        if (!staged) {
+            b_lo = max(b_lo, -iy0);
+            b_hi = min(b_hi, a.ng - 1 - iy0);
+        }
+        if (!on) b_hi = b_lo - 1;
+        for (int b = b_lo + sub; b <= b_hi; b += a.split) {
+            const float dy = hy - (float)b;
+            const float dyo = dy * ov;
+            const float dyo2 = fmaf(dyo, dyo, 1e-20f);
+            const float rem = fmaf(-dy, dy, rmax2);      // written out, as are its factors: the span must not differ by a tap
+            float2 P = make_float2(0.f, 0.f), Q = P;
+            if (rem > 0.f) {
+                const float r = fminf(rem * rsqrt_fast(rem), rmax);
+                int a_lo = max(0, (int)floorf(hx - r) + 1), a_hi = min(S - 1, (int)ceilf(hx + r) - 1);
+                if (staged) {
+                    if (a_lo <= a_hi) {
+                        float dxo[1] = {(hx - (float)a_lo) * ov}, d2[1] = {dyo2};
+                        float pr[1] = {0.f}, pi[1] = {0.f}, qr[1] = {0.f}, qi[1] = {0.f};
+                        row_taps<1>(sh.tile + (iy0 - by0 + b) * kTile + (ix0 - bx0 + a_lo), a_hi - a_lo + 1, dxo, d2, ov,
+                                    tab_adj, pr, pi, qr, qi);
+                        P = make_float2(pr[0], pi[0]);
+                        Q = make_float2(qr[0], qi[0]);
+                    }
+                } else {
+                    a_lo = max(a_lo, -ix0);
+                    a_hi = min(a_hi, a.ng - 1 - ix0);
+                    float pr = 0.f, pi = 0.f, qr = 0.f, qi = 0.f;
+                    const size_t row = (size_t)(iy0 + b) * a.ng + ix0;
+                    float dd = (hx - (float)a_lo) * ov;
+#pragma unroll 4
+                    for (int aa = a_lo; aa <= a_hi; ++aa, dd -= ov) {
+                        const float2 g = cmul(grid_cell(a, row + aa), sh.phx[aa]);
+                        const float s2 = fmaf(dd, dd, dyo2);
+                        const float tv = sqrt_fast(s2);
+                        const float tf = __fadd_rz(tv, 8388608.0f);
+                        const float2 e = lds_f2(tab_adj + ((unsigned)__float_as_int(tf) << 3));
+                        const float A = fmaf(tv, e.y, e.x);
+                        pr = fmaf(A, g.x, pr);
+                        pi = fmaf(A, g.y, pi);
+                        const float Ad = A * dd;
+                        qr = fmaf(Ad, g.x, qr);
+                        qi = fmaf(Ad, g.y, qi);
+                    }
+                    const float2 py = sh.phy[b];
+                    P = cmul(make_float2(pr, pi), py);
+                    Q = cmul(make_float2(qr, qi), py);
+                }
+            }
+            rows[b] = make_float4(P.x, P.y, Q.x, Q.y);
+        }
+        __syncwarp();
+        if (on && sub < 3) {
+            // lane 0: sum P, lane 1: sum Q, lane 2: sum dy P, in row order
+            float x = 0.f, y = 0.f;
+            for (int b = b_lo; b <= b_hi; ++b) {
+                const float2 v = reinterpret_cast<const float2 *>(rows + b)[sub == 1];
+                const float dy = hy - (float)b;
+                x = sub == 2 ? fmaf(dy, v.x, x) : x + v.x;
+                y = sub == 2 ? fmaf(dy, v.y, y) : y + v.y;
+            }
+            sums[6 * slot + 2 * sub] = x;
+            sums[6 * slot + 2 * sub + 1] = y;
+        }
+        __syncwarp();
+    }
+}
+
 // One brick: kv visibilities per thread.  acc receives the thread's 15 sums
 // (reduce mode); predict mode writes V and the derivative planes.
 // kW: the grid is a residual-w stack (EvalArgs::wp_n); every tap reads the two
 // planes around its visibility's w and interpolates, unstaged.
-template <bool kPredict, int kV, bool kW>
+// kSplit: the rows of each visibility are shared among a.split lanes (split_taps);
+// the brick, its sums and their order are those of the rectangle without it.
+template <bool kPredict, int kV, bool kW, bool kSplit>
 __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 *s_tab, BlockSharedT<!kW> &sh,
-                                           float (&acc)[kRed]) {
+                                           float4 *s_split, float (&acc)[kRed]) {
     const int tid = threadIdx.x;
     // brick -> baseline, this thread's channel c and first time step t0, and
     // the block's channels [c_first, c_first + n_ch) (lc = c - c_first)
@@ -245,7 +340,21 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
     float2 S0[kV], Su[kV], Sv[kV];
 #pragma unroll
     for (int v = 0; v < kV; ++v) S0[v] = Su[v] = Sv[v] = make_float2(0.f, 0.f);
-    if (active && !empty) {
+    if constexpr (kSplit) {
+        // each rectangle slot's window, then its sums in the same place
+        if (active) s_split[tid] = make_float4(__int_as_float(ix0[0]), __int_as_float(iy0[0]), hx[0], hy[0]);
+        __syncthreads();
+        if (!empty) split_taps(a, s_tab, sh, s_split, bl, brick, c_first, staged, bx0, by0);
+        __syncthreads();
+        if (active && !empty) {
+            const float *r = reinterpret_cast<const float *>(s_split + kMaxThreads) + 6 * tid;
+            S0[0] = make_float2(r[0], r[1]);
+            Su[0] = make_float2(r[2], r[3]);
+            Sv[0] = make_float2(r[4], r[5]);
+            const float inv_ov = 1.0f / (float)a.ov;
+            Su[0].x *= inv_ov; Su[0].y *= inv_ov;
+        }
+    } else if (active && !empty) {
         const float2 *tab = s_tab + lc * tab_stride;
         const unsigned tab_adj = (unsigned)__cvta_generic_to_shared(tab) - (0x4B000000u << 3);
         const float ov = (float)a.ov;
@@ -431,11 +540,13 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
 // more from the warps than they lose (vla27_l64ch as one interval: 5.56 ms
 // against 6.36 ms at 99 registers).  A minimum of 0 leaves the co-planar
 // instantiations with the plain bound.
-template <bool kPredict, bool kW>
-__global__ void __launch_bounds__(kMaxThreads, kW ? 4 : 0) eval_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args,
+// kSplit: the instantiation that also runs split items (its co-planar contexts
+// without them take the same code as before, at this kernel's registers).
+template <bool kPredict, bool kW, bool kSplit>
+__global__ void __launch_bounds__(kMaxThreads, kW ? 4 : kSplit ? 3 : 0) eval_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args,
                                                            const long long *__restrict__ prefix, int n_ctx,
                                                            unsigned long long *queue) {
-    extern __shared__ float2 s_tab[];                 // c_group * tab_stride
+    extern __shared__ __align__(16) float2 s_tab[];   // c_group * tab_stride, then split_taps' arrays (16-byte aligned)
     __shared__ BlockSharedT<!kW> sh;
     __shared__ EvalArgs s_a;
     __shared__ long long s_work, s_first;
@@ -482,8 +593,10 @@ __global__ void __launch_bounds__(kMaxThreads, kW ? 4 : 0) eval_kernel(const Eva
     float acc[kRed];
 #pragma unroll
     for (int k = 0; k < kRed; ++k) acc[k] = 0.f;
-    if (a.kv == 2) eval_brick<kPredict, 2, kW>(a, brick, s_tab, sh, acc);
-    else eval_brick<kPredict, 1, kW>(a, brick, s_tab, sh, acc);
+    float4 *s_split = reinterpret_cast<float4 *>(s_tab + (a.c_group * a.tab_stride + 1) / 2 * 2);
+    if (kSplit && a.split > 1) eval_brick<kPredict, 1, kW, kSplit>(a, brick, s_tab, sh, s_split, acc);
+    else if (a.kv == 2) eval_brick<kPredict, 2, kW, false>(a, brick, s_tab, sh, nullptr, acc);
+    else eval_brick<kPredict, 1, kW, false>(a, brick, s_tab, sh, nullptr, acc);
     if constexpr (!kPredict) {
         // ---- block reduction: a butterfly within each warp -- compensated
         // (Knuth's TwoSum, the rounding errors summed beside) for chi^2 and the
@@ -695,35 +808,46 @@ size_t eval_dyn_smem(int c_group, int tab_stride) {
     return sizeof(float2) * (size_t)c_group * tab_stride;
 }
 
+// split_taps' share of a block's dynamic shared memory (and its alignment).
+size_t eval_split_smem(int split, int support) {
+    return split > 1 ? 16 + sizeof(float4) * (kMaxThreads + kMaxThreads * 6 / 4 + (size_t)(kMaxThreads / split) * support) : 0;
+}
+
 cudaError_t launch_eval(const EvalArgs &a, bool predict, cudaStream_t s) {
     if (a.exact) return launch_exact(a, predict, s);
-    const int threads = ((a.flat > 0 ? a.flat : a.t_tile * a.c_group) + 31) / 32 * 32;
+    const int threads = a.split > 1 ? kMaxThreads : ((a.flat > 0 ? a.flat : a.t_tile * a.c_group) + 31) / 32 * 32;
     const int blocks = (int)a.n_bricks;
-    const size_t dyn = eval_dyn_smem(a.flat > 0 ? a.ch_span : a.c_group, a.tab_stride);
+    const size_t dyn = eval_dyn_smem(a.flat > 0 ? a.ch_span : a.c_group, a.tab_stride) + eval_split_smem(a.split, a.support);
     if (a.wp_n > 0) {
-        if (predict) eval_kernel<true, true><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
-        else eval_kernel<false, true><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+        if (predict) eval_kernel<true, true, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+        else eval_kernel<false, true, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+    } else if (a.split > 1) {
+        if (predict) eval_kernel<true, false, true><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+        else eval_kernel<false, false, true><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
     } else if (predict) {
-        eval_kernel<true, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+        eval_kernel<true, false, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
     } else {
-        eval_kernel<false, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
+        eval_kernel<false, false, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_eval_batch(const EvalArgs *args_dev, const long long *prefix_dev, int n_ctx,
-                              unsigned long long *queue, int threads, size_t dyn, int grid, bool stacked,
+                              unsigned long long *queue, int threads, size_t dyn, int grid, bool stacked, bool split,
                               cudaStream_t s) {
     EvalArgs none{};
-    if (stacked) eval_kernel<false, true><<<grid, threads, dyn, s>>>(none, args_dev, prefix_dev, n_ctx, queue);
-    else eval_kernel<false, false><<<grid, threads, dyn, s>>>(none, args_dev, prefix_dev, n_ctx, queue);
+    if (stacked) eval_kernel<false, true, false><<<grid, threads, dyn, s>>>(none, args_dev, prefix_dev, n_ctx, queue);
+    else if (split) eval_kernel<false, false, true><<<grid, threads, dyn, s>>>(none, args_dev, prefix_dev, n_ctx, queue);
+    else eval_kernel<false, false, false><<<grid, threads, dyn, s>>>(none, args_dev, prefix_dev, n_ctx, queue);
     return cudaGetLastError();
 }
 
-cudaError_t eval_batch_occupancy(int threads, size_t dyn, bool stacked, int *blocks_per_sm) {
+cudaError_t eval_batch_occupancy(int threads, size_t dyn, bool stacked, bool split, int *blocks_per_sm) {
     if (stacked)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, eval_kernel<false, true>, threads, dyn);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, eval_kernel<false, false>, threads, dyn);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, eval_kernel<false, true, false>, threads, dyn);
+    if (split)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, eval_kernel<false, false, true>, threads, dyn);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, eval_kernel<false, false, false>, threads, dyn);
 }
 
 // Dynamic shared memory the fused kernel can have on the current device: the
@@ -735,7 +859,7 @@ cudaError_t eval_smem_allowed(size_t *allowed) {
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     cudaFuncAttributes fa{};
-    e = cudaFuncGetAttributes(&fa, eval_kernel<false, false>);
+    e = cudaFuncGetAttributes(&fa, eval_kernel<false, false, false>);
     if (e != cudaSuccess) return e;
     *allowed = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
     return cudaSuccess;
@@ -750,8 +874,9 @@ cudaError_t set_eval_smem(size_t dyn) {
     cudaError_t e = eval_smem_allowed(&allowed);
     if (e != cudaSuccess) return e;
     if (dyn > allowed) return cudaErrorInvalidValue;
-    for (const void *k : {(const void *)eval_kernel<true, false>, (const void *)eval_kernel<false, false>,
-                          (const void *)eval_kernel<true, true>, (const void *)eval_kernel<false, true>}) {
+    for (const void *k : {(const void *)eval_kernel<true, false, false>, (const void *)eval_kernel<false, false, false>,
+                          (const void *)eval_kernel<true, true, false>, (const void *)eval_kernel<false, true, false>,
+                          (const void *)eval_kernel<true, false, true>, (const void *)eval_kernel<false, false, true>}) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)allowed);
         if (e != cudaSuccess) return e;
     }

@@ -57,6 +57,7 @@ struct EvalArgs {
     // holds items [b flat, (b + 1) flat), so bpb bricks per baseline, each
     // spanning at most ch_span channels.
     int flat, n_tp, bpb, ch_span;
+    int split;                 // rectangular bricks: lanes that share a visibility's rows (1, or 4 .. 32, a power of two)
     // nullptr, or [n_bl]: the baseline of each group of bpb consecutive bricks in
     // launch order (partials stay indexed by baseline: brick = bl * bpb + j)
     const int *bl_order;
@@ -176,11 +177,12 @@ cudaError_t launch_uvw(const double *enu_dev, int n_ant, double lat, double dec,
 cudaError_t launch_eval(const EvalArgs &a, bool predict, cudaStream_t s);
 // Persistent fused launch over several contexts (device arrays of EvalArgs and
 // first-brick prefixes [n_ctx + 1]; *queue must be zero at launch).  stacked:
-// every context reads a residual-w stack (else none does).
+// every context reads a residual-w stack (else none does); split: some context
+// shares its visibilities among lanes (EvalArgs::split).
 cudaError_t launch_eval_batch(const EvalArgs *args_dev, const long long *prefix_dev, int n_ctx,
                               unsigned long long *queue, int threads, size_t dyn, int grid, bool stacked,
-                              cudaStream_t s);
-cudaError_t eval_batch_occupancy(int threads, size_t dyn, bool stacked, int *blocks_per_sm);
+                              bool split, cudaStream_t s);
+cudaError_t eval_batch_occupancy(int threads, size_t dyn, bool stacked, bool split, int *blocks_per_sm);
 cudaError_t launch_reduce(const RedArgs &r, cudaStream_t s);
 cudaError_t launch_reduce_batch(const RedArgs *ra_dev, const int *bl_prefix_dev, int n_ctx, int total_bl, int max_bpb,
                                 int max_ant, cudaStream_t s);
@@ -215,6 +217,7 @@ cudaError_t launch_exact(const EvalArgs &a, bool predict, cudaStream_t s);
 size_t exact_dyn_smem(int c_group, int tab_stride);
 cudaError_t launch_exact_moments(double diam_m, const double *freq_dev, int nc, double du, int ov,
                                  const int *tab_off_dev, const int *tab_len_dev, float *kmom, cudaStream_t s);
+size_t eval_split_smem(int split, int support);
 // Dynamic shared memory of one fused-kernel block (c_group zero-padded tables).
 size_t eval_dyn_smem(int c_group, int tab_stride);
 // Largest distance (metres, u-v plane) between the baselines of consecutive
