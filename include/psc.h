@@ -346,7 +346,13 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * refused (PSC_ERR_ARG) unless every channel's aperture lies inside the
  * S x S tap window and consecutive time steps move a baseline by at most 4
  * grid cells at the highest frequency.  Results do not depend on the shape
- * beyond FP32 summation order. */
+ * beyond FP32 summation order.
+ * A context without a tiling (its current values then count as 32, 4, 1) picks its
+ * launch shape by size: from two million visibilities on, flat bricks
+ * (psc_set_flat_tiling) or, for small apertures and enough baselines, the track
+ * kernel (psc_set_track_tiling; in a batch only if every context would); below, the
+ * rectangle (32, 4, 1), with the rows of each visibility shared among lanes where
+ * there are too few visibilities to fill the chip (the same sums bit for bit). */
 psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thread);
 
 /* Flat bricks: the fused kernel's work items of a baseline are its (channel,

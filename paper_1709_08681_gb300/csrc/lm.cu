@@ -21,17 +21,18 @@
 // factored in FP64 instead.
 //
 // Shape.  What costs here is not arithmetic (20 M multiply-adds for 197
-// antennas) but serial chains, on one SM at that.  So nothing but the pivots
-// of a 32 x 32 diagonal block runs in sequence: one warp factors it in
-// registers and inverts it, the rows below are a product with that inverse, the
-// trailing update goes in 64 x 64 tiles, and once L is complete W = L^-1 is
-// formed by columns, so that each refinement round is two matrix-vector
-// products (W, then W^T) and one FP64 residual, all parallel over rows.  Systems
-// up to 2 n_ant = 90 run in one block with the matrices in shared memory; larger
-// ones on a cluster of eight blocks with the matrices in L2, every block
-// factoring the diagonal block for itself (cheaper than waiting for it).
-// Measured: 27 antennas 63 us a call (one column at a time: 75), 197 antennas 369
-// us (one block, solves from the factor: 1810).
+// antennas) but serial chains, on one SM at that.  So as little as possible runs in
+// sequence, and each refinement round is a product with an explicit inverse.
+// Up to 2 n_ant = 90, one block inverts the matrix by Gauss-Jordan elimination in
+// registers (6 x 6 elements a thread, one barrier a pivot).  Larger systems run on
+// a cluster of eight blocks with the matrices in L2: one warp of each factors a
+// 32 x 32 diagonal block in registers and inverts it (every block for itself,
+// cheaper than waiting for it), the rows below are a product with that inverse,
+// the trailing update goes in 64 x 64 tiles, and once L is complete W = L^-1 is
+// formed by columns; a round is then y = W r, d += W^T y.
+// Measured: 27 antennas 36 us a call (Cholesky column by column: 75; the
+// cluster form on one block: 63), 197
+// antennas 369 us (one block, solves from the factor: 1810).
 #include <math.h>
 
 #include <algorithm>
@@ -51,11 +52,6 @@ constexpr int kPan = 32;                // panel width of the factorisation: one
 constexpr int kTile = 64;               // trailing-update tile, 4 x 4 elements per thread
 constexpr int kLd = kPan + 1;           // padded row of the shared tiles
 constexpr unsigned kFull = 0xffffffffu;
-
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
-}
 
 __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
@@ -99,7 +95,7 @@ __host__ __device__ inline size_t tile_floats(int n2) {
 }
 
 // The matrices and exchanged vectors of one system: shared memory (small) or
-// the context's mat and mat32 (large).
+// the context's mat and mat32 (large).  Small systems keep A^-1 in place of A.
 struct SysMem {
     float *A;          // [n2][n2] lower triangle of the damped matrix, then L below its diagonal blocks
     float *W;          // [n2][n2] lower triangle: L^-1
@@ -140,8 +136,8 @@ __device__ __forceinline__ int chol_diag(float *D, float *I) {
         }
         if (lane == c) I[c] = inv;                      // 1 / L_cc for the inverse, below
     }
-    // the empty asm statements keep the compiler from merging these phases: in one of
-    // the two forms it did, and the function took 63 us instead of 5
+    // the empty asm statements keep the compiler from merging these phases: where it
+    // did, the function took 63 us instead of 5
     asm volatile("" ::: "memory");
     __syncwarp();
 #pragma unroll
@@ -171,9 +167,72 @@ __device__ __forceinline__ int chol_diag(float *D, float *I) {
     return bad;
 }
 
-// A = L L^T and W = L^-1 of one system (see the file header).  Returns nonzero
+// W = A^-1 (both triangles, rows of ldw) of a small system from A's lower triangle,
+// by Gauss-Jordan elimination without pivoting (A is positive definite: its pivots
+// are those of Cholesky's factorisation, squared).  Thread (tx, ty) holds elements
+// (ty + 16 i, tx + 16 j); rc: 4 x 96 floats.  W may be A itself.  Returns nonzero
 // (uniformly) if a pivot is not positive.
-template <bool kLarge>
+constexpr int kGj = (kSmallN2 + 15) / 16;
+__device__ int gauss_jordan(const float *A, float *W, int ldw, int n, float *rc) {
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    float a[kGj][kGj];
+#pragma unroll
+    for (int i = 0; i < kGj; ++i)
+#pragma unroll
+        for (int j = 0; j < kGj; ++j) {
+            const int r = ty + 16 * i, c = tx + 16 * j;
+            a[i][j] = r < n && c < n ? A[(size_t)max(r, c) * n + min(r, c)] : (r == c ? 1.f : 0.f);
+        }
+    int bad = 0;
+#pragma unroll
+    for (int kb = 0; kb < kGj; ++kb) {
+        const int k_hi = min(16, n - 16 * kb);
+        for (int kk = 0; kk < k_hi; ++kk) {
+            float *row = rc + (kk & 1) * 192, *col = row + 96;
+            if (ty == kk) {
+#pragma unroll
+                for (int j = 0; j < kGj; ++j) row[tx + 16 * j] = a[kb][j];
+            }
+            if (tx == kk) {
+#pragma unroll
+                for (int i = 0; i < kGj; ++i) col[ty + 16 * i] = a[i][kb];
+            }
+            __syncthreads();
+            const float p = row[16 * kb + kk];
+            const bool nonpos = !(p > 0.f);
+            bad |= nonpos;
+            const float rp = nonpos ? 1.f : 1.f / p;
+            float rj[kGj];
+#pragma unroll
+            for (int j = 0; j < kGj; ++j) rj[j] = row[tx + 16 * j] * rp;
+            const bool my_row = ty == kk, my_col = tx == kk;
+#pragma unroll
+            for (int i = 0; i < kGj; ++i) {
+                const float ci = col[ty + 16 * i];
+#pragma unroll
+                for (int j = 0; j < kGj; ++j) {
+                    float v = fmaf(-ci, rj[j], a[i][j]);
+                    if (j == kb && my_col) v = -ci * rp;
+                    if (i == kb && my_row) v = j == kb && my_col ? rp : rj[j];
+                    a[i][j] = v;
+                }
+            }
+        }
+        __syncthreads();                                 // an odd count would reuse the buffer still being read
+    }
+#pragma unroll
+    for (int i = 0; i < kGj; ++i)
+#pragma unroll
+        for (int j = 0; j < kGj; ++j) {
+            const int r = ty + 16 * i, c = tx + 16 * j;
+            if (r < n && c < n) W[(size_t)r * ldw + c] = a[i][j];
+        }
+    __syncthreads();
+    return bad;
+}
+
+// A = L L^T and W = L^-1 of one large system (see the file header).  Returns nonzero
+// (uniformly) if a pivot is not positive.
 __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nblk) {
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -186,7 +245,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
         const int kb = min(kPan, n - k0), m0 = k0 + kb;
         for (int e = tid; e < kPan * kPan; e += kLmThreads) {
             const int r = e / kPan, c = e % kPan;
-            D[r * kLd + c] = (r < kb && c <= r) ? ld<kLarge>(&A[(size_t)(k0 + r) * n + k0 + c]) : (r == c ? 1.f : 0.f);
+            D[r * kLd + c] = (r < kb && c <= r) ? ld<true>(&A[(size_t)(k0 + r) * n + k0 + c]) : (r == c ? 1.f : 0.f);
         }
         __syncthreads();
         if (warp == 0) {
@@ -206,9 +265,9 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
             for (int t = 0; t < kPan; ++t) li[t] = I[lane * kLd + t];
             const int step = nblk * kWarps;
             int i = m0 + rank * kWarps + warp;
-            float a = i < n ? ld<kLarge>(&A[(size_t)i * n + k0 + lane]) : 0.f;
+            float a = i < n ? ld<true>(&A[(size_t)i * n + k0 + lane]) : 0.f;
             for (; i < n; i += step) {
-                const float next = i + step < n ? ld<kLarge>(&A[(size_t)(i + step) * n + k0 + lane]) : 0.f;
+                const float next = i + step < n ? ld<true>(&A[(size_t)(i + step) * n + k0 + lane]) : 0.f;
                 float s0 = 0.f, s1 = 0.f;
 #pragma unroll
                 for (int t = 0; t < kPan; t += 2) {
@@ -219,7 +278,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
                 a = next;
             }
         }
-        sys_sync<kLarge>();
+        sys_sync<true>();
         // trailing update: A22 -= L21 L21^T on the lower triangle, tile by tile
         const int nt = (n - m0 + kTile - 1) / kTile;
         int t = 0;
@@ -229,8 +288,8 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
                 const int i0 = m0 + ti * kTile, j0 = m0 + tj * kTile;
                 for (int e = tid; e < kTile * kPan; e += kLmThreads) {
                     const int r = e / kPan, c = e % kPan;
-                    Ti[r * kLd + c] = i0 + r < n ? ld<kLarge>(&A[(size_t)(i0 + r) * n + k0 + c]) : 0.f;
-                    Tj[r * kLd + c] = j0 + r < n ? ld<kLarge>(&A[(size_t)(j0 + r) * n + k0 + c]) : 0.f;
+                    Ti[r * kLd + c] = i0 + r < n ? ld<true>(&A[(size_t)(i0 + r) * n + k0 + c]) : 0.f;
+                    Tj[r * kLd + c] = j0 + r < n ? ld<true>(&A[(size_t)(j0 + r) * n + k0 + c]) : 0.f;
                 }
                 float acc[4][4];
 #pragma unroll
@@ -239,7 +298,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const int j = j0 + tx + 16 * c;
-                        acc[r][c] = i < n && j <= i ? ld<kLarge>(&A[(size_t)i * n + j]) : 0.f;
+                        acc[r][c] = i < n && j <= i ? ld<true>(&A[(size_t)i * n + j]) : 0.f;
                     }
                 }
                 __syncthreads();
@@ -266,7 +325,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
                 }
                 __syncthreads();
             }
-        sys_sync<kLarge>();
+        sys_sync<true>();
     }
     const int bad = s_bad;
     // W below its diagonal blocks: W_ij = -W_ii sum_{j <= k < i} L_ik W_kj, one block of
@@ -284,7 +343,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
         const int j0 = (u >> 1) * kPan, cj = j0 + 16 * (u & 1);
         for (int e = tid; e < kPan * 16; e += kLmThreads) {
             const int r = e / 16, c = e % 16;
-            Wj[e] = j0 + r < n && cj + c < n ? ld<kLarge>(&W[(size_t)(j0 + r) * n + cj + c]) : 0.f;
+            Wj[e] = j0 + r < n && cj + c < n ? ld<true>(&W[(size_t)(j0 + r) * n + cj + c]) : 0.f;
         }
         __syncthreads();
         for (int i = (u >> 1) + 1; i < nb; ++i) {
@@ -293,8 +352,8 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int row = 4 * warp + r;
-                pre[r] = row < ib ? ld<kLarge>(&A[(size_t)(i0 + row) * n + j0 + lane]) : 0.f;
-                wii[r] = row < ib && lane < ib ? ld<kLarge>(&W[(size_t)(i0 + row) * n + i0 + lane]) : 0.f;
+                pre[r] = row < ib ? ld<true>(&A[(size_t)(i0 + row) * n + j0 + lane]) : 0.f;
+                wii[r] = row < ib && lane < ib ? ld<true>(&W[(size_t)(i0 + row) * n + i0 + lane]) : 0.f;
             }
             for (int k0 = j0; k0 < i0; k0 += kPan) {
                 __syncwarp();
@@ -302,7 +361,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
                 for (int r = 0; r < 4; ++r) {
                     Ls[r * kPan + lpos] = pre[r];
                     if (k0 + kPan < i0 && 4 * warp + r < ib)
-                        pre[r] = ld<kLarge>(&A[(size_t)(i0 + 4 * warp + r) * n + k0 + kPan + lane]);
+                        pre[r] = ld<true>(&A[(size_t)(i0 + 4 * warp + r) * n + k0 + kPan + lane]);
                 }
                 __syncwarp();
                 const float *w = Wj + (k0 - j0) * 16 + lane;             // rows k0 + 2 q + par, column col
@@ -339,7 +398,7 @@ __device__ int factor_invert(const SysMem &m, int n, float *ws, int rank, int nb
             __syncthreads();
         }
     }
-    sys_sync<kLarge>();
+    sys_sync<true>();
     return bad;
 }
 
@@ -383,7 +442,11 @@ __device__ bool solve_damped(const LMArgs &a, const double *src, double lam, con
         r1[1] = pm && qm ? (float)x[3] : 0.f;
     }
     sys_sync<kLarge>();
-    if (factor_invert<kLarge>(m, n2, sh.ws, rank, nblk)) return false;
+    if constexpr (kLarge) {
+        if (factor_invert(m, n2, sh.ws, rank, nblk)) return false;
+    } else {
+        if (gauss_jordan(m.A, m.W, n2 + 1, n2, sh.ws)) return false;
+    }
     double bmax = 0.0;
     for (int p = tid; p < n2; p += kLmThreads) bmax = fmax(bmax, fabs(sh.b[p]));
     bmax = block_max(bmax, s_tmp);
@@ -391,36 +454,48 @@ __device__ bool solve_damped(const LMArgs &a, const double *src, double lam, con
     for (int it = 0; it < kRefineMax; ++it) {
         for (int p = tid; p < n2; p += kLmThreads) sh.r32[p] = (float)sh.r[p];
         __syncthreads();
-        for (int p = rank * kWarps + warp; p < n2; p += nblk * kWarps) {       // y = W r
-            const float *row = m.W + (size_t)p * n2;
-            float s = 0.f;
-            for (int c = lane; c <= p; c += 32) s = fmaf(ld<kLarge>(&row[c]), sh.r32[c], s);
-            s = warp_sum(s);
-            if (lane == 0) m.y[p] = s;
-        }
-        sys_sync<kLarge>();
-        for (int p = tid; p < n2; p += kLmThreads) sh.y[p] = ld<kLarge>(&m.y[p]);
-        __syncthreads();
-        for (int c0 = 32 * rank; c0 < n2; c0 += 32 * nblk) {                   // d += W^T y, 32 columns at a time
-            const int c = c0 + lane;
-            float s = 0.f;
-            if (c < n2) {
-#pragma unroll 8
-                for (int p = c0 + warp; p < n2; p += kWarps)
-                    s = fmaf(p >= c ? ld<kLarge>(&m.W[(size_t)p * n2 + c]) : 0.f, sh.y[p], s);
-            }
-            red[warp * 32 + lane] = s;
-            __syncthreads();
-            if (warp == 0 && c < n2) {
+        if constexpr (!kLarge) {                             // d += A^-1 r, four lanes a row
+            for (int p = tid >> 2; p < (n2 + 7) / 8 * 8; p += kLmThreads / 4) {
                 float v = 0.f;
-                for (int w = 0; w < kWarps; ++w) v += red[w * 32 + lane];
-                m.d[c] = it == 0 ? (double)v : m.d[c] + (double)v;
+                if (p < n2)
+                    for (int c = tid & 3; c < n2; c += 4) v = fmaf(m.W[(size_t)p * (n2 + 1) + c], sh.r32[c], v);
+                v += __shfl_xor_sync(kFull, v, 1);
+                v += __shfl_xor_sync(kFull, v, 2);
+                if (p < n2 && (tid & 3) == 0) sh.d[p] = it == 0 ? (double)v : sh.d[p] + (double)v;
             }
             __syncthreads();
+        } else {
+            for (int p = rank * kWarps + warp; p < n2; p += nblk * kWarps) {       // y = W r
+                const float *row = m.W + (size_t)p * n2;
+                float s = 0.f;
+                for (int c = lane; c <= p; c += 32) s = fmaf(ld<kLarge>(&row[c]), sh.r32[c], s);
+                s = warp_sum(s);
+                if (lane == 0) m.y[p] = s;
+            }
+            sys_sync<kLarge>();
+            for (int p = tid; p < n2; p += kLmThreads) sh.y[p] = ld<kLarge>(&m.y[p]);
+            __syncthreads();
+            for (int c0 = 32 * rank; c0 < n2; c0 += 32 * nblk) {                   // d += W^T y, 32 columns at a time
+                const int c = c0 + lane;
+                float s = 0.f;
+                if (c < n2) {
+#pragma unroll 8
+                    for (int p = c0 + warp; p < n2; p += kWarps)
+                        s = fmaf(p >= c ? ld<kLarge>(&m.W[(size_t)p * n2 + c]) : 0.f, sh.y[p], s);
+                }
+                red[warp * 32 + lane] = s;
+                __syncthreads();
+                if (warp == 0 && c < n2) {
+                    float v = 0.f;
+                    for (int w = 0; w < kWarps; ++w) v += red[w * 32 + lane];
+                    m.d[c] = it == 0 ? (double)v : m.d[c] + (double)v;
+                }
+                __syncthreads();
+            }
+            sys_sync<kLarge>();
+            for (int p = tid; p < n2; p += kLmThreads) sh.d[p] = ld<kLarge>(&m.d[p]);
+            __syncthreads();
         }
-        sys_sync<kLarge>();
-        for (int p = tid; p < n2; p += kLmThreads) sh.d[p] = ld<kLarge>(&m.d[p]);
-        __syncthreads();
         // r = b - A d in FP64, eight lanes per antenna: a warp's FP64 instruction costs
         // the same for one lane as for 32, so few lanes may idle
         for (int a0 = (rank * kWarps + warp) * 4; a0 < n; a0 += nblk * kWarps * 4) {
@@ -620,8 +695,8 @@ __device__ void lm_update(const LMArgs &a, double *s_dyn, int rank, int nblk) {
             m.r = a.mat + ((size_t)n2 * n2 + 1) / 2;
             m.y = (float *)(m.r + n2);
         } else {
-            m.A = sh.ws + tile_floats(n2);
-            m.W = m.A + (size_t)n2 * n2;
+            m.A = sh.ws + 4 * 96;
+            m.W = m.A;
             m.r = sh.r;
             m.y = sh.y;
             m.d = sh.d;
@@ -685,14 +760,15 @@ __global__ void lm_restart_kernel(const LMArgs a0, const LMState *st00, const do
     }
 }
 
-// Dynamic shared memory of the LM kernel: six vectors (b, r, d in FP64; r, y in
-// FP32; the flags), the tiles, and for small systems both matrices
-// and the cross blocks.
+// Dynamic shared memory of the LM kernels: six vectors (b, r, d in FP64; r, y in
+// FP32; the flags), then the tiles (large systems) or the pivot rows, the matrix (its
+// inverse has rows of n2 + 1) and the cross blocks (small ones).
 size_t lm_dyn_smem(int n_ant) {
     const int n2 = 2 * n_ant;
-    const size_t base = (size_t)n2 * (3 * sizeof(double) + 2 * sizeof(float) + sizeof(int)) + 16 + sizeof(float) * tile_floats(n2);
     const size_t n_bl = (size_t)n_ant * (n_ant - 1) / 2;
-    return n2 <= kSmallN2 ? base + 2 * sizeof(float) * (size_t)n2 * n2 + 4 * sizeof(double) * n_bl : base;
+    const size_t base = (size_t)n2 * (3 * sizeof(double) + 2 * sizeof(float) + sizeof(int)) + 16;
+    if (n2 <= kSmallN2) return base + sizeof(float) * (4 * 96 + (size_t)n2 * (n2 + 1)) + 4 * sizeof(double) * n_bl;
+    return base + sizeof(float) * tile_floats(n2);
 }
 
 // Launches the update of n_ctx contexts: clusters if any of them is large.
