@@ -256,8 +256,9 @@ psc_status psc_snapshot_components(int n_comp, const double *comp_in, double a, 
  * n_planes = 0 returns to its grid.  It checks on the GPU that the stack
  * covers the residual w of every baseline, time and channel of the context,
  * and refuses with PSC_ERR_ARG otherwise (the message gives both ranges).
- * Taps then read two planes each from global memory (the grid is never
- * staged).  Gaussian kernel model and FP32 grid only: this call refuses a
+ * A thread block stages the cells of the planes that its visibilities touch,
+ * or its taps read two planes each from global memory.
+ * Gaussian kernel model and FP32 grid only: this call refuses a
  * context with the exact kernel or the BF16 grid copy, psc_set_kernel_model
  * and psc_set_grid_precision refuse those while a stack is set.  A batch
  * takes either only stacked contexts (its persistent launch then runs the

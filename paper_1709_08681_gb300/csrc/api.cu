@@ -1538,7 +1538,7 @@ psc_status build_tables(psc_batch *b) {
         lm[k] = lm_args(c);
         st0[k] = c->d_state0;
         lm0[k] = c->d_lm0;
-        dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support));
+        dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support) + eval_stack_smem(c->wp_n));
         lmd = std::max(lmd, lm_smem_bytes(c->n_ant));
         max_ant = std::max(max_ant, c->n_ant);
         max_bpb = std::max(max_bpb, red[k].bpb);
@@ -1572,7 +1572,7 @@ psc_status build_tables(psc_batch *b) {
         PSC_BCUDA(b, set_track_smem(tdyn));
         PSC_BCUDA(b, track_occupancy(b->track, tdyn, &per_sm));
     } else {
-        PSC_BCUDA(b, set_eval_smem(dyn));
+        PSC_BCUDA(b, set_eval_smem(dyn - eval_stack_smem(b->ctxs[0]->wp_n)));
         PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, b->split, &per_sm));
     }
     PSC_BCUDA(b, cudaGetDevice(&dev));

@@ -67,7 +67,10 @@ struct BlockSharedT {
     float bl[4];
     int box[4];
     int taps;          // taps of the brick's visibilities (pi rho_max^2 each, rounded up)
+    int wp[2];         // residual-w stack: lowest and highest lower plane of the brick's visibilities
 };
+
+constexpr int kWCap = 3060;            // staged cells of all planes (24 KB: 4.85 ms in the case above; 32 KB 4.97, 40 KB 5.46, fewer blocks an SM)
 
 // The tap sums of a rectangle's visibilities with a.split lanes per visibility:
 // lane g takes rows g, g + split, ..., the row sums go through shared memory, and
@@ -165,12 +168,15 @@ __device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_ta
 // One brick: kv visibilities per thread.  acc receives the thread's 15 sums
 // (reduce mode); predict mode writes V and the derivative planes.
 // kW: the grid is a residual-w stack (EvalArgs::wp_n); every tap reads the two
-// planes around its visibility's w and interpolates, unstaged.
+// planes around its visibility's w and interpolates.  A brick's w changes slowly: the
+// block stages the box of every plane that its visibilities touch (s_wtile, up to
+// kWCap cells in all); bricks that need more read the planes tap by tap.  27 antennas, 600 x 64, 33 planes: 4.85 ms
+// against 5.83 with every tap unstaged.
 // kSplit: the rows of each visibility are shared among a.split lanes (split_taps);
 // the brick, its sums and their order are those of the rectangle without it.
 template <bool kPredict, int kV, bool kW, bool kSplit>
 __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 *s_tab, BlockSharedT<!kW> &sh,
-                                           float4 *s_split, float (&acc)[kRed]) {
+                                           float4 *s_split, float2 *s_wtile, float (&acc)[kRed]) {
     const int tid = threadIdx.x;
     // brick -> baseline, this thread's channel c and first time step t0, and
     // the block's channels [c_first, c_first + n_ch) (lc = c - c_first)
@@ -212,6 +218,7 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
         sh.bl[3] = (float)(mi - mj);
         sh.box[0] = INT_MAX; sh.box[1] = INT_MIN; sh.box[2] = INT_MAX; sh.box[3] = INT_MIN;
         sh.taps = 0;
+        sh.wp[0] = INT_MAX; sh.wp[1] = INT_MIN;
     }
     __syncthreads();
     const float L = sh.bl[0], M = sh.bl[1], dL = sh.bl[2], dM = sh.bl[3];
@@ -223,7 +230,7 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
     int ix0[kV], iy0[kV];
     float hx[kV], hy[kV];
     float rmax = 0.f;
-    size_t woff[kV];                                  // kW: first cell of the lower plane
+    int wpl[kV];                                      // kW: the lower plane
     float wf[kV];                                     // kW: weight of the upper plane
     if (active) {
         const ChanConst ch = a.chan[c];
@@ -254,7 +261,7 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
                 double q = (p[2] - a.wp_a * p[0] - a.wp_b * p[1]) * ch.uv_scale * a.wp_scale - a.wp_q0;
                 q = fmin(fmax(q, 0.0), (double)(a.wp_n - 1));
                 const int pl = min((int)floor(q), a.wp_n - 2);
-                woff[v] = (size_t)pl * a.ng * a.ng;
+                wpl[v] = pl;
                 wf[v] = (float)(q - (double)pl);
             }
             ix0[v] = nx - S / 2 + 1;
@@ -272,6 +279,13 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
             atomicMin(&sh.box[2], loy); atomicMax(&sh.box[3], hiy);
             const int nv = min(kV, a.nt - t0);
             atomicAdd(&sh.taps, nv * (int)ceilf(3.14159265f * rmax * rmax));
+            if constexpr (kW) {
+#pragma unroll
+                for (int v = 0; v < kV; ++v) {
+                    atomicMin(&sh.wp[0], wpl[v]);
+                    atomicMax(&sh.wp[1], wpl[v]);
+                }
+            }
         }
     }
     // radial tables of this block's channels as (c_n, s_n), zero-padded
@@ -296,7 +310,10 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
     // a global load, two complex products and a store (about four unstaged
     // taps' extra work), so stage only boxes of at most taps / 4 cells that
     // fit the tile.  Uniform over the block.
-    const bool staged = !kW && !a.no_stage && ex <= kTile && ey <= kTile && 4 * ex * ey <= sh.taps;
+    const int n_pl = kW && !empty ? sh.wp[1] - sh.wp[0] + 2 : 1;        // planes that the brick touches
+    const bool staged = kW ? !a.no_stage && !empty && ex <= kTile && ey <= kTile && n_pl <= kWCap / (ex * ey) &&
+                                 2 * n_pl * ex * ey <= sh.taps
+                           : !a.no_stage && ex <= kTile && ey <= kTile && 4 * ex * ey <= sh.taps;
 
     // per-cell half of the ramp, exp(-i pi du (k_x L + k_y M)) = phx[k_x] phy[k_y],
     // with (k_x, k_y) relative to the tile origin (staged) or to each
@@ -340,7 +357,77 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
     float2 S0[kV], Su[kV], Sv[kV];
 #pragma unroll
     for (int v = 0; v < kV; ++v) S0[v] = Su[v] = Sv[v] = make_float2(0.f, 0.f);
-    if constexpr (kSplit) {
+    if (kW && staged) {
+        const int p0 = sh.wp[0], cells = ex * ey;
+        for (int k = tid; k < cells; k += blockDim.x) {
+            const int yy = k / ex, xx = k - yy * ex;
+            const int gx = bx0 + xx, gy = by0 + yy;
+            const bool in = gx >= 0 && gx < a.ng && gy >= 0 && gy < a.ng;
+            const float2 z = cmul(sh.phx[xx], sh.phy[yy]);
+            const float2 *src = a.grid + (size_t)p0 * a.ng * a.ng + (in ? (size_t)gy * a.ng + gx : 0);
+#pragma unroll 4
+            for (int p = 0; p < n_pl; ++p, src += (size_t)a.ng * a.ng)
+                s_wtile[p * cells + k] = in ? cmul(__ldg(src), z) : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        if (active) {
+            const unsigned tab_adj = (unsigned)__cvta_generic_to_shared(s_tab + lc * tab_stride) - (0x4B000000u << 3);
+            const float ov = (float)a.ov;
+            const float rmax2 = rmax * rmax;
+            int wx[kV], wy[kV];
+            int r_lo = INT_MAX, r_hi = INT_MIN;
+#pragma unroll
+            for (int v = 0; v < kV; ++v) {
+                wx[v] = ix0[v] - bx0;
+                wy[v] = iy0[v] - by0;
+                r_lo = min(r_lo, wy[v] + max(0, (int)floorf(hy[v] - rmax) + 1));
+                r_hi = max(r_hi, wy[v] + min(S - 1, (int)ceilf(hy[v] + rmax) - 1));
+            }
+            for (int cy = r_lo; cy <= r_hi; ++cy) {
+                float dy[kV], dyo2[kV];
+                int c_lo = INT_MAX, c_hi = INT_MIN;
+#pragma unroll
+                for (int v = 0; v < kV; ++v) {
+                    dy[v] = hy[v] - (float)(cy - wy[v]);
+                    const float dyo = dy[v] * ov;
+                    dyo2[v] = fmaf(dyo, dyo, 1e-20f);
+                    const float rem = rmax2 - dy[v] * dy[v];
+                    if (rem > 0.f) {
+                        const float r = fminf(rem * rsqrt_fast(rem), rmax);
+                        const int a_lo = max(0, (int)floorf(hx[v] - r) + 1);
+                        const int a_hi = min(S - 1, (int)ceilf(hx[v] + r) - 1);
+                        if (a_lo <= a_hi) {
+                            c_lo = min(c_lo, wx[v] + a_lo);
+                            c_hi = max(c_hi, wx[v] + a_hi);
+                        }
+                    }
+                }
+                if (c_lo > c_hi) continue;
+                float dxo[kV], pr[kV], pi[kV], qr[kV], qi[kV];
+#pragma unroll
+                for (int v = 0; v < kV; ++v) {
+                    dxo[v] = (hx[v] - (float)(c_lo - wx[v])) * ov;
+                    pr[v] = pi[v] = qr[v] = qi[v] = 0.f;
+                }
+                const float2 *lo[kV];
+#pragma unroll
+                for (int v = 0; v < kV; ++v) lo[v] = s_wtile + (wpl[v] - p0) * cells + cy * ex + c_lo;
+                row_taps_w<kV>(lo, cells, c_hi - c_lo + 1, dxo, dyo2, wf, ov, tab_adj, pr, pi, qr, qi);
+#pragma unroll
+                for (int v = 0; v < kV; ++v) {
+                    S0[v].x += pr[v]; S0[v].y += pi[v];
+                    Su[v].x += qr[v]; Su[v].y += qi[v];
+                    Sv[v].x = fmaf(dy[v], pr[v], Sv[v].x);
+                    Sv[v].y = fmaf(dy[v], pi[v], Sv[v].y);
+                }
+            }
+        }
+        const float inv_ov = 1.0f / (float)a.ov;
+#pragma unroll
+        for (int v = 0; v < kV; ++v) {                       // Q was accumulated with dx * ov
+            Su[v].x *= inv_ov; Su[v].y *= inv_ov;
+        }
+    } else if constexpr (kSplit) {
         // each rectangle slot's window, then its sums in the same place
         if (active) s_split[tid] = make_float4(__int_as_float(ix0[0]), __int_as_float(iy0[0]), hx[0], hy[0]);
         __syncthreads();
@@ -414,6 +501,7 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
             // comes from phx / phy; rows and columns are clipped to the grid
 #pragma unroll
             for (int v = 0; v < kV; ++v) {
+                const float2 *lo = kW ? a.grid + (size_t)wpl[v] * a.ng * a.ng : a.grid, *hi = lo + (size_t)a.ng * a.ng;    // kW: the two planes
                 const int b_lo = max(max(0, (int)floorf(hy[v] - rmax) + 1), -iy0[v]);
                 const int b_hi = min(min(S - 1, (int)ceilf(hy[v] + rmax) - 1), a.ng - 1 - iy0[v]);
                 for (int b = b_lo; b <= b_hi; ++b) {
@@ -431,8 +519,8 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
                     for (int aa = a_lo; aa <= a_hi; ++aa, dd -= ov) {
                         float2 gc;
                         if constexpr (kW) {
-                            const float2 g0 = __ldg(&a.grid[woff[v] + row + aa]);
-                            const float2 g1 = __ldg(&a.grid[woff[v] + (size_t)a.ng * a.ng + row + aa]);
+                            const float2 g0 = __ldg(&lo[row + aa]);
+                            const float2 g1 = __ldg(&hi[row + aa]);
                             gc = make_float2(fmaf(wf[v], g1.x - g0.x, g0.x), fmaf(wf[v], g1.y - g0.y, g0.y));
                         } else {
                             gc = grid_cell(a, row + aa);
@@ -535,15 +623,13 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
 // brick numbers from an atomic queue until all sum(bricks) are taken; prefix
 // holds the first global brick of each context).  Every brick writes its own
 // partial record, so the result does not depend on which block ran it.
-// The stacked instantiation (kW) asks for 4 blocks of kMaxThreads per SM,
-// i.e. at most 64 registers (some spill): its unstaged two-plane taps gain
-// more from the warps than they lose (vla27_l64ch as one interval: 5.56 ms
-// against 6.36 ms at 99 registers).  A minimum of 0 leaves the co-planar
-// instantiations with the plain bound.
+// The stacked instantiation (kW) asks for 3 blocks of kMaxThreads per SM, i.e. at
+// most 85 registers; a minimum of 0 leaves the co-planar instantiations with the
+// plain bound.
 // kSplit: the instantiation that also runs split items (its co-planar contexts
 // without them take the same code as before, at this kernel's registers).
 template <bool kPredict, bool kW, bool kSplit>
-__global__ void __launch_bounds__(kMaxThreads, kW ? 4 : kSplit ? 3 : 0) eval_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args,
+__global__ void __launch_bounds__(kMaxThreads, kW || kSplit ? 3 : 0) eval_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args,
                                                            const long long *__restrict__ prefix, int n_ctx,
                                                            unsigned long long *queue) {
     extern __shared__ __align__(16) float2 s_tab[];   // c_group * tab_stride, then split_taps' arrays (16-byte aligned)
@@ -594,9 +680,11 @@ __global__ void __launch_bounds__(kMaxThreads, kW ? 4 : kSplit ? 3 : 0) eval_ker
 #pragma unroll
     for (int k = 0; k < kRed; ++k) acc[k] = 0.f;
     float4 *s_split = reinterpret_cast<float4 *>(s_tab + (a.c_group * a.tab_stride + 1) / 2 * 2);
-    if (kSplit && a.split > 1) eval_brick<kPredict, 1, kW, kSplit>(a, brick, s_tab, sh, s_split, acc);
-    else if (a.kv == 2) eval_brick<kPredict, 2, kW, false>(a, brick, s_tab, sh, nullptr, acc);
-    else eval_brick<kPredict, 1, kW, false>(a, brick, s_tab, sh, nullptr, acc);
+    // the stack's tile starts after the tables, whatever their number (a multiple of 16 bytes)
+    float2 *s_wtile = s_tab + ((a.flat > 0 ? a.ch_span : a.c_group) * a.tab_stride + 1) / 2 * 2;
+    if (kSplit && a.split > 1) eval_brick<kPredict, 1, kW, kSplit>(a, brick, s_tab, sh, s_split, nullptr, acc);
+    else if (a.kv == 2) eval_brick<kPredict, 2, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc);
+    else eval_brick<kPredict, 1, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc);
     if constexpr (!kPredict) {
         // ---- block reduction: a butterfly within each warp -- compensated
         // (Knuth's TwoSum, the rounding errors summed beside) for chi^2 and the
@@ -813,11 +901,14 @@ size_t eval_split_smem(int split, int support) {
     return split > 1 ? 16 + sizeof(float4) * (kMaxThreads + kMaxThreads * 6 / 4 + (size_t)(kMaxThreads / split) * support) : 0;
 }
 
+// The staged planes' share (and its alignment).
+size_t eval_stack_smem(int wp_n) { return wp_n > 0 ? 16 + sizeof(float2) * kWCap : 0; }
+
 cudaError_t launch_eval(const EvalArgs &a, bool predict, cudaStream_t s) {
     if (a.exact) return launch_exact(a, predict, s);
     const int threads = a.split > 1 ? kMaxThreads : ((a.flat > 0 ? a.flat : a.t_tile * a.c_group) + 31) / 32 * 32;
     const int blocks = (int)a.n_bricks;
-    const size_t dyn = eval_dyn_smem(a.flat > 0 ? a.ch_span : a.c_group, a.tab_stride) + eval_split_smem(a.split, a.support);
+    const size_t dyn = eval_dyn_smem(a.flat > 0 ? a.ch_span : a.c_group, a.tab_stride) + eval_split_smem(a.split, a.support) + eval_stack_smem(a.wp_n);
     if (a.wp_n > 0) {
         if (predict) eval_kernel<true, true, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
         else eval_kernel<false, true, false><<<blocks, threads, dyn, s>>>(a, nullptr, nullptr, 0, nullptr);
@@ -874,10 +965,18 @@ cudaError_t set_eval_smem(size_t dyn) {
     cudaError_t e = eval_smem_allowed(&allowed);
     if (e != cudaSuccess) return e;
     if (dyn > allowed) return cudaErrorInvalidValue;
+    int dev = 0, optin = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
     for (const void *k : {(const void *)eval_kernel<true, false, false>, (const void *)eval_kernel<false, false, false>,
                           (const void *)eval_kernel<true, true, false>, (const void *)eval_kernel<false, true, false>,
                           (const void *)eval_kernel<true, false, true>, (const void *)eval_kernel<false, false, true>}) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)allowed);
+        // the stacked kernels hold a smaller static part, and more dynamic memory (eval_stack_smem)
+        cudaFuncAttributes fa{};
+        e = cudaFuncGetAttributes(&fa, k);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

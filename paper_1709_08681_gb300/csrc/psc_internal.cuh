@@ -64,7 +64,7 @@ struct EvalArgs {
     // Residual-w stack (wp_n >= 2): grid holds wp_n planes of ng^2 cells.  A
     // visibility at q = (w - wp_a u - wp_b v) uv_scale wp_scale - wp_q0 (uvw in
     // metres, q clamped to [0, wp_n - 1]) reads (1 - f) plane p + f plane p + 1,
-    // p = min(floor(q), wp_n - 2), f = q - p.  Taps read the planes unstaged.
+    // p = min(floor(q), wp_n - 2), f = q - p.
     int wp_n;
     double wp_a, wp_b, wp_scale, wp_q0;
     // Track kernel (track.cu; trk_kv > 0, reduce mode only): one warp per item
@@ -218,6 +218,7 @@ size_t exact_dyn_smem(int c_group, int tab_stride);
 cudaError_t launch_exact_moments(double diam_m, const double *freq_dev, int nc, double du, int ov,
                                  const int *tab_off_dev, const int *tab_len_dev, float *kmom, cudaStream_t s);
 size_t eval_split_smem(int split, int support);
+size_t eval_stack_smem(int wp_n);
 // Dynamic shared memory of one fused-kernel block (c_group zero-padded tables).
 size_t eval_dyn_smem(int c_group, int tab_stride);
 // Largest distance (metres, u-v plane) between the baselines of consecutive

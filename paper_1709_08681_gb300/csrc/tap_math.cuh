@@ -148,5 +148,29 @@ __device__ __forceinline__ void row_taps(const float2 *__restrict__ row, int n, 
     }
 }
 
+// row_taps on staged w-planes: visibility v's cells start at lo[v] in its lower plane
+// and `next` cells further in the upper one, whose weight is wf[v].
+template <int kV>
+__device__ __forceinline__ void row_taps_w(const float2 *const (&lo)[kV], int next, int n, float (&dxo)[kV],
+                                           const float (&dyo2)[kV], const float (&wf)[kV], float ov, unsigned tab_adj,
+                                           float (&pr)[kV], float (&pi)[kV], float (&qr)[kV], float (&qi)[kV]) {
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+#pragma unroll
+        for (int v = 0; v < kV; ++v) {
+            const float2 g0 = lo[v][k], g1 = lo[v][next + k];
+            const float2 g = ffma2(make_float2(wf[v], wf[v]), g1, ffma2(make_float2(-wf[v], -wf[v]), g0, g0));
+            const float s2 = fmaf(dxo[v], dxo[v], dyo2[v]);
+            const float t = sqrt_fast(s2);
+            const float tf = __fadd_rz(t, 8388608.0f);          // floor(t) + 2^23
+            const float2 e = lds_f2(tab_adj + ((unsigned)__float_as_int(tf) << 3));
+            const float A = fmaf(t, e.y, e.x);
+            fma2_acc(pr[v], pi[v], A, g.x, g.y);
+            fma2_acc(qr[v], qi[v], A * dxo[v], g.x, g.y);
+            dxo[v] -= ov;
+        }
+    }
+}
+
 }  // namespace tap
 }  // namespace psc
