@@ -96,28 +96,40 @@ __device__ __forceinline__ float2 fadd2_rz(float2 a, float2 b) {
     return d;
 }
 
-// The row loop for two visibilities with their per-visibility scalars
-// packed in pairs: s2, floor(t) + 2^23, A dxo and the dxo step are one packed
-// instruction for both.
-__device__ __forceinline__ void row_taps2(const float2 *__restrict__ row, int n, float2 dxo, float2 dyo2, float ov,
-                                          unsigned tab_adj, float (&pr)[2], float (&pi)[2], float (&qr)[2],
-                                          float (&qi)[2]) {
+// Two neighbouring rows of taps for two visibilities, n cells from row_a and row_b,
+// the visibilities' scalars packed in pairs (s2, floor(t) + 2^23, A dxo and the dxo step
+// are one packed instruction for both): the same column offsets for both rows, twice
+// the independent work per step of the sqrt -> table -> FMA chain that one row at a
+// time waited for.  Returns each row's P = sum A G' (pa, pb) and both rows'
+// Q = sum A dxo G'.
+__device__ __forceinline__ void row_pair_taps2(const float2 *__restrict__ row_a, const float2 *__restrict__ row_b, int n,
+                                               float2 dxo, float2 dyo2a, float2 dyo2b, float ov, unsigned tab_adj,
+                                               float2 (&pa)[2], float2 (&pb)[2], float2 (&q)[2]) {
     const float2 step = make_float2(-ov, -ov);
     const float2 magic = make_float2(8388608.0f, 8388608.0f);
+    pa[0] = pa[1] = pb[0] = pb[1] = q[0] = q[1] = make_float2(0.f, 0.f);
 #pragma unroll 2
     for (int k = 0; k < n; ++k) {
-        const float2 g = row[k];
-        const float2 s2 = ffma2(dxo, dxo, dyo2);
-        const float2 t = make_float2(sqrt_fast(s2.x), sqrt_fast(s2.y));
-        const float2 tf = fadd2_rz(t, magic);                       // floor(t) + 2^23, both
-        const float2 e0 = lds_f2(tab_adj + ((unsigned)__float_as_int(tf.x) << 3));
-        const float2 e1 = lds_f2(tab_adj + ((unsigned)__float_as_int(tf.y) << 3));
-        const float2 A = make_float2(fmaf(t.x, e0.y, e0.x), fmaf(t.y, e1.y, e1.x));
-        const float2 Ad = fmul2(A, dxo);
-        fma2_acc(pr[0], pi[0], A.x, g.x, g.y);
-        fma2_acc(pr[1], pi[1], A.y, g.x, g.y);
-        fma2_acc(qr[0], qi[0], Ad.x, g.x, g.y);
-        fma2_acc(qr[1], qi[1], Ad.y, g.x, g.y);
+        const float2 ga = row_a[k], gb = row_b[k];
+        const float2 sa = ffma2(dxo, dxo, dyo2a), sb = ffma2(dxo, dxo, dyo2b);
+        const float2 ta = make_float2(sqrt_fast(sa.x), sqrt_fast(sa.y));
+        const float2 tb = make_float2(sqrt_fast(sb.x), sqrt_fast(sb.y));
+        const float2 fa = fadd2_rz(ta, magic), fb = fadd2_rz(tb, magic);
+        const float2 ea0 = lds_f2(tab_adj + ((unsigned)__float_as_int(fa.x) << 3));
+        const float2 ea1 = lds_f2(tab_adj + ((unsigned)__float_as_int(fa.y) << 3));
+        const float2 eb0 = lds_f2(tab_adj + ((unsigned)__float_as_int(fb.x) << 3));
+        const float2 eb1 = lds_f2(tab_adj + ((unsigned)__float_as_int(fb.y) << 3));
+        const float2 Aa = make_float2(fmaf(ta.x, ea0.y, ea0.x), fmaf(ta.y, ea1.y, ea1.x));
+        const float2 Ab = make_float2(fmaf(tb.x, eb0.y, eb0.x), fmaf(tb.y, eb1.y, eb1.x));
+        const float2 Ada = fmul2(Aa, dxo), Adb = fmul2(Ab, dxo);
+        fma2_acc(pa[0].x, pa[0].y, Aa.x, ga.x, ga.y);
+        fma2_acc(pa[1].x, pa[1].y, Aa.y, ga.x, ga.y);
+        fma2_acc(pb[0].x, pb[0].y, Ab.x, gb.x, gb.y);
+        fma2_acc(pb[1].x, pb[1].y, Ab.y, gb.x, gb.y);
+        fma2_acc(q[0].x, q[0].y, Ada.x, ga.x, ga.y);
+        fma2_acc(q[1].x, q[1].y, Ada.y, ga.x, ga.y);
+        fma2_acc(q[0].x, q[0].y, Adb.x, gb.x, gb.y);
+        fma2_acc(q[1].x, q[1].y, Adb.y, gb.x, gb.y);
         dxo = fadd2(dxo, step);
     }
 }
@@ -142,8 +154,8 @@ __device__ __forceinline__ void row_taps(const float2 *__restrict__ row, int n, 
             const float2 e = lds_f2(tab_adj + ((unsigned)__float_as_int(tf) << 3));
             const float A = fmaf(t, e.y, e.x);
             fma2_acc(pr[v], pi[v], A, g.x, g.y);
-            fma2_acc(qr[v], qi[v], A * dxo[v], g.x, g.y);
-            dxo[v] -= ov;
+            fma2_acc(qr[v], qi[v], __fmul_rn(A, dxo[v]), g.x, g.y);
+            dxo[v] = __fsub_rn(dxo[v], ov);
         }
     }
 }
