@@ -148,13 +148,15 @@ __global__ void __launch_bounds__(256) dft_cols_kernel(const float2 *__restrict_
 //   pass 2: G[gy][gx]^T tile: rows gx, columns gy, sum over r of T[r][gx] E[gy][r]
 // with E[g][c] = W((g - Ng/2)(c - N/2)).  Pass 1 writes T already split and
 // transposed (planes [3][Ng][N]) so that both passes read K-major operands.
-// A block owns a 128 x 64 tile with FP32 accumulators in tensor memory; K
-// advances in chunks of 32 through shared-memory buffers of all operand
-// planes.  One thread runs the pipeline over three shared-memory buffers: it
-// loads chunks two ahead with TMA (cp.async.bulk.tensor, one copy per source
-// and 8-wide K column: the box 8 x rows x 3 planes lands as [plane][row][8
-// elements], i.e. the no-swizzle K-major core-matrix layout, K columns
-// 3 * rows * 16 bytes apart), waits for a chunk's copies on its buffer's load
+// A block owns a 128 x 64 (pass 1) or 128 x 128 tile (pass 2: its four accumulators
+// then fill the tensor memory; with 64 columns each MMA's operand reads outweighed its
+// work) with FP32 accumulators in tensor memory; K advances in chunks of 32 through
+// shared-memory buffers of all operand planes.  One thread runs the pipeline over three (two) shared-memory buffers: it
+// loads chunks two (one) ahead with TMA (cp.async.bulk.tensor, one copy per source:
+// the box 32 x rows x 3 planes lands as [plane][row][32 elements] in the 64-byte
+// swizzle; boxes of one 16-byte K column, in no swizzle, left the copy engine with
+// four times the row requests, which bound the kernel: pass 2 of 2000 components on
+// 2048^2 took 345 us, 429 us with 64 columns, and takes 221 us), waits for a chunk's copies on its buffer's load
 // mbarrier, issues the MMAs (kind::f16, the negative term of the complex
 // product by the descriptor's negate-A bit), commits them to the buffer's MMA
 // mbarrier, and refills the previous chunk's buffer once those MMAs are done.
@@ -162,13 +164,15 @@ __global__ void __launch_bounds__(256) dft_cols_kernel(const float2 *__restrict_
 // with zeros to a multiple of the chunk.  Every wait is bounded (*err).
 
 typedef __nv_bfloat16 bf16;
-constexpr int kTM = 128, kTN = 64, kTK = 32;
-constexpr int kColA = 3 * kTM * 16;                 // one 8-wide K column of an A source, 3 planes (6 KB)
-constexpr int kColB = 3 * kTN * 16;                 // the same of a B source (3 KB)
-constexpr int kSrcA = kTK / 8 * kColA;              // an A source's share of a chunk (24 KB)
-constexpr int kSrcB = kTK / 8 * kColB;              // a B source's share (12 KB)
+constexpr int kTM = 128, kTK = 32;
+// Tile columns, threads (a warpgroup per 64 columns) and buffers of a pass.
+__host__ __device__ constexpr int tc_cols(int pass) { return pass == 1 ? 64 : 128; }
+__host__ __device__ constexpr int tc_threads(int pass) { return pass == 1 ? 128 : 256; }
+__host__ __device__ constexpr int tc_stages(int pass) { return pass == 1 ? 3 : 2; }
+constexpr int kRow = kTK * 2;                       // bytes of a row of a chunk: the swizzle's width
+constexpr int kSrcA = 3 * kTM * kRow;               // an A source's share of a chunk, 3 planes (24 KB)
+__host__ __device__ constexpr int tc_src_b(int pass) { return 3 * tc_cols(pass) * kRow; }         // a B source's share
 constexpr int kEpoch = 4;                            // chunks (K = 128) between promotions to registers
-constexpr int kStages = 3;                           // shared-memory buffers of the TMA pipeline
 constexpr long kTcWait = 1L << 24;
 
 __device__ __forceinline__ void split3(float x, bf16 &h, bf16 &m, bf16 &l) {
@@ -354,10 +358,11 @@ __global__ void comp_edge_kernel(const bf16 *__restrict__ Ar, const bf16 *__rest
     if (lane == 0) G[(size_t)gy * ng + gx] = make_float2(re, im);
 }
 
-__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t k_stride) {
-    // K-major, no swizzle: K-adjacent core matrices k_stride bytes apart, 8-row groups 128 B apart
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((k_stride >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)(128 >> 4) << 32) | ((uint64_t)1 << 46);
+__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
+    // K-major, 64-byte swizzle (layout 4): 8-row groups 8 kRow bytes apart; a K step
+    // of 16 elements within the row moves the start address alone
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(8 * kRow >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
 // TMA load of one box of a 3-D tensor map into shared memory, completing on mbar.
@@ -406,11 +411,13 @@ struct TcPassArgs {
 };
 
 template <int kPass>
-__global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, const __grid_constant__ CUtensorMap mA0,
+__global__ void __launch_bounds__(tc_threads(kPass), 1) dft_tc_kernel(const TcPassArgs g, const __grid_constant__ CUtensorMap mA0,
                                                         const __grid_constant__ CUtensorMap mA1,
                                                         const __grid_constant__ CUtensorMap mB0,
                                                         const __grid_constant__ CUtensorMap mB1) {
     constexpr int kNA = kPass == 1 ? 1 : 2;
+    constexpr int kTN = tc_cols(kPass), kStages = tc_stages(kPass), kSrcB = tc_src_b(kPass);
+    constexpr int kHalf = 64;                                  // columns of one warpgroup
     constexpr int kStage = kNA * kSrcA + 2 * kSrcB;           // A sources, then B sources (E re, E im)
     constexpr uint32_t kBytes = (uint32_t)kStage;              // TMA bytes of one chunk (zero fill included)
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -455,11 +462,12 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
                            ((uint32_t)(kTM >> 4) << 24);
     const uint32_t idesc_neg = idesc | (1u << 13);  // negate A
     const int nk = (g.k + kTK - 1) / kTK;
-    const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem);
-    const uint32_t lane_base = tmem + ((uint32_t)(32 * warp) << 16);
-    float sum_re[kTN], sum_im[kTN];
+    const uint32_t smem_base = ((uint32_t)__cvta_generic_to_shared(smem) + 1023u) & ~1023u;   // the swizzle's pattern starts there
+    const int col_base = (warp >> 2) * kHalf;                  // the warp's columns; its rows: 32 (warp & 3) ..
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col_base;
+    float sum_re[kHalf], sum_im[kHalf];
 #pragma unroll
-    for (int j = 0; j < kTN; ++j) { sum_re[j] = 0.f; sum_im[j] = 0.f; }
+    for (int j = 0; j < kHalf; ++j) { sum_re[j] = 0.f; sum_im[j] = 0.f; }
     bool ok = true;
     bool started[4] = {false, false, false, false};  // used by thread 0 only
     // Only thread 0 waits on the buffers' barriers (in chunk order, so never
@@ -476,12 +484,8 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
         const uint32_t sb = smem_base + (uint32_t)(bb * kStage);
         mbar_expect(lb[bb], kBytes);
         const int k0 = ch * kTK;
-        for (int j = 0; j < kTK / 8; ++j) {
-            for (int s_ = 0; s_ < kNA; ++s_)
-                tma_load3(sb + (uint32_t)(s_ * kSrcA + j * kColA), mapA[s_], k0 + 8 * j, m0, 0, lb[bb]);
-            for (int s_ = 0; s_ < 2; ++s_)
-                tma_load3(sb + (uint32_t)(kNA * kSrcA + s_ * kSrcB + j * kColB), mapB[s_], k0 + 8 * j, n0, 0, lb[bb]);
-        }
+        for (int s_ = 0; s_ < kNA; ++s_) tma_load3(sb + (uint32_t)(s_ * kSrcA), mapA[s_], k0, m0, 0, lb[bb]);
+        for (int s_ = 0; s_ < 2; ++s_) tma_load3(sb + (uint32_t)(kNA * kSrcA + s_ * kSrcB), mapB[s_], k0, n0, 0, lb[bb]);
         loads = ch + 1;
     };
     if (tid == 0)
@@ -506,15 +510,13 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
                 for (int t = 0; t < kTerms; ++t) {
                     const int acc = terms[t][0], sa = terms[t][1], sbs = terms[t][2], neg = terms[t][3];
                     for (int q = 0; q < 6; ++q) {
-                        // plane p of source s: K column j at + j * kCol, plane p at + p * rows * 16
-                        const uint32_t a_pl = sb + (uint32_t)(sa * kSrcA + pp[q][0] * kTM * 16);
-                        const uint32_t b_pl = sb + (uint32_t)(kNA * kSrcA + sbs * kSrcB + pp[q][1] * kTN * 16);
+                        const uint32_t a_pl = sb + (uint32_t)(sa * kSrcA + pp[q][0] * kTM * kRow);
+                        const uint32_t b_pl = sb + (uint32_t)(kNA * kSrcA + sbs * kSrcB + pp[q][1] * kTN * kRow);
                         const int dst = acc + (q == 0 ? 0 : 2);
 #pragma unroll
                         for (int kk = 0; kk < kTK / 16; ++kk) {
-                            tc_mma(tmem + (uint32_t)(dst * kTN), tc_desc(a_pl + (uint32_t)(2 * kk * kColA), kColA),
-                                   tc_desc(b_pl + (uint32_t)(2 * kk * kColB), kColB), neg ? idesc_neg : idesc,
-                                   started[dst] ? 1u : 0u);
+                            tc_mma(tmem + (uint32_t)(dst * kTN), tc_desc(a_pl + 32u * kk), tc_desc(b_pl + 32u * kk),
+                                   neg ? idesc_neg : idesc, started[dst] ? 1u : 0u);
                             started[dst] = true;
                         }
                     }
@@ -540,7 +542,7 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-            for (int c0 = 0; c0 < kTN; c0 += 16) {
+            for (int c0 = 0; c0 < kHalf; c0 += 16) {
                 uint32_t re[16], im[16], rs[16], is[16];
                 tc_ld16(lane_base + (uint32_t)c0, re);
                 tc_ld16(lane_base + (uint32_t)(kTN + c0), im);
@@ -570,11 +572,11 @@ __global__ void __launch_bounds__(128, 1) dft_tc_kernel(const TcPassArgs g, cons
         }
     }
     if (ok) {
-        const int m = m0 + 32 * warp + lane;         // accumulator lane: pass 1 image row, pass 2 grid column gx
+        const int m = m0 + 32 * (warp & 3) + lane;   // accumulator lane: pass 1 image row, pass 2 grid column gx
         if (m < g.a_rows) {
 #pragma unroll
-            for (int j = 0; j < kTN; ++j) {
-                const int col = n0 + j;                      // pass 1: grid column g; pass 2: grid row gy
+            for (int j = 0; j < kHalf; ++j) {
+                const int col = n0 + col_base + j;                      // pass 1: grid column g; pass 2: grid row gy
                 if (col >= g.b_rows) break;
                 if constexpr (kPass == 1) {
                     const size_t plane_t = (size_t)g.b_rows * g.k;
@@ -626,8 +628,8 @@ cudaError_t encode_fn(EncodeTiled *out) {
 }
 
 // Tensor map of split bfloat16 planes [3][rows][k] (k % 8 == 0, 16-byte aligned
-// base): dimensions (k, rows, 3), box 8 x box_rows x 3 (one 8-wide K column of a
-// tile, all planes), zero fill outside.
+// base): dimensions (k, rows, 3), box kTK x box_rows x 3 (a chunk of a tile, all
+// planes) in the 64-byte swizzle, zero fill outside.
 cudaError_t plane_map(CUtensorMap *m, const bf16 *base, int rows, int k, int box_rows) {
     if (k % 8 || ((uintptr_t)base & 15)) return cudaErrorInvalidValue;
     EncodeTiled fn = nullptr;
@@ -635,10 +637,10 @@ cudaError_t plane_map(CUtensorMap *m, const bf16 *base, int rows, int k, int box
     if (e != cudaSuccess) return e;
     const cuuint64_t dims[3] = {(cuuint64_t)k, (cuuint64_t)rows, 3};
     const cuuint64_t strides[2] = {(cuuint64_t)k * 2, (cuuint64_t)rows * (cuuint64_t)k * 2};
-    const cuuint32_t box[3] = {8, (cuuint32_t)box_rows, 3};
+    const cuuint32_t box[3] = {kTK, (cuuint32_t)box_rows, 3};
     const cuuint32_t es[3] = {1, 1, 1};
     const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16 *>(base), dims, strides, box, es,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -648,7 +650,8 @@ cudaError_t plane_map(CUtensorMap *m, const bf16 *base, int rows, int k, int box
 template <int kPass>
 cudaError_t launch_tc_pass(const TcPassArgs &a, cudaStream_t s) {
     constexpr int kNA = kPass == 1 ? 1 : 2;
-    const int smem = kStages * (kNA * kSrcA + 2 * kSrcB);
+    constexpr int kTN = tc_cols(kPass);
+    const int smem = tc_stages(kPass) * (kNA * kSrcA + 2 * tc_src_b(kPass)) + 1024;    // + alignment
     CUtensorMap mA[2], mB[2];
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < kNA && e == cudaSuccess; ++i) e = plane_map(&mA[i], a.A[i], a.a_rows, a.k, kTM);
@@ -658,7 +661,7 @@ cudaError_t launch_tc_pass(const TcPassArgs &a, cudaStream_t s) {
     e = cudaFuncSetAttribute(dft_tc_kernel<kPass>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.b_rows + kTN - 1) / kTN, (a.a_rows + kTM - 1) / kTM);
-    dft_tc_kernel<kPass><<<grid, 128, smem, s>>>(a, mA[0], mA[1], mB[0], mB[1]);
+    dft_tc_kernel<kPass><<<grid, tc_threads(kPass), smem, s>>>(a, mA[0], mA[1], mB[0], mB[1]);
     return cudaGetLastError();
 }
 }  // namespace
