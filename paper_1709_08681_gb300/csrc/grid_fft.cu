@@ -4,7 +4,7 @@
 // Ng x Ng, as grid_dft.cu states it.
 //
 // Two passes, no workspace but the twiddle tables (of the powers of two: one
-// constant table a device, filled once):
+// constant table a context, filled once):
 //   columns: the image is real, so columns c and c + 1 go through one complex
 //     transform of length Ng (z = I_c + i I_{c+1}), of which the rows k = 0 ..
 //     Ng/2 are kept (U[k][c]; the others are their conjugates);
@@ -30,6 +30,8 @@
 // (grid_dft.cu, which grids of a long odd part still take), and its error
 // against 64 bits is 0.9-1.6e-7 (relative L2, 128^2 to 8192^2 grids) against
 // 1.5-4.1e-7.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cstdint>
 #include <mutex>
@@ -338,25 +340,46 @@ size_t model_grid_fft_ws_bytes(int n_grid) {
     return p.odd == 1 ? 0 : sizeof(float2) * (size_t)p.tw_len;
 }
 
+int context_slot() {
+    using CtxGetId = CUresult (*)(CUcontext, unsigned long long *);
+    static std::mutex mu;
+    static CtxGetId get_id = nullptr;
+    static unsigned long long ids[kCtxSlots];
+    static int n = 0;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!get_id) {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess || !p)
+            return -1;
+        get_id = reinterpret_cast<CtxGetId>(p);
+    }
+    unsigned long long id = 0;
+    if (cudaFree(nullptr) != cudaSuccess || get_id(nullptr, &id) != CUDA_SUCCESS) return -1;    // cudaFree: a current context
+    for (int i = 0; i < n; ++i)
+        if (ids[i] == id) return i;
+    if (n == kCtxSlots) return -1;
+    ids[n] = id;
+    return n++;
+}
+
 namespace {
 // Twiddle tables of every power of two: size n's at [n, 2n).  Allocating and
 // building the table on each call cost 140 us of the 490 us that 2048^2 ->
-// 8192^2 took; constants for the process's life cost 256 KB.
-constexpr int kMaxLog = 14, kMaxDevices = 64;
+// 8192^2 took; constants for the context's life cost 256 KB.
+constexpr int kMaxLog = 14;
 __device__ float2 g_pow2_tw[2 << kMaxLog];
-std::mutex g_tw_mu;
-float2 *g_tw_addr[kMaxDevices] = {};
 
-// The current device's tables, filled and complete on return.
+// The current context's tables, filled and complete on return.
 cudaError_t pow2_tables(float2 **out) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lk(g_tw_mu);
-    if (!g_tw_addr[dev]) {
+    static std::mutex mu;
+    static float2 *addr[kCtxSlots] = {};
+    const int slot = context_slot();
+    std::lock_guard<std::mutex> lk(mu);
+    if (slot < 0 || !addr[slot]) {
         void *q = nullptr;
-        e = cudaGetSymbolAddress(&q, g_pow2_tw);
+        cudaError_t e = cudaGetSymbolAddress(&q, g_pow2_tw);
         cudaStream_t s = nullptr;
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
         if (e != cudaSuccess) return e;
@@ -368,9 +391,11 @@ cudaError_t pow2_tables(float2 **out) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         cudaStreamDestroy(s);
         if (e != cudaSuccess) return e;
-        g_tw_addr[dev] = (float2 *)q;
+        *out = (float2 *)q;
+        if (slot >= 0) addr[slot] = *out;
+        return cudaSuccess;
     }
-    *out = g_tw_addr[dev];
+    *out = addr[slot];
     return cudaSuccess;
 }
 

@@ -173,6 +173,12 @@ long long wait_limit();
 cudaError_t launch_uvw(const double *enu_dev, int n_ant, double lat, double dec, const double *ha_dev, int n_time,
                        double *uvw_dev, cudaStream_t s);
 
+// Number of the calling thread's current CUDA context among those seen by the library
+// (-1: none, or more than kCtxSlots of them): what the library keeps on the device
+// beside a psc_ctx belongs to one such context.
+constexpr int kCtxSlots = 16;
+int context_slot();
+
 // Launchers (defined in the .cu files).
 cudaError_t launch_eval(const EvalArgs &a, bool predict, cudaStream_t s);
 // Persistent fused launch over several contexts (device arrays of EvalArgs and
