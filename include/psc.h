@@ -183,8 +183,10 @@ psc_status psc_uvw(int n_ant, const double *ant_enu_m, double lat_rad, double de
  * parts, FP32 accumulation; error at FP32 rounding level; operands staged by
  * TMA) with a temporary workspace of 6 N K + 24 Ng K bytes, K = N rounded
  * up to a multiple of 32; otherwise FP32 SIMT with a temporary complex64
- * [N][Ng].  Synchronises the stream before freeing the
- * workspace and returning; PSC_ERR_TIMEOUT if a tensor-core wait ran out. */
+ * [N][Ng].  Synchronises the stream before returning; the workspaces of this
+ * and the other model-grid calls come from a pool of the library's own, which keeps up to
+ * 128 MB between calls until the last psc_ctx is destroyed.  PSC_ERR_TIMEOUT if a
+ * tensor-core wait ran out. */
 psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void *grid_out,
                           void *stream);
 

@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -145,6 +146,67 @@ cudaError_t dalloc(T **p, size_t n) {
     return cudaMalloc((void **)p, sizeof(T) * (n ? n : 1));
 }
 
+// Workspaces of the calls that make a model grid, from a pool of the library's own, one
+// a CUDA context: allocating and freeing 75 MB took 220 of the 790 us of
+// psc_model_grid_components.  Stream-ordered (safe with several threads and streams); up
+// to kPoolKeep bytes stay with the pool between calls and go back when the last psc_ctx
+// is destroyed.  Without a pool, cudaMalloc.
+constexpr uint64_t kPoolKeep = (uint64_t)128 << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kCtxSlots] = {};
+int g_live_ctx = 0;
+
+struct Workspace {
+    void *p = nullptr;
+    bool pooled = false;
+};
+
+cudaError_t ws_alloc(Workspace *w, size_t bytes, cudaStream_t s) {
+    const int slot = context_slot();
+    cudaMemPool_t pool = nullptr;
+    if (slot >= 0) {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        if (!g_pool[slot]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            uint64_t keep = kPoolKeep;
+            cudaError_t e = cudaGetDevice(&props.location.id);
+            if (e == cudaSuccess) e = cudaMemPoolCreate(&pool, &props);
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e == cudaSuccess) g_pool[slot] = pool;
+            else if (pool) cudaMemPoolDestroy(pool);
+        }
+        pool = g_pool[slot];
+    }
+    if (pool && cudaMallocFromPoolAsync(&w->p, bytes, pool, s) == cudaSuccess) {
+        w->pooled = true;
+        return cudaSuccess;
+    }
+    cudaGetLastError();
+    w->p = nullptr;
+    return cudaMalloc(&w->p, bytes);
+}
+
+// Frees the workspace and waits for the stream (and what it still does with it).
+cudaError_t ws_free(Workspace *w, cudaStream_t s) {
+    if (w->p && w->pooled) cudaFreeAsync(w->p, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (w->p && !w->pooled) cudaFree(w->p);
+    w->p = nullptr;
+    return e;
+}
+
+// One psc_ctx more or less; the last one's end returns what its CUDA context's pool holds.
+void count_ctx(int by) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_live_ctx += by;
+    if (g_live_ctx > 0) return;
+    const int slot = context_slot();
+    if (slot >= 0 && g_pool[slot]) cudaMemPoolTrimTo(g_pool[slot], 0);
+}
+
 void free_ctx(psc_ctx *c) {
     if (!c) return;
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -164,6 +226,7 @@ void free_ctx(psc_ctx *c) {
     cudaFree(c->d_lm_cur); cudaFree(c->d_mat); cudaFree(c->d_mat32); cudaFree(c->d_rhs); cudaFree(c->d_state);
     cudaFree(c->d_state0); cudaFree(c->d_lm0);
     delete c;
+    count_ctx(-1);
 }
 
 // Largest visibility separation within one thread's kv time steps (cells).
@@ -583,15 +646,15 @@ psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void 
     if (!check_grid_desc(gd, &why)) return fail(nullptr, PSC_ERR_ARG, why);
     if (!image_dev || !grid_out) return fail(nullptr, PSC_ERR_ARG, "image and grid pointers must be non-NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    void *ws = nullptr;
+    Workspace ws;
     int *err_dev = nullptr;
     int herr = 0;
     const size_t ws_bytes = model_grid_ws_bytes(gd->n_img, gd->n_grid);
-    cudaError_t e = ws_bytes ? cudaMalloc(&ws, ws_bytes) : cudaSuccess;
-    if (e == cudaSuccess) e = launch_model_grid(gd->n_img, gd->n_grid, image_dev, ws, (float2 *)grid_out, &err_dev, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && err_dev) e = cudaMemcpy(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost);
-    if (ws) cudaFree(ws);
+    cudaError_t e = ws_bytes ? ws_alloc(&ws, ws_bytes, s) : cudaSuccess;
+    if (e == cudaSuccess) e = launch_model_grid(gd->n_img, gd->n_grid, image_dev, ws.p, (float2 *)grid_out, &err_dev, s);
+    if (e == cudaSuccess && err_dev) e = cudaMemcpyAsync(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+    const cudaError_t se = ws_free(&ws, s);
+    if (e == cudaSuccess) e = se;
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "psc_model_grid");
     if (herr) return fail(nullptr, PSC_ERR_TIMEOUT, "psc_model_grid: a tensor-core wait timed out");
     return PSC_OK;
@@ -607,16 +670,16 @@ psc_status psc_model_grid_components(int n_comp, const double *comp_lmS, int n_g
     for (int k = 0; k < 3 * n_comp; ++k)
         if (!std::isfinite(comp_lmS[k])) return fail(nullptr, PSC_ERR_ARG, "components must be finite");
     cudaStream_t s = (cudaStream_t)stream;
-    void *ws = nullptr;
+    Workspace ws;
     int *err_dev = nullptr;
     int herr = 0;
     const double du = 1.0 / (n_grid * cell_rad);
-    cudaError_t e = cudaMalloc(&ws, model_grid_comp_ws_bytes(n_comp, n_grid, 3));
+    cudaError_t e = ws_alloc(&ws, model_grid_comp_ws_bytes(n_comp, n_grid, 3), s);
     if (e == cudaSuccess)
-        e = launch_model_grid_comp(n_comp, comp_lmS, 3, 0.0, n_grid, du, ws, (float2 *)grid_out, &err_dev, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaMemcpy(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaFree(ws);
+        e = launch_model_grid_comp(n_comp, comp_lmS, 3, 0.0, n_grid, du, ws.p, (float2 *)grid_out, &err_dev, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+    const cudaError_t se = ws_free(&ws, s);
+    if (e == cudaSuccess) e = se;
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "psc_model_grid_components");
     if (herr) return fail(nullptr, PSC_ERR_TIMEOUT, "psc_model_grid_components: a tensor-core wait timed out");
     return PSC_OK;
@@ -734,21 +797,22 @@ psc_status psc_model_grid_wstack(int n_comp, const double *comp_lmSn, int n_grid
     for (int k = 0; k < 4 * n_comp; ++k)
         if (!std::isfinite(comp_lmSn[k])) return fail(nullptr, PSC_ERR_ARG, "components must be finite");
     cudaStream_t s = (cudaStream_t)stream;
-    void *ws = nullptr;
+    Workspace ws;
     int *err_dev = nullptr;
     int herr = 0;
     const double du = 1.0 / (n_grid * cell_rad);
     const size_t plane = (size_t)n_grid * n_grid;
-    cudaError_t e = cudaMalloc(&ws, model_grid_comp_ws_bytes(n_comp, n_grid, 4));
+    cudaError_t e = ws_alloc(&ws, model_grid_comp_ws_bytes(n_comp, n_grid, 4), s);
     for (int p = 0; p < n_planes && e == cudaSuccess; ++p) {
-        e = launch_model_grid_comp(n_comp, comp_lmSn, 4, w0 + p * dw, n_grid, du, ws, (float2 *)grids_out + p * plane,
+        e = launch_model_grid_comp(n_comp, comp_lmSn, 4, w0 + p * dw, n_grid, du, ws.p, (float2 *)grids_out + p * plane,
                                    &err_dev, s);
         // the workspace (and its error flag) is reused by the next plane
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = cudaMemcpy(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost);
         if (herr) break;
     }
-    cudaFree(ws);
+    const cudaError_t se = ws_free(&ws, s);
+    if (e == cudaSuccess) e = se;
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "psc_model_grid_wstack");
     if (herr) return fail(nullptr, PSC_ERR_TIMEOUT, "psc_model_grid_wstack: a tensor-core wait timed out");
     return PSC_OK;
@@ -771,6 +835,7 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
         if (!(obs->freq_hz[c] > 0.0) || !std::isfinite(obs->freq_hz[c])) return fail(nullptr, PSC_ERR_ARG, "frequencies must be > 0");
 
     psc_ctx *c = new psc_ctx();
+    count_ctx(1);
     c->stream = (cudaStream_t)stream;
     c->n_ant = obs->n_ant;
     c->n_bl = obs->n_ant * (obs->n_ant - 1) / 2;
