@@ -353,7 +353,7 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * A context without a tiling (its current values then count as 32, 4, 1) picks its
  * launch shape by size: from two million visibilities on, flat bricks
  * (psc_set_flat_tiling) or, for small apertures and enough baselines, the track
- * kernel (psc_set_track_tiling; in a batch only if every context would); below, the
+ * kernel (psc_set_track_tiling; in a batch only if no context has a tiling); below, the
  * rectangle (32, 4, 1), with the rows of each visibility shared among lanes where
  * there are too few visibilities to fill the chip (the same sums bit for bit). */
 psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thread);
@@ -579,7 +579,8 @@ const char *psc_batch_last_error(const psc_batch *b);
 
 /* Name of the fused kernel that the batch's persistent launch runs
  * ("eval_kernel<...>" for brick tilings, "track_kernel<kv>" when every
- * context has the track tiling).  Static storage; never NULL. */
+ * context runs the track kernel; a batch without tilings may run some of its
+ * contexts in a second launch of that kernel).  Static storage; never NULL. */
 const char *psc_batch_kernel(const psc_batch *b);
 
 /* Picks each context's launch shape by timing the fused kernel on its own

@@ -369,7 +369,12 @@ psc_status ensure_partials(psc_ctx *c, const Shape &s) {
     size_t need = (size_t)c->n_bl * bricks_per_bl(c, s);
     // room for the other kernel too where the choice depends on the rest of a
     // batch: another batch's tables must not lose the records they point at
-    if (!c->trk_set) need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, brick_shape(c)));
+    if (!c->trk_set) {
+        Shape o = brick_shape(c);
+        need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, o));
+        o.trk_kv = want_track(c) > 0 ? 1 : 0;                         // more records than two a lane
+        need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, o));
+    }
     if (need <= c->partials_cap) return PSC_OK;
     cudaFree(c->d_partials);
     c->d_partials = nullptr;
@@ -1498,13 +1503,13 @@ struct psc_batch {
     std::vector<double> w_scale;
     // device tables (rebuilt by build_tables)
     EvalArgs *d_eval = nullptr;
-    long long *d_prefix = nullptr;
+    long long *d_prefix = nullptr;   // bricks before each context, then (n + 1 on) track items before each
     RedArgs *d_red = nullptr;
     int *d_bl_prefix = nullptr;
     LMArgs *d_lm = nullptr;
     const LMState **d_st0 = nullptr;
     const double **d_lm0 = nullptr;
-    unsigned long long *d_queue = nullptr;
+    unsigned long long *d_queue = nullptr;   // of the brick and of the track kernel
     int *d_active = nullptr;
     // psc_batch_end: every context's offsets, solver state and wait flag
     // gathered on the device ([lm 2n_ant...][state...][flag...]) and copied
@@ -1514,11 +1519,12 @@ struct psc_batch {
     std::vector<size_t> lm_off;
     int total_bl = 0;
     int max_ant = 0, max_bpb = 0;    // most antennas of a context, most records of a baseline
-    int grid = 0;
-    int threads = 128;           // fused-kernel block size: the widest context's shape
+    int grid = 0, trk_grid = 0;
+    bool bricks = false;         // some context runs the brick kernel
+    int threads = 128;           // brick-kernel block size: the widest context's shape
     bool split = false;          // some context shares its visibilities among lanes
     bool stacked = false;        // every context reads a residual-w stack (else none does)
-    int track = 0;               // > 0: the persistent launch runs the track kernel, this many visibilities per lane
+    int track = 0;               // > 0: some context runs the track kernel, this many visibilities per lane
     int trk_tabc = 0;            // track kernel: table capacity of a warp buffer (entries)
     size_t eval_dyn = 0, lm_dyn = 0;
     cudaGraph_t graph = nullptr;
@@ -1567,7 +1573,7 @@ void free_batch(psc_batch *b) {
 psc_status build_tables(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     std::vector<EvalArgs> ev(n);
-    std::vector<long long> prefix(n + 1, 0);
+    std::vector<long long> prefix(2 * (n + 1), 0);
     std::vector<RedArgs> red(n);
     std::vector<int> blp(n + 1, 0);
     std::vector<LMArgs> lm(n);
@@ -1575,20 +1581,23 @@ psc_status build_tables(psc_batch *b) {
     std::vector<const double *> lm0(n);
     size_t dyn = 0, lmd = 0;
     int threads = 32, max_ant = 0, max_bpb = 0;
-    // contexts without a tiling take the track kernel only if all of them would, with
-    // the same visibilities per lane: one fused kernel serves the launch
-    int all_trk = auto_track(b->ctxs[0]);
-    for (psc_ctx *c : b->ctxs)
-        if (auto_track(c) != all_trk) all_trk = 0;
-    bool split = false;
+    // Where no context has a tiling, each takes its own kernel (two persistent launches
+    // an iteration; one for 27 to 197 antennas, 38 to 411 x 16, took 5.7 ms of bricks
+    // against 4.6 in both), all of the track kernel with the fewest visibilities per
+    // lane among them; one fused kernel serves a batch with tilings.
+    bool any_set = false;
+    int kv_auto = 2;
+    for (psc_ctx *c : b->ctxs) {
+        any_set = any_set || c->trk_set;
+        if (auto_track(c) > 0) kv_auto = std::min(kv_auto, auto_track(c));
+    }
+    bool split = false, bricks = false;
     std::vector<Shape> shapes(n);
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
         shapes[k] = brick_shape(c);
-        shapes[k].trk_kv = c->trk_set ? c->trk_kv : all_trk;
+        shapes[k].trk_kv = c->trk_set ? c->trk_kv : !any_set && auto_track(c) > 0 ? kv_auto : 0;
         const Shape &shape = shapes[k];
-        threads = std::max(threads, eval_threads(shape));
-        split = split || (shape.trk_kv == 0 && shape.split > 1);
         psc_status st = ensure_partials(c, shape);
         if (st == PSC_OK && shape.trk_kv > 0) st = trk_prepare(c);
         if (st != PSC_OK) return bfail(b, st, c->err);
@@ -1597,13 +1606,20 @@ psc_status build_tables(psc_batch *b) {
         ev[k].w = b->w[k];
         ev[k].w_scale = (float)b->w_scale[k];
         ev[k].skip = c->d_done;
-        prefix[k + 1] = prefix[k] + ev[k].n_bricks;
+        const bool trk = shape.trk_kv > 0;
+        prefix[k + 1] = prefix[k] + (trk ? 0 : ev[k].n_bricks);
+        prefix[n + 2 + k] = prefix[n + 1 + k] + (trk ? ev[k].n_bricks : 0);
         red[k] = red_args(c, shape, c->d_ev, c->d_done);
         blp[k + 1] = blp[k] + c->n_bl;
         lm[k] = lm_args(c);
         st0[k] = c->d_state0;
         lm0[k] = c->d_lm0;
-        dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support) + eval_stack_smem(c->wp_n));
+        if (!trk) {
+            bricks = true;
+            split = split || shape.split > 1;
+            threads = std::max(threads, eval_threads(shape));
+            dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support) + eval_stack_smem(c->wp_n));
+        }
         lmd = std::max(lmd, lm_smem_bytes(c->n_ant));
         max_ant = std::max(max_ant, c->n_ant);
         max_bpb = std::max(max_bpb, red[k].bpb);
@@ -1614,8 +1630,7 @@ psc_status build_tables(psc_batch *b) {
     b->max_bpb = max_bpb;
     b->eval_dyn = dyn;
     b->lm_dyn = lmd;
-    // one fused kernel per persistent launch: the track kernel for all
-    // contexts (same visibilities per lane) or for none
+    // with tilings: the track kernel for all contexts (same visibilities per lane) or for none
     int n_trk = 0, kv_trk = 0, tabc = 0;
     for (int k = 0; k < n; ++k) {
         const int kv = shapes[k].trk_kv;
@@ -1625,38 +1640,41 @@ psc_status build_tables(psc_batch *b) {
         else if (kv_trk == 0) kv_trk = kv;
         tabc = std::max(tabc, ev[k].trk_tabc);
     }
-    if (n_trk != 0 && (n_trk != n || kv_trk < 0))
+    if (any_set && n_trk != 0 && (n_trk != n || kv_trk < 0))
         return bfail(b, PSC_ERR_ARG, "a batch runs one fused kernel: give every context the same track tiling, or none");
     b->track = n_trk ? kv_trk : 0;
     b->trk_tabc = tabc;
-    int per_sm = 0, dev = 0, n_sm = 0;
+    int per_sm = 0, trk_per_sm = 0, dev = 0, n_sm = 0;
     b->stacked = b->ctxs[0]->wp_n > 0;
     b->split = split;
+    b->bricks = bricks;
     if (b->track) {
         const size_t tdyn = track_dyn_smem(kTrkCap, tabc);
         PSC_BCUDA(b, set_track_smem(tdyn));
-        PSC_BCUDA(b, track_occupancy(b->track, tdyn, &per_sm));
-    } else {
+        PSC_BCUDA(b, track_occupancy(b->track, tdyn, &trk_per_sm));
+    }
+    if (bricks) {
         PSC_BCUDA(b, set_eval_smem(dyn - eval_stack_smem(b->ctxs[0]->wp_n)));
         PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, b->split, &per_sm));
     }
     PSC_BCUDA(b, cudaGetDevice(&dev));
     PSC_BCUDA(b, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     b->grid = std::max(1, per_sm) * n_sm;
+    b->trk_grid = std::max(1, trk_per_sm) * n_sm;
     if (!b->d_eval) {
         PSC_BCUDA(b, dalloc(&b->d_eval, n));
-        PSC_BCUDA(b, dalloc(&b->d_prefix, n + 1));
+        PSC_BCUDA(b, dalloc(&b->d_prefix, 2 * (n + 1)));
         PSC_BCUDA(b, dalloc(&b->d_red, n));
         PSC_BCUDA(b, dalloc(&b->d_bl_prefix, n + 1));
         PSC_BCUDA(b, dalloc(&b->d_lm, n));
         PSC_BCUDA(b, dalloc(&b->d_st0, n));
         PSC_BCUDA(b, dalloc(&b->d_lm0, n));
-        PSC_BCUDA(b, dalloc(&b->d_queue, 1));
+        PSC_BCUDA(b, dalloc(&b->d_queue, 2));
         PSC_BCUDA(b, dalloc(&b->d_active, 1));
     }
     cudaStream_t s = b->stream;
     PSC_BCUDA(b, cudaMemcpyAsync(b->d_eval, ev.data(), sizeof(EvalArgs) * n, cudaMemcpyHostToDevice, s));
-    PSC_BCUDA(b, cudaMemcpyAsync(b->d_prefix, prefix.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice, s));
+    PSC_BCUDA(b, cudaMemcpyAsync(b->d_prefix, prefix.data(), sizeof(long long) * prefix.size(), cudaMemcpyHostToDevice, s));
     PSC_BCUDA(b, cudaMemcpyAsync(b->d_red, red.data(), sizeof(RedArgs) * n, cudaMemcpyHostToDevice, s));
     PSC_BCUDA(b, cudaMemcpyAsync(b->d_bl_prefix, blp.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
     PSC_BCUDA(b, cudaMemcpyAsync(b->d_lm, lm.data(), sizeof(LMArgs) * n, cudaMemcpyHostToDevice, s));
@@ -1667,13 +1685,14 @@ psc_status build_tables(psc_batch *b) {
     return PSC_OK;
 }
 
-// The batch's persistent fused launch (its work queue already reset).
+// The batch's persistent fused launches (their work queues already reset).
 psc_status launch_fused(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
     if (b->track)
-        PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->track, kTrkCap, b->trk_tabc, b->grid, s));
-    else
+        PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix + n + 1, n, b->d_queue + 1, b->track, kTrkCap, b->trk_tabc,
+                                        b->trk_grid, s));
+    if (b->bricks)
         PSC_BCUDA(b, launch_eval_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->threads, b->eval_dyn, b->grid,
                                        b->stacked, b->split, s));
     return PSC_OK;
@@ -1683,7 +1702,7 @@ psc_status launch_fused(psc_batch *b) {
 psc_status enqueue_iteration(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
-    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned long long), s));
+    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(unsigned long long), s));
     if (b->prof) {
         while (b->ev_pool.size() < b->ev_used + 2) {
             cudaEvent_t e;
@@ -2003,7 +2022,7 @@ psc_status psc_batch_autotune(psc_batch *b, int *tiling_out) {
             float ms = 0.f;
             for (int r = 0; r < 2 && st == PSC_OK; ++r) {             // warm, then timed
                 if (r == 1) e = cudaEventRecord(e0, b->stream);
-                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned long long), b->stream);
+                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(unsigned long long), b->stream);
                 if (e == cudaSuccess) st = launch_fused(b);
                 if (r == 1 && e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             }
@@ -2175,8 +2194,8 @@ const char *psc_batch_last_error(const psc_batch *b) { return b ? b->err.c_str()
 
 const char *psc_batch_kernel(const psc_batch *b) {
     if (!b) return "";
-    if (b->track == 2) return "track_kernel<2>";
-    if (b->track == 1) return "track_kernel<1>";
+    if (b->track == 2 && !b->bricks) return "track_kernel<2>";
+    if (b->track == 1 && !b->bricks) return "track_kernel<1>";
     return b->stacked ? "eval_kernel<false, true>" : "eval_kernel<false, false>";
 }
 
