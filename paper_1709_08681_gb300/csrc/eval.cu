@@ -77,16 +77,22 @@ constexpr int kWCap = 3060;            // staged cells of all planes (24 KB: 4.8
 // three of the lanes add them up in row order -- the additions of the one-lane loop
 // in eval_brick, so every sum has the same bits.  For contexts with too few
 // visibilities to fill the chip, where a lane's chain of some 600 taps is what the
-// launch waits for: 21,060 visibilities, 185 us with a lane each, 72 us with 8.  Shared memory s_split: [kMaxThreads] windows, [kMaxThreads][6] sums, then
-// [kMaxThreads / split][support] row sums (P, Q).
+// launch waits for: 21,060 visibilities, 185 us with a lane each, 56 us with 8.  A
+// visibility's lanes sit in different warps: the lanes of one warp then walk the same
+// row of neighbouring visibilities, spans of one length from neighbouring addresses
+// (next to each other, in different rows, they took 70 us).  Shared memory s_split:
+// [kMaxThreads] windows, [kMaxThreads][6] sums, then [support][kMaxThreads / split]
+// row sums (P, Q).
 __device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_tab, const BlockSharedT<true> &sh,
                                            float4 *s_split, int bl, int brick, int c_first, bool staged, int bx0, int by0) {
     const int tid = threadIdx.x, S = a.support;
-    const int grp = tid / a.split, sub = tid & (a.split - 1), groups = blockDim.x / a.split;
+    const int groups = blockDim.x / a.split, grp = tid & (groups - 1), sub = tid / groups;
     const int t_first = (brick % a.n_tt) * a.t_tile;
     const int n_t = min(a.t_tile, a.nt - t_first), n_c = min(a.c_group, a.nc - c_first);
+    // an even number of cells a row and an aligned grid: every aligned pair of cells lies within it
+    const bool pairs = a.grid_bf16 == nullptr && a.ng % 2 == 0 && ((uintptr_t)a.grid & 15) == 0;
     float *sums = reinterpret_cast<float *>(s_split + kMaxThreads);
-    float4 *rows = s_split + kMaxThreads + kMaxThreads * 6 / 4 + grp * S;
+    float4 *rows = s_split + kMaxThreads + kMaxThreads * 6 / 4 + grp;       // [support][groups]
     const float ov = (float)a.ov;
     for (int i0 = 0; i0 < n_t * n_c; i0 += groups) {
         const int i = i0 + grp;
@@ -125,35 +131,58 @@ __device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_ta
                     a_lo = max(a_lo, -ix0);
                     a_hi = min(a_hi, a.ng - 1 - ix0);
                     float pr = 0.f, pi = 0.f, qr = 0.f, qi = 0.f;
-                    const size_t row = (size_t)(iy0 + b) * a.ng + ix0;
-                    float dd = __fmul_rn(hx - (float)a_lo, ov);
-#pragma unroll 4
-                    for (int aa = a_lo; aa <= a_hi; ++aa, dd = __fsub_rn(dd, ov)) {
-                        const float2 g = cmul(grid_cell(a, row + aa), sh.phx[aa]);
-                        const float s2 = fmaf(dd, dd, dyo2);
-                        const float tv = sqrt_fast(s2);
-                        const float tf = __fadd_rz(tv, 8388608.0f);
-                        const float2 e = lds_f2(tab_adj + ((unsigned)__float_as_int(tf) << 3));
-                        const float A = fmaf(tv, e.y, e.x);
-                        pr = fmaf(A, g.x, pr);
-                        pi = fmaf(A, g.y, pi);
-                        const float Ad = __fmul_rn(A, dd);
-                        qr = fmaf(Ad, g.x, qr);
-                        qi = fmaf(Ad, g.y, qi);
+                    if (a_lo <= a_hi) {
+                        // Four cells at a time, the next four fetched ahead, as aligned pairs
+                        // where rows hold them (one cell a load: 72 us); cells outside the
+                        // row's span take a factor of zero, which leaves the sums.
+                        const size_t row = (size_t)(iy0 + b) * a.ng + ix0;
+                        const int first = pairs ? a_lo - ((ix0 + a_lo) & 1) : a_lo;
+                        const int last = pairs ? a_hi - ((ix0 + a_hi) & 1) : a_hi;
+                        auto load2 = [&](int aa) {
+                            if (pairs) return __ldg(reinterpret_cast<const float4 *>(a.grid + row + min(aa, last)));
+                            const float2 g0 = grid_cell(a, row + min(aa, last)), g1 = grid_cell(a, row + min(aa + 1, last));
+                            return make_float4(g0.x, g0.y, g1.x, g1.y);
+                        };
+                        float dd = __fmul_rn(hx - (float)a_lo, ov);
+                        float4 n0 = load2(first), n1 = load2(first + 2);
+                        for (int aa = first; aa <= a_hi; aa += 4) {
+                            const float2 gc[4] = {make_float2(n0.x, n0.y), make_float2(n0.z, n0.w),
+                                                  make_float2(n1.x, n1.y), make_float2(n1.z, n1.w)};
+                            n0 = load2(aa + 4);
+                            n1 = load2(aa + 6);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const bool in = aa + j >= a_lo && aa + j <= a_hi;
+                                float2 g = cmul(gc[j], sh.phx[in ? aa + j : a_lo]);
+                                g = make_float2(in ? g.x : 0.f, in ? g.y : 0.f);
+                                const float d = in ? dd : 0.f;
+                                const float s2 = fmaf(d, d, dyo2);
+                                const float tv = sqrt_fast(s2);
+                                const float tf = __fadd_rz(tv, 8388608.0f);
+                                const float2 e = lds_f2(tab_adj + ((unsigned)__float_as_int(tf) << 3));
+                                const float A = fmaf(tv, e.y, e.x);
+                                pr = fmaf(A, g.x, pr);
+                                pi = fmaf(A, g.y, pi);
+                                const float Ad = __fmul_rn(A, d);
+                                qr = fmaf(Ad, g.x, qr);
+                                qi = fmaf(Ad, g.y, qi);
+                                dd = in ? __fsub_rn(dd, ov) : dd;
+                            }
+                        }
                     }
                     const float2 py = sh.phy[b];
                     P = cmul(make_float2(pr, pi), py);
                     Q = cmul(make_float2(qr, qi), py);
                 }
             }
-            rows[b] = make_float4(P.x, P.y, Q.x, Q.y);
+            rows[b * groups] = make_float4(P.x, P.y, Q.x, Q.y);
         }
-        __syncwarp();
+        __syncthreads();
         if (on && sub < 3) {
-            // lane 0: sum P, lane 1: sum Q, lane 2: sum dy P, in row order
+            // the first lane: sum P, the second: sum Q, the third: sum dy P, in row order
             float x = 0.f, y = 0.f;
             for (int b = b_lo; b <= b_hi; ++b) {
-                const float2 v = reinterpret_cast<const float2 *>(rows + b)[sub == 1];
+                const float2 v = reinterpret_cast<const float2 *>(rows + b * groups)[sub == 1];
                 const float dy = hy - (float)b;
                 x = sub == 2 ? fmaf(dy, v.x, x) : x + v.x;
                 y = sub == 2 ? fmaf(dy, v.y, y) : y + v.y;
@@ -161,7 +190,7 @@ __device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_ta
             sums[6 * slot + 2 * sub] = x;
             sums[6 * slot + 2 * sub + 1] = y;
         }
-        __syncwarp();
+        __syncthreads();
     }
 }
 
@@ -176,12 +205,11 @@ __device__ __forceinline__ void split_taps(const EvalArgs &a, const float2 *s_ta
 // the brick, its sums and their order are those of the rectangle without it.
 template <bool kPredict, int kV, bool kW, bool kSplit>
 __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 *s_tab, BlockSharedT<!kW> &sh,
-                                           float4 *s_split, float2 *s_wtile, float (&acc)[kRed]) {
+                                           float4 *s_split, float2 *s_wtile, float (&acc)[kRed], bool &active) {
     const int tid = threadIdx.x;
     // brick -> baseline, this thread's channel c and first time step t0, and
     // the block's channels [c_first, c_first + n_ch) (lc = c - c_first)
     int bl, c, t0, c_first, n_ch;
-    bool active;
     if (a.flat > 0) {
         bl = brick / a.bpb;
         const int first = (brick - bl * a.bpb) * a.flat;
@@ -289,7 +317,7 @@ __device__ __forceinline__ void eval_brick(const EvalArgs &a, int brick, float2 
         }
     }
     // radial tables of this block's channels as (c_n, s_n), zero-padded
-    for (int j = 0; j < n_ch; ++j) {
+    for (int j = 0; j < (kSplit ? min(n_ch, a.nc - c_first) : n_ch); ++j) {
         const int cc = c_first + j;
         const int off = cc < a.nc ? a.chan[cc].tab_off : 0;
         const int len = cc < a.nc ? a.chan[cc].tab_len : 0;
@@ -720,16 +748,19 @@ __global__ void __launch_bounds__(kMaxThreads, kW || kSplit ? 3 : 0) eval_kernel
     float4 *s_split = reinterpret_cast<float4 *>(s_tab + (a.c_group * a.tab_stride + 1) / 2 * 2);
     // the stack's tile starts after the tables, whatever their number (a multiple of 16 bytes)
     float2 *s_wtile = s_tab + ((a.flat > 0 ? a.ch_span : a.c_group) * a.tab_stride + 1) / 2 * 2;
-    if (kSplit && a.split > 1) eval_brick<kPredict, 1, kW, kSplit>(a, brick, s_tab, sh, s_split, nullptr, acc);
-    else if (a.kv == 2) eval_brick<kPredict, 2, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc);
-    else eval_brick<kPredict, 1, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc);
+    bool active = false;                              // this thread holds a visibility
+    if (kSplit && a.split > 1) eval_brick<kPredict, 1, kW, kSplit>(a, brick, s_tab, sh, s_split, nullptr, acc, active);
+    else if (a.kv == 2) eval_brick<kPredict, 2, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc, active);
+    else eval_brick<kPredict, 1, kW, false>(a, brick, s_tab, sh, nullptr, s_wtile, acc, active);
     if constexpr (!kPredict) {
         // ---- block reduction: a butterfly within each warp -- compensated
         // (Knuth's TwoSum, the rounding errors summed beside) for chi^2 and the
         // gradient, plain FP32 for the normal blocks -- then FP64 across warps ----
         float comp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+        // few warps of a split brick hold visibilities (the others' sums are zeros)
+        const bool any = !kSplit || __any_sync(0xffffffffu, active);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = any ? 16 : 0; o > 0; o >>= 1) {
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
                 const float so = __shfl_xor_sync(0xffffffffu, acc[k], o);
