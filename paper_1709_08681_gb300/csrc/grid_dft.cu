@@ -235,9 +235,11 @@ __global__ void split_dft_matrix_kernel(const double2 *__restrict__ W, int n, in
 // components on a 2048^2 grid took).  With g - Ng/2 = kQ h + q + g_0 a phasor is the
 // product of one of kQ and one of Ng / kQ others, which a block evaluates once in
 // FP64 for its kKb components and multiplies as pairs of FP32 (error below 2^-44,
-// against the split's 2^-24): 104 us.
+// against the split's 2^-24); the kQ fine ones in turn are products of two.  59 us
+// (106 us with each fine one evaluated).
 constexpr int kKb = 16;                              // components of a block
-constexpr int kQ = 64;                               // fine steps
+constexpr int kQ = 64;                               // fine steps, themselves products of kQ0 and kQ / kQ0 phasors
+constexpr int kQ0 = 8;
 
 struct C2 { float rh, ih, rl, il; };                 // a complex number as two FP32 parts
 
@@ -277,12 +279,24 @@ __device__ __forceinline__ void split3p(float hi, float lo, bf16 &h, bf16 &m, bf
 __global__ void __launch_bounds__(256) split_comp_kernel(const double *__restrict__ comp, int n_comp, int stride, double wp,
                                                          int kp, int ng, int b_rows, double du, bf16 *__restrict__ Ar,
                                                          bf16 *__restrict__ Ai, bf16 *__restrict__ Br, bf16 *__restrict__ Bi) {
-    __shared__ C2 s_q[2][kQ][kKb];                   // fine steps of u l and v m
+    __shared__ C2 s_f[2][2][kQ0][kKb];               // steps of one cell and of kQ0 cells of u l and v m
+    __shared__ C2 s_q[2][kQ][kKb];                   // fine steps
     __shared__ C2 s_h[2][kKb];                       // this group of kQ rows
     const int k0 = blockIdx.x * kKb, tid = threadIdx.x;
+    static_assert(kQ == kQ0 * kQ0);
+    for (int e = tid; e < 4 * kQ0 * kKb; e += blockDim.x) {
+        const int d = e / (2 * kQ0 * kKb), lvl = e / (kQ0 * kKb) % 2, q = e / kKb % kQ0, k = k0 + e % kKb;
+        const double step = (double)(lvl ? kQ0 * q : q) * du;
+        s_f[d][lvl][q][e % kKb] = k < n_comp ? c2_phasor(step * comp[(size_t)stride * k + d], 1.0) : C2{0.f, 0.f, 0.f, 0.f};
+    }
+    __syncthreads();
     for (int e = tid; e < 2 * kQ * kKb; e += blockDim.x) {
-        const int d = e / (kQ * kKb), q = e / kKb % kQ, k = k0 + e % kKb;
-        s_q[d][q][e % kKb] = k < n_comp ? c2_phasor((double)q * du * comp[(size_t)stride * k + d], 1.0) : C2{0.f, 0.f, 0.f, 0.f};
+        const int d = e / (kQ * kKb), q = e / kKb % kQ, kk = e % kKb;
+        const C2 x = s_f[d][0][q % kQ0][kk], y = s_f[d][1][q / kQ0][kk];
+        C2 z;
+        c2_dot(x.rh, x.rl, y.rh, y.rl, -x.ih, -x.il, y.ih, y.il, z.rh, z.rl);
+        c2_dot(x.rh, x.rl, y.ih, y.il, x.ih, x.il, y.rh, y.rl, z.ih, z.il);
+        s_q[d][q][kk] = z;
     }
     const int n_grp = (ng + kQ - 1) / kQ;
     for (int grp = blockIdx.y; grp < n_grp; grp += gridDim.y) {
@@ -327,7 +341,8 @@ __global__ void __launch_bounds__(256) split_comp_kernel(const double *__restric
 
 // What the half-plane pass leaves of a Hermitian component grid (B's rows end at
 // Ng/2): row v = 0, the sums of A's rows, and column gx = 0 for v > 0, the sums of
-// A[0] conj(B[Ng - gy]).  A warp per cell.
+// A[0] conj(B[Ng - gy]).  A warp per cell, 16-byte loads (19 us for Ng = 2048, 2000
+// components; 37 us with single elements, whose loads in flight bounded it).
 __global__ void comp_edge_kernel(const bf16 *__restrict__ Ar, const bf16 *__restrict__ Ai, const bf16 *__restrict__ Br,
                                  const bf16 *__restrict__ Bi, int ng, int kp, float2 *__restrict__ G) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -337,19 +352,41 @@ __global__ void comp_edge_kernel(const bf16 *__restrict__ Ar, const bf16 *__rest
     const int gx = row ? w : 0, gy = row ? half : half + 1 + (w - ng);
     const size_t pa = (size_t)ng * kp, pb = (size_t)half * kp;
     const size_t oa = (size_t)gx * kp, ob = (size_t)(ng - gy) * kp;
-    auto sum3 = [](const bf16 *p, size_t plane, size_t at) {
-        return (__bfloat162float(p[at]) + __bfloat162float(p[plane + at])) + __bfloat162float(p[2 * plane + at]);
-    };
     float re = 0.f, im = 0.f;
-    for (int k = lane; k < kp; k += 32) {
-        const float ar = sum3(Ar, pa, oa + k), ai = sum3(Ai, pa, oa + k);
-        float br = 1.f, bi = 0.f;
-        if (!row) {
-            br = sum3(Br, pb, ob + k);
-            bi = -sum3(Bi, pb, ob + k);
+    // eight neighbouring k of a plane a load (rows are multiples of 32 long)
+    auto add8 = [](const bf16 *p, float (&x)[8]) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[2 * i] += __uint_as_float(u[i] << 16);
+            x[2 * i + 1] += __uint_as_float(u[i] & 0xFFFF0000u);
         }
-        re += ar * br - ai * bi;
-        im += ar * bi + ai * br;
+    };
+    auto sum8 = [&](const bf16 *p, size_t plane, size_t at, float (&x)[8]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = 0.f;
+        add8(p + at, x);
+        add8(p + plane + at, x);
+        add8(p + 2 * plane + at, x);
+    };
+    for (int k = 8 * lane; k < kp; k += 256) {
+        float ar[8], ai[8];
+        sum8(Ar, pa, oa + k, ar);
+        sum8(Ai, pa, oa + k, ai);
+        if (row) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { re += ar[i]; im += ai[i]; }
+        } else {
+            float br[8], bi[8];
+            sum8(Br, pb, ob + k, br);
+            sum8(Bi, pb, ob + k, bi);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                re += ar[i] * br[i] + ai[i] * bi[i];
+                im += ai[i] * br[i] - ar[i] * bi[i];
+            }
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         re += __shfl_xor_sync(0xffffffffu, re, o);
@@ -776,7 +813,7 @@ cudaError_t launch_model_grid_comp(int n_comp, const double *comp_host, int stri
     e = launch_tc_pass<2>(a2, s);
     if (e != cudaSuccess || !a2.hermitian) return e;
     const int cells = n_grid + n_grid / 2 - 1;
-    comp_edge_kernel<<<(cells * 32 + 255) / 256, 256, 0, s>>>(Ar, Ai, Br, Bi, n_grid, kp, grid_out);
+    comp_edge_kernel<<<(cells * 32 + 127) / 128, 128, 0, s>>>(Ar, Ai, Br, Bi, n_grid, kp, grid_out);
     return cudaGetLastError();
 }
 
