@@ -349,7 +349,7 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * refused (PSC_ERR_ARG) unless every channel's aperture lies inside the
  * S x S tap window and consecutive time steps move a baseline by at most 4
  * grid cells at the highest frequency.  Results do not depend on the shape
- * beyond FP32 summation order.
+ * beyond FP32 rounding.
  * A context without a tiling (its current values then count as 32, 4, 1) picks its
  * launch shape by size: from two million visibilities on, flat bricks
  * (psc_set_flat_tiling) or, for small apertures and enough baselines, the track
@@ -393,7 +393,8 @@ psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread);
  * context uses the exact kernel, a residual-w stack or the BF16 grid copy, a
  * grid not 16-byte aligned, an aperture reaching outside the S x S window,
  * or (vis_per_lane 2) consecutive time steps more than 4 cells apart.
- * Results equal the brick kernel's up to FP32 summation order. */
+ * Results equal the brick kernel's up to FP32 rounding (positions, taps and sums
+ * are ordered differently; the phases are formed alike). */
 psc_status psc_set_track_tiling(psc_ctx *ctx, int vis_per_lane);
 
 /* Polls of one bounded mbarrier wait of the track kernel (psc_set_track_tiling),

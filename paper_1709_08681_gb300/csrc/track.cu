@@ -55,6 +55,7 @@ using namespace tap;
 constexpr int kTrkWarps = kTrkThreads / 32;
 constexpr int kBoxRows = 8;                 // rows of one TMA copy
 constexpr int kMaxBoxW = 32;                // widest staged box (cells)
+constexpr int kMaxBoxRows = 64;             // tallest: the tile in rows of 8
 constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kDrainPolls = 1LL << 26;
 
@@ -280,6 +281,7 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
     __shared__ __align__(8) unsigned long long s_mbar[kTrkWarps][2];
     __shared__ float s_mom[kTrkWarps][14][32];      // the lanes' running channel moments
     __shared__ float4 s_q[kTrkWarps][2][32];         // per lane: first (u, v) split; (du1, dv1, wv0, wv1)
+    __shared__ float2 s_ph[kTrkWarps][kMaxBoxW + kMaxBoxRows];   // per item: phasors of columns, then of rows
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool persistent = queue != nullptr;
     EvalArgs &a = s_args[warp];
@@ -302,6 +304,13 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
     long long first = 0;
     long long gi_static = (long long)blockIdx.x * kTrkWarps + warp;
     const float pi_f = 3.14159265358979f;
+    float2 *const col_ph = s_ph[warp], *const row_ph = col_ph + kMaxBoxW;
+    // exp(i pi x), as the brick kernel forms its phasors
+    auto phasor = [](float x) {
+        float sn, cs;
+        sincospif(x, &sn, &cs);
+        return make_float2(cs, sn);
+    };
 
     for (;;) {
         long long gi;
@@ -342,6 +351,16 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
         const float dL = (float)(li - lj), dM = (float)(mi - mj);     // decorrelation
         const int nt = a.nt, nc = a.nc, n_bl = a.n_bl, half = a.ng / 2;
         const float du = a.du, ov = (float)a.ov;
+        // The cell half of the ramp, exp(-i pi du (k L + r M)) at k columns and r rows from
+        // an origin, as a column's phasor times a row's, the same for every channel, like
+        // the brick kernel's.  Hardware sines and a step's phasor multiplied along the rows
+        // had an error common to a box, up to 8 times the brick kernel's in chi^2; exact
+        // ones take 17.83 ms where those took 17.42 (two LM iterations of 2 x 197
+        // antennas, 60 x 128; per channel instead of per item: 18.18)
+        __syncwarp();
+        col_ph[lane] = phasor(-du * ((float)lane * L));
+        for (int r = lane; r < kMaxBoxRows; r += 32) row_ph[r] = phasor(-du * ((float)r * M));
+        __syncwarp();
         const int tb = chunk * 32 * kV + lane * kV;
         // rows of the lane's visibilities in uvs (past the interval's end: the
         // last step again, with weight 0) and of their first channel in vis_obs
@@ -458,31 +477,25 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
             float2 S0[kV], Su[kV], Sv[kV];
 #pragma unroll
             for (int v = 0; v < kV; ++v) S0[v] = Su[v] = Sv[v] = make_float2(0.f, 0.f);
-            float parg[kV];                            // the visibility half of the ramp: its phase
+            float parg[kV];                            // the visibility half of the ramp: its phase / pi
             if (staged) {
-                // cell half of the ramp, in place: cell (col, r) *= exp(-i pi du (col L + r M))
+                // cell half of the ramp, in place, from the box corner
                 const int lw = W == 8 ? 3 : W == 16 ? 4 : 5;
                 const int col = lane & (W - 1);
                 const int rstep = 32 >> lw;
                 const int rows = box.y1 - box.y0 + 1;
                 if (col <= box.x1 - box.x0) {
                     int r = lane >> lw;
-                    float zs, zc, ss, sc;
-                    __sincosf(-pi_f * du * ((float)col * L + (float)r * M), &zs, &zc);
-                    __sincosf(-pi_f * du * ((float)rstep * M), &ss, &sc);
-                    float2 z = make_float2(zc, zs);
-                    const float2 stp = make_float2(sc, ss);
+                    const float2 zcol = col_ph[col];
                     uint32_t cell = tile + (uint32_t)(r * W + col) * 8u;
                     const uint32_t cstep = (uint32_t)(rstep * W) * 8u;
-                    for (; r < rows; r += rstep, cell += cstep) {
-                        sts_f2(cell, cmul(lds_f2(cell), z));
-                        z = cmul(z, stp);
-                    }
+                    for (; r < rows; r += rstep, cell += cstep)
+                        sts_f2(cell, cmul(lds_f2(cell), cmul(zcol, row_ph[r])));
                 }
                 __syncwarp();
 #pragma unroll
                 for (int v = 0; v < kV; ++v) {
-                    parg[v] = pi_f * du * (((float)(nx[v] - box.x0) + fx[v]) * L + ((float)(ny[v] - box.y0) + fy[v]) * M);
+                    parg[v] = du * (((float)(nx[v] - box.x0) + fx[v]) * L + ((float)(ny[v] - box.y0) + fy[v]) * M);
                 }
                 // The tap pattern, the same for every lane of the warp (no
                 // divergence, no per-lane spans): relative to the lane's base
@@ -562,14 +575,17 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
                     }
                 }
             } else {
-                // fallback: taps read the grid (L1/L2), ramp per tap from each
-                // visibility's own cell (nx, ny)
-                float zxs, zxc;
-                __sincosf(-pi_f * du * L, &zxs, &zxc);
-                const float2 zx = make_float2(zxc, zxs);
+                // fallback: taps read the grid (L1/L2); the ramp from each visibility's own
+                // cell (nx, ny), whose taps lie at most 31 columns and rows away (the
+                // apertures end inside a window of at most 64): those below by conjugates
+                auto ramp = [](const float2 *tab, int k) {
+                    float2 z = tab[abs(k)];
+                    z.y = k < 0 ? -z.y : z.y;
+                    return z;
+                };
 #pragma unroll
                 for (int v = 0; v < kV; ++v) {
-                    parg[v] = pi_f * du * (fx[v] * L + fy[v] * M);
+                    parg[v] = du * (fx[v] * L + fy[v] * M);
                     const int b_lo = max((int)floorf(fy[v] - rmax) + 1, -ny[v]);
                     const int b_hi = min((int)ceilf(fy[v] + rmax) - 1, a.ng - 1 - ny[v]);
                     for (int bb = b_lo; bb <= b_hi; ++bb) {
@@ -582,17 +598,13 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
                         if (a_lo > a_hi) continue;
                         const float dyo = dy * ov;
                         const float dyo2 = fmaf(dyo, dyo, 1e-20f);
-                        float zs, zc;
-                        __sincosf(-pi_f * du * ((float)a_lo * L + (float)bb * M), &zs, &zc);
-                        float2 z = make_float2(zc, zs);
                         float pr = 0.f, pi = 0.f, qr = 0.f, qi = 0.f;
                         const float2 *rowp = a.grid + (size_t)(ny[v] + bb) * a.ng + nx[v];
                         float dd = (fx[v] - (float)a_lo) * ov;
                         // unrolled: four grid loads in flight per lane instead of one
 #pragma unroll 4
                         for (int aa = a_lo; aa <= a_hi; ++aa, dd -= ov) {
-                            const float2 g = cmul(__ldg(&rowp[aa]), z);
-                            z = cmul(z, zx);
+                            const float2 g = cmul(__ldg(&rowp[aa]), ramp(col_ph, aa));
                             const float s2 = fmaf(dd, dd, dyo2);
                             const float tv = sqrt_fast(s2);
                             const float2 e = lds_f2(tab_addr(tab_adj, __fadd_rz(tv, 8388608.0f)));
@@ -603,10 +615,12 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
                             qr = fmaf(Ad, g.x, qr);
                             qi = fmaf(Ad, g.y, qi);
                         }
-                        S0[v].x += pr; S0[v].y += pi;
-                        Su[v].x += qr; Su[v].y += qi;
-                        Sv[v].x = fmaf(dy, pr, Sv[v].x);
-                        Sv[v].y = fmaf(dy, pi, Sv[v].y);
+                        const float2 py = ramp(row_ph, bb);
+                        const float2 P = cmul(make_float2(pr, pi), py), Q = cmul(make_float2(qr, qi), py);
+                        S0[v].x += P.x; S0[v].y += P.y;
+                        Su[v].x += Q.x; Su[v].y += Q.y;
+                        Sv[v].x = fmaf(dy, P.x, Sv[v].x);
+                        Sv[v].y = fmaf(dy, P.y, Sv[v].y);
                     }
                 }
             }
@@ -629,16 +643,14 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
             float D = 1.f, a2 = 0.f;
             if (a.decorrelation) {
                 a2 = ch.alpha2;
-                D = __expf(-0.5f * a2 * (dL * dL + dM * dM));
+                D = expf(-0.5f * a2 * (dL * dL + dM * dM));
             }
             const float su = pi_f * du / ov;         // Q was accumulated with dx ov; Px = i pi Tu
             const float sv = pi_f * du;
             float rr = 0.f, rt = 0.f, rx = 0.f, ry = 0.f, tt = 0.f, tx = 0.f, ty = 0.f, xx = 0.f, xy = 0.f, yy = 0.f;
 #pragma unroll
             for (int v = 0; v < kV; ++v) {
-                float s, co;
-                __sincosf(parg[v], &s, &co);
-                const float2 ph = make_float2(co, s);
+                const float2 ph = phasor(parg[v]);
                 const float2 T = cmul(ph, S0[v]);
                 const float2 U = cmul(ph, Su[v]), W2 = cmul(ph, Sv[v]);
                 const float2 Px = make_float2(-su * U.y, su * U.x);
