@@ -424,8 +424,10 @@ psc_status psc_fp32_fma_rate(double *tflops, void *stream);
  * of the pointing ramp applied) into shared memory when they fit a 64 x 64
  * tile, else reads them from global memory.  PSC_STAGE_NEVER: always read
  * from global memory (pays off for small apertures and long baselines, where
- * a brick's visibilities share few cells).  Results are the same up to FP32
- * summation order.  Errors: PSC_ERR_ARG for an unknown mode. */
+ * a brick's visibilities share few cells); a context without a tiling then runs
+ * the brick kernel.  The track kernel, once chosen by a call, stages its boxes in
+ * either mode.  Results are the same up to FP32
+ * rounding.  Errors: PSC_ERR_ARG for an unknown mode. */
 psc_status psc_set_staging(psc_ctx *ctx, int mode);
 
 /* Launch order of the fused kernel's bricks.  PSC_ORDER_BASELINE: baselines

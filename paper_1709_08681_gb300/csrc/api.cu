@@ -328,8 +328,10 @@ Shape brick_shape(const psc_ctx *c) {
 // brick, 8 x 64: 1660 with one against 3784; but 30 antennas, 20 x 16 (435 items):
 // 46 against 33.  Fast-moving baselines fall back to reading taps from the grid,
 // where the track kernel wins only in large arrays (197 antennas, 77 x 16: 2184
-// against 2918; 60 antennas: 346 against 299).
+// against 2918; 60 antennas: 346 against 299).  It stages its boxes, so a context that
+// asked for reads from global memory keeps the bricks.
 int want_track(const psc_ctx *c) {
+    if (c->no_stage) return 0;
     if (c->rho_top > 4.5 || (double)c->nt * c->n_bl * c->nc < kLargeVis) return 0;
     const int kv = c->nt > 32 && c->step_cells <= 0.5 ? 2 : 1;
     const long long items = (long long)c->n_bl * ((c->nt + 32 * kv - 1) / (32 * kv));
@@ -372,7 +374,7 @@ psc_status ensure_partials(psc_ctx *c, const Shape &s) {
     if (!c->trk_set) {
         Shape o = brick_shape(c);
         need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, o));
-        o.trk_kv = want_track(c) > 0 ? 1 : 0;                         // more records than two a lane
+        o.trk_kv = c->d_tmap ? 1 : 0;                                 // more records than two a lane
         need = std::max(need, (size_t)c->n_bl * (size_t)bricks_per_bl(c, o));
     }
     if (need <= c->partials_cap) return PSC_OK;
