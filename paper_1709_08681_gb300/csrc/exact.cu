@@ -514,24 +514,10 @@ cudaError_t launch_exact(const EvalArgs &a, bool predict, cudaStream_t s) {
     const int threads = ((a.flat > 0 ? a.flat : a.t_tile * a.c_group) + 31) / 32 * 32;
     const int blocks = (int)a.n_bricks;
     const size_t dyn = exact_dyn_smem(a.flat > 0 ? a.ch_span : a.c_group, a.tab_stride);
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = allow_smem(predict ? (const void *)exact_kernel<true> : (const void *)exact_kernel<false>, dyn);
     if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa{};
-    e = cudaFuncGetAttributes(&fa, predict ? exact_kernel<true> : exact_kernel<false>);
-    if (e != cudaSuccess) return e;
-    if (dyn + fa.sharedSizeBytes > (size_t)optin) return cudaErrorInvalidValue;
-    if (predict) {
-        e = cudaFuncSetAttribute(exact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        if (e != cudaSuccess) return e;
-        exact_kernel<true><<<blocks, threads, dyn, s>>>(a);
-    } else {
-        e = cudaFuncSetAttribute(exact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        if (e != cudaSuccess) return e;
-        exact_kernel<false><<<blocks, threads, dyn, s>>>(a);
-    }
+    if (predict) exact_kernel<true><<<blocks, threads, dyn, s>>>(a);
+    else exact_kernel<false><<<blocks, threads, dyn, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -458,8 +458,7 @@ size_t stencil_dyn_smem(const StencilArgs &a, int threads) {
 cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *prefix_dev, const FeatPair *pairs_dev,
                                   int n, long long total_blocks, int threads, size_t dyn, int max_bl, int max_ant,
                                   bool direct, float sigma, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(stencil_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(dyn > 48 * 1024 ? dyn : 48 * 1024));
+    cudaError_t e = allow_smem((const void *)stencil_batch_kernel, dyn);
     if (e != cudaSuccess) return e;
     if (total_blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     stencil_batch_kernel<<<(unsigned)total_blocks, threads, dyn, s>>>(args_dev, prefix_dev, n);
@@ -478,8 +477,7 @@ cudaError_t launch_features_batch(const StencilArgs *args_dev, const long long *
 cudaError_t launch_features(const StencilArgs &a, double *blsum, int n_ant, float *feat, cudaStream_t s) {
     const int threads = a.wpb > 1 ? 32 * a.wpb : (a.t_tile * a.c_group + 31) / 32 * 32;
     const size_t dyn = stencil_dyn_smem(a, threads);
-    cudaError_t e = cudaFuncSetAttribute(stencil_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(dyn > 48 * 1024 ? dyn : 48 * 1024));
+    cudaError_t e = allow_smem((const void *)stencil_kernel, dyn);
     if (e != cudaSuccess) return e;
     stencil_kernel<<<(int)((a.n_bricks + a.wpb - 1) / a.wpb), threads, dyn, s>>>(a);
     e = cudaGetLastError();

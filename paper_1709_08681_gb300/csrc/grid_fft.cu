@@ -404,7 +404,7 @@ cudaError_t fft_launch(const FftPlan &p, int n_img, const float *image, float2 *
     const size_t smem = buf_bytes(p.n);
     const int threads = std::max(64, ((p.n + kE - 1) / kE + 31) / 32 * 32);
     for (const void *k : {(const void *)fft_cols_kernel<k16, kPow2>, (const void *)fft_rows_kernel<k16, kPow2>}) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(k, smem);
         if (e != cudaSuccess) return e;
     }
     if (!kPow2) fft_twiddle_kernel<<<(p.tw_len + 127) / 128, 128, 0, s>>>(p, tw);

@@ -179,6 +179,22 @@ cudaError_t launch_uvw(const double *enu_dev, int n_ant, double lat, double dec,
 constexpr int kCtxSlots = 16;
 int context_slot();
 
+// Raises a kernel's dynamic shared memory limit to the most that it can have, and
+// refuses more.  The limit belongs to the kernel in its CUDA context, not to a launch:
+// set to each launch's own size, another thread's (or another context's) smaller launch
+// could lower it before this one ran.
+inline cudaError_t allow_smem(const void *kernel, size_t dyn) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa{};
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)fa.sharedSizeBytes;
+    if (most < 0 || dyn > (size_t)most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Launchers (defined in the .cu files).
 cudaError_t launch_eval(const EvalArgs &a, bool predict, cudaStream_t s);
 // Persistent fused launch over several contexts (device arrays of EvalArgs and

@@ -771,7 +771,7 @@ size_t track_dyn_smem(int cap, int tabc) {
 
 cudaError_t set_track_smem(size_t dyn) {
     for (const void *k : {(const void *)track_kernel<1>, (const void *)track_kernel<2>}) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        cudaError_t e = allow_smem(k, dyn);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
