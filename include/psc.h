@@ -353,7 +353,7 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * A context without a tiling (its current values then count as 32, 4, 1) picks its
  * launch shape by size: from two million visibilities on, flat bricks
  * (psc_set_flat_tiling) or, for small apertures and enough baselines, the track
- * kernel (psc_set_track_tiling; in a batch only if no context has a tiling); below, the
+ * kernel (psc_set_track_tiling); below, the
  * rectangle (32, 4, 1), with the rows of each visibility shared among lanes where
  * there are too few visibilities to fill the chip (the same sums bit for bit). */
 psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thread);
@@ -557,13 +557,18 @@ psc_status psc_learned_init(psc_ctx *ctx, psc_mlp *m, const void *vis_obs, const
 /* ---- Batches of solution intervals (Algorithm 1's loop over all data) ----
  * A batch groups contexts -- normally one per solution interval, of any
  * array, length and channel set -- with their observed data, so that one LM
- * iteration of all of them is one persistent fused launch: thread blocks pull
- * (baseline, channel group, time tile) bricks of every context from one
- * device work queue, so intervals of uneven size share the GPU.  The
+ * iteration of all of them is one persistent fused launch for each fused kernel
+ * that they run (the brick kernel, the track kernel with one and with two
+ * visibilities per lane): thread blocks pull the bricks or items of its contexts
+ * from one device work queue, so intervals of uneven size share the GPU.  A context
+ * without a tiling runs the kernel that it runs alone, and its results do not
+ * depend on what else the batch holds; one that was given the track kernel
+ * (psc_set_track_tiling) goes with contexts of the same track tiling only
+ * (PSC_ERR_ARG).  The
  * reductions and the LM updates of all contexts follow as one launch each,
  * and the iteration is captured once in a CUDA graph and replayed (unless the
  * batch runs on the legacy NULL stream).  Contexts whose solver stopped skip
- * their bricks.  The persistent launch uses the block size of the widest
+ * their bricks.  The brick kernel's launch uses the block size of the widest
  * context's shape (t_tile * c_group rounded up to a multiple of 32); narrower
  * contexts leave the extra lanes idle.
  * The contexts must all use the Gaussian kernel model, and either all read
@@ -582,8 +587,8 @@ const char *psc_batch_last_error(const psc_batch *b);
 
 /* Name of the fused kernel that the batch's persistent launch runs
  * ("eval_kernel<...>" for brick tilings, "track_kernel<kv>" when every
- * context runs the track kernel; a batch without tilings may run some of its
- * contexts in a second launch of that kernel).  Static storage; never NULL. */
+ * context runs the track kernel; contexts without tilings may run in further
+ * launches of that kernel).  Static storage; never NULL. */
 const char *psc_batch_kernel(const psc_batch *b);
 
 /* Picks each context's launch shape by timing the fused kernel on its own

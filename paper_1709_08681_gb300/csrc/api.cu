@@ -1505,13 +1505,15 @@ struct psc_batch {
     std::vector<double> w_scale;
     // device tables (rebuilt by build_tables)
     EvalArgs *d_eval = nullptr;
-    long long *d_prefix = nullptr;   // bricks before each context, then (n + 1 on) track items before each
+    // bricks before each context [n + 1], then track items before each with one and with
+    // two visibilities per lane
+    long long *d_prefix = nullptr;
     RedArgs *d_red = nullptr;
     int *d_bl_prefix = nullptr;
     LMArgs *d_lm = nullptr;
     const LMState **d_st0 = nullptr;
     const double **d_lm0 = nullptr;
-    unsigned long long *d_queue = nullptr;   // of the brick and of the track kernel
+    unsigned long long *d_queue = nullptr;   // [3] of the bricks and the two track launches
     int *d_active = nullptr;
     // psc_batch_end: every context's offsets, solver state and wait flag
     // gathered on the device ([lm 2n_ant...][state...][flag...]) and copied
@@ -1521,13 +1523,14 @@ struct psc_batch {
     std::vector<size_t> lm_off;
     int total_bl = 0;
     int max_ant = 0, max_bpb = 0;    // most antennas of a context, most records of a baseline
-    int grid = 0, trk_grid = 0;
+    int grid = 0;
     bool bricks = false;         // some context runs the brick kernel
     int threads = 128;           // brick-kernel block size: the widest context's shape
     bool split = false;          // some context shares its visibilities among lanes
     bool stacked = false;        // every context reads a residual-w stack (else none does)
-    int track = 0;               // > 0: some context runs the track kernel, this many visibilities per lane
-    int trk_tabc = 0;            // track kernel: table capacity of a warp buffer (entries)
+    // the track launches with one and two visibilities per lane (index 0 unused):
+    // blocks (0: no such context) and table capacity of a warp buffer (entries)
+    int trk_grid[3] = {0, 0, 0}, trk_tabc[3] = {0, 0, 0};
     size_t eval_dyn = 0, lm_dyn = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1575,7 +1578,7 @@ void free_batch(psc_batch *b) {
 psc_status build_tables(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     std::vector<EvalArgs> ev(n);
-    std::vector<long long> prefix(2 * (n + 1), 0);
+    std::vector<long long> prefix(3 * (n + 1), 0);
     std::vector<RedArgs> red(n);
     std::vector<int> blp(n + 1, 0);
     std::vector<LMArgs> lm(n);
@@ -1583,22 +1586,24 @@ psc_status build_tables(psc_batch *b) {
     std::vector<const double *> lm0(n);
     size_t dyn = 0, lmd = 0;
     int threads = 32, max_ant = 0, max_bpb = 0;
-    // Where no context has a tiling, each takes its own kernel (two persistent launches
-    // an iteration; one for 27 to 197 antennas, 38 to 411 x 16, took 5.7 ms of bricks
-    // against 4.6 in both), all of the track kernel with the fewest visibilities per
-    // lane among them; one fused kernel serves a batch with tilings.
-    bool any_set = false;
-    int kv_auto = 2;
+    // One fused kernel for the contexts that were given the track kernel and those beside them
+    int n_trk = 0;
+    bool same = true;
     for (psc_ctx *c : b->ctxs) {
-        any_set = any_set || c->trk_set;
-        if (auto_track(c) > 0) kv_auto = std::min(kv_auto, auto_track(c));
+        n_trk += c->trk_kv > 0;
+        same = same && c->trk_kv == b->ctxs[0]->trk_kv;
     }
+    if (n_trk > 0 && !same)
+        return bfail(b, PSC_ERR_ARG, "a batch runs one fused kernel: give every context the same track tiling, or none");
+    // Contexts without a tiling take the kernel that they take alone, whatever is beside
+    // them: up to three persistent launches an iteration (one for 27 to 197 antennas,
+    // 38 to 411 x 16, took 5.7 ms of bricks against 4.6 in two).
     bool split = false, bricks = false;
+    int tabc[3] = {0, 0, 0};
     std::vector<Shape> shapes(n);
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
-        shapes[k] = brick_shape(c);
-        shapes[k].trk_kv = c->trk_set ? c->trk_kv : !any_set && auto_track(c) > 0 ? kv_auto : 0;
+        shapes[k] = eval_shape(c);
         const Shape &shape = shapes[k];
         psc_status st = ensure_partials(c, shape);
         if (st == PSC_OK && shape.trk_kv > 0) st = trk_prepare(c);
@@ -1609,8 +1614,11 @@ psc_status build_tables(psc_batch *b) {
         ev[k].w_scale = (float)b->w_scale[k];
         ev[k].skip = c->d_done;
         const bool trk = shape.trk_kv > 0;
-        prefix[k + 1] = prefix[k] + (trk ? 0 : ev[k].n_bricks);
-        prefix[n + 2 + k] = prefix[n + 1 + k] + (trk ? ev[k].n_bricks : 0);
+        for (int q = 0; q < 3; ++q) {
+            long long *p = prefix.data() + q * (n + 1) + k;
+            p[1] = p[0] + (shape.trk_kv == q ? ev[k].n_bricks : 0);
+        }
+        if (trk) tabc[shape.trk_kv] = std::max(tabc[shape.trk_kv], ev[k].trk_tabc);
         red[k] = red_args(c, shape, c->d_ev, c->d_done);
         blp[k + 1] = blp[k] + c->n_bl;
         lm[k] = lm_args(c);
@@ -1632,46 +1640,35 @@ psc_status build_tables(psc_batch *b) {
     b->max_bpb = max_bpb;
     b->eval_dyn = dyn;
     b->lm_dyn = lmd;
-    // with tilings: the track kernel for all contexts (same visibilities per lane) or for none
-    int n_trk = 0, kv_trk = 0, tabc = 0;
-    for (int k = 0; k < n; ++k) {
-        const int kv = shapes[k].trk_kv;
-        if (kv <= 0) continue;
-        ++n_trk;
-        if (kv_trk && kv_trk != kv) kv_trk = -1;
-        else if (kv_trk == 0) kv_trk = kv;
-        tabc = std::max(tabc, ev[k].trk_tabc);
-    }
-    if (any_set && n_trk != 0 && (n_trk != n || kv_trk < 0))
-        return bfail(b, PSC_ERR_ARG, "a batch runs one fused kernel: give every context the same track tiling, or none");
-    b->track = n_trk ? kv_trk : 0;
-    b->trk_tabc = tabc;
-    int per_sm = 0, trk_per_sm = 0, dev = 0, n_sm = 0;
+    int per_sm = 0, dev = 0, n_sm = 0;
+    PSC_BCUDA(b, cudaGetDevice(&dev));
+    PSC_BCUDA(b, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     b->stacked = b->ctxs[0]->wp_n > 0;
     b->split = split;
     b->bricks = bricks;
-    if (b->track) {
-        const size_t tdyn = track_dyn_smem(kTrkCap, tabc);
+    for (int kv = 1; kv <= 2; ++kv) {
+        b->trk_tabc[kv] = tabc[kv];
+        b->trk_grid[kv] = 0;
+        if (!tabc[kv]) continue;
+        const size_t tdyn = track_dyn_smem(kTrkCap, tabc[kv]);
         PSC_BCUDA(b, set_track_smem(tdyn));
-        PSC_BCUDA(b, track_occupancy(b->track, tdyn, &trk_per_sm));
+        PSC_BCUDA(b, track_occupancy(kv, tdyn, &per_sm));
+        b->trk_grid[kv] = std::max(1, per_sm) * n_sm;
     }
     if (bricks) {
         PSC_BCUDA(b, set_eval_smem(dyn - eval_stack_smem(b->ctxs[0]->wp_n)));
         PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, b->split, &per_sm));
+        b->grid = std::max(1, per_sm) * n_sm;
     }
-    PSC_BCUDA(b, cudaGetDevice(&dev));
-    PSC_BCUDA(b, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-    b->grid = std::max(1, per_sm) * n_sm;
-    b->trk_grid = std::max(1, trk_per_sm) * n_sm;
     if (!b->d_eval) {
         PSC_BCUDA(b, dalloc(&b->d_eval, n));
-        PSC_BCUDA(b, dalloc(&b->d_prefix, 2 * (n + 1)));
+        PSC_BCUDA(b, dalloc(&b->d_prefix, 3 * (n + 1)));
         PSC_BCUDA(b, dalloc(&b->d_red, n));
         PSC_BCUDA(b, dalloc(&b->d_bl_prefix, n + 1));
         PSC_BCUDA(b, dalloc(&b->d_lm, n));
         PSC_BCUDA(b, dalloc(&b->d_st0, n));
         PSC_BCUDA(b, dalloc(&b->d_lm0, n));
-        PSC_BCUDA(b, dalloc(&b->d_queue, 2));
+        PSC_BCUDA(b, dalloc(&b->d_queue, 3));
         PSC_BCUDA(b, dalloc(&b->d_active, 1));
     }
     cudaStream_t s = b->stream;
@@ -1691,9 +1688,10 @@ psc_status build_tables(psc_batch *b) {
 psc_status launch_fused(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
-    if (b->track)
-        PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix + n + 1, n, b->d_queue + 1, b->track, kTrkCap, b->trk_tabc,
-                                        b->trk_grid, s));
+    for (int kv = 1; kv <= 2; ++kv)
+        if (b->trk_grid[kv] > 0)
+            PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix + kv * (n + 1), n, b->d_queue + kv, kv, kTrkCap,
+                                            b->trk_tabc[kv], b->trk_grid[kv], s));
     if (b->bricks)
         PSC_BCUDA(b, launch_eval_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->threads, b->eval_dyn, b->grid,
                                        b->stacked, b->split, s));
@@ -1704,7 +1702,7 @@ psc_status launch_fused(psc_batch *b) {
 psc_status enqueue_iteration(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
-    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(unsigned long long), s));
+    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, 3 * sizeof(unsigned long long), s));
     if (b->prof) {
         while (b->ev_pool.size() < b->ev_used + 2) {
             cudaEvent_t e;
@@ -2024,7 +2022,7 @@ psc_status psc_batch_autotune(psc_batch *b, int *tiling_out) {
             float ms = 0.f;
             for (int r = 0; r < 2 && st == PSC_OK; ++r) {             // warm, then timed
                 if (r == 1) e = cudaEventRecord(e0, b->stream);
-                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, 2 * sizeof(unsigned long long), b->stream);
+                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, 3 * sizeof(unsigned long long), b->stream);
                 if (e == cudaSuccess) st = launch_fused(b);
                 if (r == 1 && e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             }
@@ -2196,8 +2194,8 @@ const char *psc_batch_last_error(const psc_batch *b) { return b ? b->err.c_str()
 
 const char *psc_batch_kernel(const psc_batch *b) {
     if (!b) return "";
-    if (b->track == 2 && !b->bricks) return "track_kernel<2>";
-    if (b->track == 1 && !b->bricks) return "track_kernel<1>";
+    if (b->trk_grid[2] && !b->bricks) return "track_kernel<2>";
+    if (b->trk_grid[1] && !b->bricks) return "track_kernel<1>";
     return b->stacked ? "eval_kernel<false, true>" : "eval_kernel<false, false>";
 }
 

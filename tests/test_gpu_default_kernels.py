@@ -1,13 +1,15 @@
 """Which fused kernel a context without a tiling runs, and that nothing else decides its
-results' bits: not the staging mode's staged kernels where staging was refused."""
+results' bits: not the staging mode's staged kernels where staging was refused, and not
+what else a batch holds (other contexts without a tiling, or contexts with one)."""
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 # (antennas, time steps, channels, hours): the track kernel with one and two
-# visibilities per lane
+# visibilities per lane, flat bricks, the rectangle, rows shared among lanes
 ONE, TWO = (64, 20, 50, 0.02), (60, 45, 26, 0.05)
+FLAT, RECT, SHARED = (12, 480, 64, 4.0), (20, 60, 8, 0.05), (6, 20, 4, 0.05)
 
 
 def _problem(n_ant, nt, nc, span):
@@ -44,3 +46,40 @@ def test_unstaged_contexts_keep_the_bricks(shape, name):
     gp.ctx.psc_set_track_tiling(0)                    # the brick kernel, by a call
     brick = gp.ctx.psc_residual_grad(lm, vis, None, 1e6, cross=True)
     assert auto[0] == brick[0] and all(np.array_equal(x, y) for x, y in zip(auto[1:], brick[1:]))
+
+
+def _offsets(probs):
+    b = _batch(probs)
+    b.psc_batch_begin([np.zeros((gp.m.n_ant, 2)) for gp, _ in probs])
+    b.psc_batch_iterate(2)
+    lms, _ = b.psc_batch_end()
+    b.close()
+    return lms
+
+
+def _alone(gp, vis):
+    """The same two iterations without a batch."""
+    gp.ctx.psc_lm_begin(np.zeros((gp.m.n_ant, 2)))
+    gp.ctx.psc_lm_iterate(vis, None, 1e6, 2)
+    return gp.ctx.psc_lm_end()[0]
+
+
+# "set": a context that was given the rectangle (32, 4, 1) by a call
+@pytest.mark.parametrize("shapes", [(ONE, TWO), (TWO, ONE, SHARED), (TWO, "set"), ("set", ONE, FLAT, RECT)])
+def test_a_batch_does_not_change_its_contexts(shapes):
+    probs = [_problem(*(RECT if s == "set" else s)) for s in shapes]
+    for (gp, _), s in zip(probs, shapes):
+        if s == "set":
+            gp.ctx.psc_set_tiling(32, 4, 1)
+    for lm, (gp, vis) in zip(_offsets(probs), probs):
+        assert np.array_equal(lm, _offsets([(gp, vis)])[0])
+        assert np.array_equal(lm, _alone(gp, vis))
+
+
+def test_batches_refuse_contexts_beside_the_track_tiling():
+    from paper_1709_08681_gb300 import _abi
+    probs = [_problem(*s) for s in (ONE, TWO)]
+    probs[1][0].ctx.psc_set_track_tiling(2)                   # ONE's context runs the track kernel, but not by a call
+    with pytest.raises(_abi.PscError) as e:
+        _batch(probs)
+    assert e.value.status == _abi.PSC_ERR_ARG
