@@ -585,10 +585,10 @@ psc_status psc_batch_create(psc_batch **out, psc_ctx *const *ctxs, int n_ctx, co
 void psc_batch_destroy(psc_batch *b);
 const char *psc_batch_last_error(const psc_batch *b);
 
-/* Name of the fused kernel that the batch's persistent launch runs
- * ("eval_kernel<...>" for brick tilings, "track_kernel<kv>" when every
- * context runs the track kernel; contexts without tilings may run in further
- * launches of that kernel).  Static storage; never NULL. */
+/* Names of the fused kernels that the batch's persistent launches run, joined by
+ * " + ": "eval_kernel<false, stacked, shared>" (bricks, of a residual-w stack, with
+ * rows shared among lanes), then "track_kernel<vis_per_lane>".  Static storage; never
+ * NULL. */
 const char *psc_batch_kernel(const psc_batch *b);
 
 /* Picks each context's launch shape by timing the fused kernel on its own

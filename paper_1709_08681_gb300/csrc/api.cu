@@ -2193,10 +2193,20 @@ psc_status psc_solve_batch(psc_ctx *const *ctxs, int n_ctx, const void *const *v
 const char *psc_batch_last_error(const psc_batch *b) { return b ? b->err.c_str() : g_err.c_str(); }
 
 const char *psc_batch_kernel(const psc_batch *b) {
+    static const char *const part[] = {"eval_kernel<false, false, false>", "eval_kernel<false, true, false>",
+                                       "eval_kernel<false, false, true>", "track_kernel<1>", "track_kernel<2>"};
+    static const std::array<std::string, 32> names = [] {       // every set of them
+        std::array<std::string, 32> s;
+        for (int set = 0; set < 32; ++set)
+            for (int k = 0; k < 5; ++k)
+                if (set >> k & 1) s[set] += (s[set].empty() ? "" : " + ") + std::string(part[k]);
+        return s;
+    }();
     if (!b) return "";
-    if (b->trk_grid[2] && !b->bricks) return "track_kernel<2>";
-    if (b->trk_grid[1] && !b->bricks) return "track_kernel<1>";
-    return b->stacked ? "eval_kernel<false, true>" : "eval_kernel<false, false>";
+    int set = b->trk_grid[1] ? 8 : 0;
+    if (b->trk_grid[2]) set |= 16;
+    if (b->bricks) set |= b->stacked ? 2 : b->split ? 4 : 1;
+    return names[set].c_str();
 }
 
 psc_status psc_batch_profile(psc_batch *b, int enable) {

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 # (antennas, time steps, channels, hours): the track kernel with one and two
 # visibilities per lane, flat bricks, the rectangle, rows shared among lanes
 ONE, TWO = (64, 20, 50, 0.02), (60, 45, 26, 0.05)
-FLAT, RECT, SHARED = (12, 480, 64, 4.0), (20, 60, 8, 0.05), (6, 20, 4, 0.05)
+FLAT, RECT, SHARED = (12, 480, 64, 4.0), (24, 60, 12, 0.05), (6, 20, 4, 0.05)
 
 
 def _problem(n_ant, nt, nc, span):
@@ -18,7 +18,7 @@ def _problem(n_ant, nt, nc, span):
     from gpu_cases import GpuProblem
     m, _, _, img = cases.problem(("disk", 512, 5.0, 1024), n_ant=3, n_time=1, freqs=(1.2e9,))
     m.uvw_m, m.freq_hz = cases.geometry(n_ant, 300.0, nt, span, tuple(np.linspace(1.2e9, 1.6e9, nc)))
-    m.n_ant, m.diam_m = n_ant, 8.0
+    m.n_ant, m.diam_m = n_ant, 25.0
     gp = GpuProblem(m, img)
     vis = torch.empty(gp.shape, dtype=torch.complex64, device="cuda")
     gp.ctx.psc_predict(np.random.default_rng(n_ant).normal(0, 1e-4, (n_ant, 2)), vis, None)
@@ -83,3 +83,16 @@ def test_batches_refuse_contexts_beside_the_track_tiling():
     with pytest.raises(_abi.PscError) as e:
         _batch(probs)
     assert e.value.status == _abi.PSC_ERR_ARG
+
+
+BRICKS, SHARED_ROWS = "eval_kernel<false, false, false>", "eval_kernel<false, false, true>"
+
+
+@pytest.mark.parametrize("shapes,name", [
+    ((ONE, TWO), "track_kernel<1> + track_kernel<2>"), ((FLAT, TWO), BRICKS + " + track_kernel<2>"),
+    ((RECT, FLAT), BRICKS), ((SHARED, SHARED), SHARED_ROWS),
+])
+def test_the_kernels_of_a_batch_by_name(shapes, name):
+    b = _batch([_problem(*s) for s in shapes])
+    assert b.psc_batch_kernel() == name
+    b.close()
