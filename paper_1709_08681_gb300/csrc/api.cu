@@ -1497,6 +1497,12 @@ psc_status psc_profile_read(psc_ctx *ctx, double *total_ms, int *n_launches) {
 // ---------------------------------------------------------------------------
 // Batches of contexts: one persistent fused launch per LM iteration.
 
+namespace {
+// A batch's fused kernels (psc_batch::fused).
+constexpr int kBricks = 0, kTrack1 = 1, kTrack2 = 2, kShared = 3, kFused = 4;
+int fused_of(const Shape &s) { return s.trk_kv > 0 ? kTrack1 + s.trk_kv - 1 : s.split > 1 ? kShared : kBricks; }
+}  // namespace
+
 struct psc_batch {
     cudaStream_t stream = nullptr;
     std::vector<psc_ctx *> ctxs;
@@ -1505,15 +1511,13 @@ struct psc_batch {
     std::vector<double> w_scale;
     // device tables (rebuilt by build_tables)
     EvalArgs *d_eval = nullptr;
-    // bricks before each context [n + 1], then track items before each with one and with
-    // two visibilities per lane
-    long long *d_prefix = nullptr;
+    long long *d_prefix = nullptr;   // [kFused][n + 1] bricks or items before each context
     RedArgs *d_red = nullptr;
     int *d_bl_prefix = nullptr;
     LMArgs *d_lm = nullptr;
     const LMState **d_st0 = nullptr;
     const double **d_lm0 = nullptr;
-    unsigned long long *d_queue = nullptr;   // [3] of the bricks and the two track launches
+    unsigned long long *d_queue = nullptr;   // [kFused]
     int *d_active = nullptr;
     // psc_batch_end: every context's offsets, solver state and wait flag
     // gathered on the device ([lm 2n_ant...][state...][flag...]) and copied
@@ -1523,15 +1527,20 @@ struct psc_batch {
     std::vector<size_t> lm_off;
     int total_bl = 0;
     int max_ant = 0, max_bpb = 0;    // most antennas of a context, most records of a baseline
-    int grid = 0;
-    bool bricks = false;         // some context runs the brick kernel
-    int threads = 128;           // brick-kernel block size: the widest context's shape
-    bool split = false;          // some context shares its visibilities among lanes
     bool stacked = false;        // every context reads a residual-w stack (else none does)
-    // the track launches with one and two visibilities per lane (index 0 unused):
-    // blocks (0: no such context) and table capacity of a warp buffer (entries)
-    int trk_grid[3] = {0, 0, 0}, trk_tabc[3] = {0, 0, 0};
-    size_t eval_dyn = 0, lm_dyn = 0;
+    // The persistent launches of an iteration, by fused kernel: bricks, the track kernel
+    // with one and with two visibilities per lane, and bricks whose visibilities' rows
+    // are shared among lanes (apart, as that kernel's registers and shared memory would
+    // slow the others: 16 intervals of 27 antennas, 60 x 16, beside one of 60 x 1 took
+    // 3279 us an iteration in one launch, 2428 in two and 2357 without it; where little is
+    // beside it, the second launch's tail costs more: 792 and 823 with one of 150 x 64).
+    struct Fused {
+        int grid = 0;            // blocks; 0: no context runs it
+        int threads = 32;        // bricks: the widest context's shape
+        size_t dyn = 0;          // bricks: dynamic shared memory
+        int tabc = 0;            // track kernel: table capacity of a warp buffer (entries)
+    } fused[kFused];
+    size_t lm_dyn = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     // fused-kernel timing (psc_batch_profile): direct launches with event pairs
@@ -1578,14 +1587,15 @@ void free_batch(psc_batch *b) {
 psc_status build_tables(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     std::vector<EvalArgs> ev(n);
-    std::vector<long long> prefix(3 * (n + 1), 0);
+    std::vector<long long> prefix(kFused * (n + 1), 0);
     std::vector<RedArgs> red(n);
     std::vector<int> blp(n + 1, 0);
     std::vector<LMArgs> lm(n);
     std::vector<const LMState *> st0(n);
     std::vector<const double *> lm0(n);
-    size_t dyn = 0, lmd = 0;
-    int threads = 32, max_ant = 0, max_bpb = 0;
+    size_t lmd = 0;
+    int max_ant = 0, max_bpb = 0;
+    psc_batch::Fused fused[kFused];
     // One fused kernel for the contexts that were given the track kernel and those beside them
     int n_trk = 0;
     bool same = true;
@@ -1596,10 +1606,8 @@ psc_status build_tables(psc_batch *b) {
     if (n_trk > 0 && !same)
         return bfail(b, PSC_ERR_ARG, "a batch runs one fused kernel: give every context the same track tiling, or none");
     // Contexts without a tiling take the kernel that they take alone, whatever is beside
-    // them: up to three persistent launches an iteration (one for 27 to 197 antennas,
+    // them: up to kFused persistent launches an iteration (one for 27 to 197 antennas,
     // 38 to 411 x 16, took 5.7 ms of bricks against 4.6 in two).
-    bool split = false, bricks = false;
-    int tabc[3] = {0, 0, 0};
     std::vector<Shape> shapes(n);
     for (int k = 0; k < n; ++k) {
         psc_ctx *c = b->ctxs[k];
@@ -1613,62 +1621,58 @@ psc_status build_tables(psc_batch *b) {
         ev[k].w = b->w[k];
         ev[k].w_scale = (float)b->w_scale[k];
         ev[k].skip = c->d_done;
-        const bool trk = shape.trk_kv > 0;
-        for (int q = 0; q < 3; ++q) {
+        const int kind = fused_of(shape);
+        for (int q = 0; q < kFused; ++q) {
             long long *p = prefix.data() + q * (n + 1) + k;
-            p[1] = p[0] + (shape.trk_kv == q ? ev[k].n_bricks : 0);
+            p[1] = p[0] + (kind == q ? ev[k].n_bricks : 0);
         }
-        if (trk) tabc[shape.trk_kv] = std::max(tabc[shape.trk_kv], ev[k].trk_tabc);
+        psc_batch::Fused &f = fused[kind];
+        f.grid = 1;
+        f.tabc = std::max(f.tabc, ev[k].trk_tabc);
+        f.threads = std::max(f.threads, eval_threads(shape));
+        if (shape.trk_kv == 0)
+            f.dyn = std::max(f.dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) +
+                                        eval_split_smem(shape.split, c->gd.support) + eval_stack_smem(c->wp_n));
         red[k] = red_args(c, shape, c->d_ev, c->d_done);
         blp[k + 1] = blp[k] + c->n_bl;
         lm[k] = lm_args(c);
         st0[k] = c->d_state0;
         lm0[k] = c->d_lm0;
-        if (!trk) {
-            bricks = true;
-            split = split || shape.split > 1;
-            threads = std::max(threads, eval_threads(shape));
-            dyn = std::max(dyn, eval_dyn_smem(ch_span(c, shape), tab_stride(c, shape.kv)) + eval_split_smem(shape.split, c->gd.support) + eval_stack_smem(c->wp_n));
-        }
         lmd = std::max(lmd, lm_smem_bytes(c->n_ant));
         max_ant = std::max(max_ant, c->n_ant);
         max_bpb = std::max(max_bpb, red[k].bpb);
     }
     b->total_bl = blp[n];
-    b->threads = threads;
     b->max_ant = max_ant;
     b->max_bpb = max_bpb;
-    b->eval_dyn = dyn;
     b->lm_dyn = lmd;
     int per_sm = 0, dev = 0, n_sm = 0;
     PSC_BCUDA(b, cudaGetDevice(&dev));
     PSC_BCUDA(b, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     b->stacked = b->ctxs[0]->wp_n > 0;
-    b->split = split;
-    b->bricks = bricks;
-    for (int kv = 1; kv <= 2; ++kv) {
-        b->trk_tabc[kv] = tabc[kv];
-        b->trk_grid[kv] = 0;
-        if (!tabc[kv]) continue;
-        const size_t tdyn = track_dyn_smem(kTrkCap, tabc[kv]);
-        PSC_BCUDA(b, set_track_smem(tdyn));
-        PSC_BCUDA(b, track_occupancy(kv, tdyn, &per_sm));
-        b->trk_grid[kv] = std::max(1, per_sm) * n_sm;
+    for (int q = 0; q < kFused; ++q) {
+        psc_batch::Fused &f = fused[q];
+        if (f.grid == 0) continue;
+        if (q == kTrack1 || q == kTrack2) {
+            const size_t tdyn = track_dyn_smem(kTrkCap, f.tabc);
+            PSC_BCUDA(b, set_track_smem(tdyn));
+            PSC_BCUDA(b, track_occupancy(q == kTrack1 ? 1 : 2, tdyn, &per_sm));
+        } else {
+            PSC_BCUDA(b, set_eval_smem(f.dyn - eval_stack_smem(b->ctxs[0]->wp_n)));
+            PSC_BCUDA(b, eval_batch_occupancy(f.threads, f.dyn, b->stacked, q == kShared, &per_sm));
+        }
+        f.grid = std::max(1, per_sm) * n_sm;
     }
-    if (bricks) {
-        PSC_BCUDA(b, set_eval_smem(dyn - eval_stack_smem(b->ctxs[0]->wp_n)));
-        PSC_BCUDA(b, eval_batch_occupancy(b->threads, dyn, b->stacked, b->split, &per_sm));
-        b->grid = std::max(1, per_sm) * n_sm;
-    }
+    std::copy(fused, fused + kFused, b->fused);
     if (!b->d_eval) {
         PSC_BCUDA(b, dalloc(&b->d_eval, n));
-        PSC_BCUDA(b, dalloc(&b->d_prefix, 3 * (n + 1)));
+        PSC_BCUDA(b, dalloc(&b->d_prefix, kFused * (n + 1)));
         PSC_BCUDA(b, dalloc(&b->d_red, n));
         PSC_BCUDA(b, dalloc(&b->d_bl_prefix, n + 1));
         PSC_BCUDA(b, dalloc(&b->d_lm, n));
         PSC_BCUDA(b, dalloc(&b->d_st0, n));
         PSC_BCUDA(b, dalloc(&b->d_lm0, n));
-        PSC_BCUDA(b, dalloc(&b->d_queue, 3));
+        PSC_BCUDA(b, dalloc(&b->d_queue, kFused));
         PSC_BCUDA(b, dalloc(&b->d_active, 1));
     }
     cudaStream_t s = b->stream;
@@ -1688,13 +1692,16 @@ psc_status build_tables(psc_batch *b) {
 psc_status launch_fused(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
-    for (int kv = 1; kv <= 2; ++kv)
-        if (b->trk_grid[kv] > 0)
-            PSC_BCUDA(b, launch_track_batch(b->d_eval, b->d_prefix + kv * (n + 1), n, b->d_queue + kv, kv, kTrkCap,
-                                            b->trk_tabc[kv], b->trk_grid[kv], s));
-    if (b->bricks)
-        PSC_BCUDA(b, launch_eval_batch(b->d_eval, b->d_prefix, n, b->d_queue, b->threads, b->eval_dyn, b->grid,
-                                       b->stacked, b->split, s));
+    for (int q = 0; q < kFused; ++q) {
+        const psc_batch::Fused &f = b->fused[q];
+        const long long *prefix = b->d_prefix + q * (n + 1);
+        unsigned long long *queue = b->d_queue + q;
+        if (f.grid == 0) continue;
+        if (q == kTrack1 || q == kTrack2)
+            PSC_BCUDA(b, launch_track_batch(b->d_eval, prefix, n, queue, q == kTrack1 ? 1 : 2, kTrkCap, f.tabc, f.grid, s));
+        else
+            PSC_BCUDA(b, launch_eval_batch(b->d_eval, prefix, n, queue, f.threads, f.dyn, f.grid, b->stacked, q == kShared, s));
+    }
     return PSC_OK;
 }
 
@@ -1702,7 +1709,7 @@ psc_status launch_fused(psc_batch *b) {
 psc_status enqueue_iteration(psc_batch *b) {
     const int n = (int)b->ctxs.size();
     cudaStream_t s = b->stream;
-    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, 3 * sizeof(unsigned long long), s));
+    PSC_BCUDA(b, cudaMemsetAsync(b->d_queue, 0, kFused * sizeof(unsigned long long), s));
     if (b->prof) {
         while (b->ev_pool.size() < b->ev_used + 2) {
             cudaEvent_t e;
@@ -2022,7 +2029,7 @@ psc_status psc_batch_autotune(psc_batch *b, int *tiling_out) {
             float ms = 0.f;
             for (int r = 0; r < 2 && st == PSC_OK; ++r) {             // warm, then timed
                 if (r == 1) e = cudaEventRecord(e0, b->stream);
-                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, 3 * sizeof(unsigned long long), b->stream);
+                if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue, 0, kFused * sizeof(unsigned long long), b->stream);
                 if (e == cudaSuccess) st = launch_fused(b);
                 if (r == 1 && e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
             }
@@ -2203,9 +2210,11 @@ const char *psc_batch_kernel(const psc_batch *b) {
         return s;
     }();
     if (!b) return "";
-    int set = b->trk_grid[1] ? 8 : 0;
-    if (b->trk_grid[2]) set |= 16;
-    if (b->bricks) set |= b->stacked ? 2 : b->split ? 4 : 1;
+    int set = 0;
+    if (b->fused[kBricks].grid) set |= b->stacked ? 2 : 1;
+    if (b->fused[kShared].grid) set |= 4;
+    if (b->fused[kTrack1].grid) set |= 8;
+    if (b->fused[kTrack2].grid) set |= 16;
     return names[set].c_str();
 }
 

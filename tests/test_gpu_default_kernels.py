@@ -91,6 +91,7 @@ BRICKS, SHARED_ROWS = "eval_kernel<false, false, false>", "eval_kernel<false, fa
 @pytest.mark.parametrize("shapes,name", [
     ((ONE, TWO), "track_kernel<1> + track_kernel<2>"), ((FLAT, TWO), BRICKS + " + track_kernel<2>"),
     ((RECT, FLAT), BRICKS), ((SHARED, SHARED), SHARED_ROWS),
+    ((RECT, SHARED, ONE), BRICKS + " + " + SHARED_ROWS + " + track_kernel<1>"),      # each at its own registers
 ])
 def test_the_kernels_of_a_batch_by_name(shapes, name):
     b = _batch([_problem(*s) for s in shapes])
