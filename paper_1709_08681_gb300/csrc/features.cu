@@ -163,7 +163,7 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, uns
         const unsigned tab_adj = (unsigned)__cvta_generic_to_shared(tab) - (0x4B000000u << 3);
         const float ov = (float)a.ov;
         const float rmax = ch.rho_max;
-        const float rmax2 = rmax * rmax;
+        const float rmax2 = __fmul_rn(rmax, rmax);
         const int b_lo = max(0, (int)floorf(hy - rmax) + 1);
         const int b_hi = min(a.support - 1, (int)ceilf(hy + rmax) - 1);
         float stp_s, stp_c;
@@ -171,13 +171,19 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, uns
         const int pitch = ring_pitch(a.ring);
         const bool ring = !staged && a.ring > 0;
         const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(s_big) + (uint32_t)(2 * tid * pitch);
-        // copies row b's cells within rho_max, from an even column, into the lane's ring row
-        auto fetch = [&](int b) {
+        // the columns lo .. hi of row b that lie within rho_max (none: hi < lo)
+        auto span = [&](int b, int &lo, int &hi) {
             const float dy = hy - (float)b;
-            const float rem = rmax2 - dy * dy;
+            const float rem = fmaf(-dy, dy, rmax2);
+            lo = 0;
+            hi = -2;                                 // no cell, from an odd column either
             if (!(rem > 0.f)) return;
-            const float r = fminf(rem * rsqrt_fast(rem), rmax);
-            const int lo = max(0, (int)floorf(hx - r) + 1), hi = min(a.support - 1, (int)ceilf(hx + r) - 1);
+            const float r = fminf(rem * rsqrt_fast(rem), rmax);     // keeps the span inside the staged box
+            lo = max(0, (int)floorf(hx - r) + 1);
+            hi = min(a.support - 1, (int)ceilf(hx + r) - 1);
+        };
+        // copies row b's cells of that span, from an even column, into the lane's ring row
+        auto fetch = [&](int b, int lo, int hi) {
             const int gy = iy0 + b, x0 = (ix0 + lo) & ~1, x1 = ix0 + hi;
             const uint32_t dst = ring0 + (uint32_t)((b & 1) * pitch);
             const float2 *src = a.grid + (size_t)min(max(gy, 0), a.ng - 1) * a.ng;
@@ -187,17 +193,20 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, uns
                 cp_cells(dst + (uint32_t)(x - x0) * 8u, src + (in ? x : 0), in ? 16 : 0);
             }
         };
-        if (ring && b_lo <= b_hi) fetch(b_lo);
+        // A row's span is computed once, for its copy and for the taps that read it: formed
+        // at both places, it might be rounded differently, and the copy's origin with it
+        int n_lo = 0, n_hi = -2;
+        if (b_lo <= b_hi) span(b_lo, n_lo, n_hi);
+        if (ring) fetch(b_lo, n_lo, n_hi);
         asm volatile("cp.async.commit_group;" ::: "memory");
         for (int b = b_lo; b <= b_hi; ++b) {
-            if (ring && b < b_hi) fetch(b + 1);
+            const int a_lo = n_lo, a_hi = n_hi;
+            n_hi = n_lo - 2;
+            if (b < b_hi) span(b + 1, n_lo, n_hi);
+            if (ring) fetch(b + 1, n_lo, n_hi);
             asm volatile("cp.async.commit_group;\ncp.async.wait_group 1;" ::: "memory");
+            if (a_lo > a_hi) continue;
             const float dy = hy - (float)b;
-            const float rem = rmax2 - dy * dy;
-            if (!(rem > 0.f)) continue;
-            const float r = fminf(rem * rsqrt_fast(rem), rmax);     // keeps the span inside the staged box
-            const int a_lo = max(0, (int)floorf(hx - r) + 1);
-            const int a_hi = min(a.support - 1, (int)ceilf(hx + r) - 1);
             const float dyo = dy * ov;
             const float dyo2 = fmaf(dyo, dyo, 1e-20f);
             float dxo = (hx - (float)a_lo) * ov;
