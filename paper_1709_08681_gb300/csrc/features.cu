@@ -215,12 +215,13 @@ __device__ __forceinline__ void stencil_brick(const StencilArgs &a, int blk, uns
             float Rr[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, Ri[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
             float qr = 0.f, qi = 0.f;
             // the row's first tap: in the tile or in the ring
-            const uint32_t cell0 = staged ? (uint32_t)__cvta_generic_to_shared(s_tile + (iy0 - by0 + b) * kTile + (ix0 - bx0 + a_lo))
-                                          : ring0 + (uint32_t)((b & 1) * pitch + ((ix0 + a_lo) & 1) * 8);
+            // (plain loads, which stay behind the waits above)
+            const float2 *cells = staged ? s_tile + (iy0 - by0 + b) * kTile + (ix0 - bx0 + a_lo)
+                                         : reinterpret_cast<const float2 *>(s_big + (2 * tid + (b & 1)) * pitch) + ((ix0 + a_lo) & 1);
             for (int aa = a_lo; aa <= a_hi; ++aa) {
                 float2 g;
                 if (staged || ring) {
-                    g = lds_f2(cell0 + (uint32_t)(aa - a_lo) * 8u);
+                    g = cells[aa - a_lo];
                 } else {
                     const int gx = ix0 + aa, gy = iy0 + b;
                     g = make_float2(0.f, 0.f);
