@@ -535,6 +535,7 @@ __device__ bool solve_damped(const LMArgs &a, const double *src, double lam, con
         rmax = block_max(rmax, s_tmp);
         if (rmax <= kRefineTol * bmax) return true;
     }
+    sys_sync<kLarge>();                                  // the fallback writes over r, which others may still read
     return false;
 }
 
