@@ -184,11 +184,17 @@ psc_status psc_uvw(int n_ant, const double *ant_enu_m, double lat_rad, double de
  * TMA) with a temporary workspace of 6 N K + 24 Ng K bytes, K = N rounded
  * up to a multiple of 32; otherwise FP32 SIMT with a temporary complex64
  * [N][Ng].  Synchronises the stream before returning; the workspaces of this
- * and the other model-grid calls come from a pool of the library's own, which keeps up to
- * 128 MB between calls until the last psc_ctx is destroyed.  PSC_ERR_TIMEOUT if a
+ * and the other model-grid calls come from a pool of the library's own for the CUDA
+ * context, which keeps up to 128 MB between calls until the last psc_ctx of that CUDA
+ * context is destroyed or psc_release_workspace is called.  PSC_ERR_TIMEOUT if a
  * tensor-core wait ran out. */
 psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void *grid_out,
                           void *stream);
+
+/* Gives back what the model-grid calls' pool of the current CUDA context holds between
+ * calls (the next of them allocates again).  Safe beside calls of other threads.
+ * Errors: PSC_ERR_CUDA. */
+psc_status psc_release_workspace(void);
 
 /* V° of a model given as n_comp point components (comp_lmS: host
  * [n_comp][3] = l, m (radians), S (Jy)): G[gy][gx] = sum_k S_k

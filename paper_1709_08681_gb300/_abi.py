@@ -26,7 +26,7 @@ PSC_ORDER_BASELINE, PSC_ORDER_UV = 0, 1
 PSC_LM_FULL, PSC_LM_BLOCK = 0, 1
 STOP_REASONS = {0: "none", 1: "step", 2: "chi2", 3: "lambda", 4: "max_iter", 5: "numeric"}
 
-EXPORTS = ("psc_solve_opts_default", "psc_model_grid", "psc_model_grid_components", "psc_snapshot_plane",
+EXPORTS = ("psc_solve_opts_default", "psc_model_grid", "psc_release_workspace", "psc_model_grid_components", "psc_snapshot_plane",
            "psc_snapshot_components", "psc_wstack_components", "psc_wstack_range", "psc_model_grid_wstack",
            "psc_set_wstack", "psc_create", "psc_destroy", "psc_last_error",
            "psc_predict", "psc_residual_grad", "psc_solve_offsets", "psc_lm_begin", "psc_lm_iterate",
@@ -102,6 +102,7 @@ def lib():
         path = _build.build()
         L = ctypes.CDLL(path)
         sig = {
+            "psc_release_workspace": (ctypes.c_int, []),
             "psc_solve_opts_default": (None, [ctypes.POINTER(psc_solve_opts)]),
             "psc_model_grid": (ctypes.c_int, [ctypes.POINTER(psc_grid_desc), _V, _V, _V]),
             "psc_model_grid_components": (ctypes.c_int, [ctypes.c_int, _D, ctypes.c_int, ctypes.c_double, _V, _V]),
@@ -245,6 +246,11 @@ def psc_solve_opts_default() -> psc_solve_opts:
 def psc_model_grid(n_img, n_grid, cell_rad, support, oversample, image_dev, grid_out, stream=None):
     gd = psc_grid_desc(n_img, n_grid, cell_rad, support, oversample)
     _check(lib().psc_model_grid(ctypes.byref(gd), _ptr(image_dev), _ptr(grid_out), _stream(stream)))
+
+
+def psc_release_workspace():
+    """Gives back the device memory that the model-grid calls keep between calls."""
+    _check(lib().psc_release_workspace())
 
 
 def psc_model_grid_components(comp_lmS, n_grid, cell_rad, grid_out, stream=None):

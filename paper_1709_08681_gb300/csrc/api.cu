@@ -44,6 +44,7 @@ struct psc_ctx {
     LMState *d_state0 = nullptr; // state written by psc_lm_begin (for psc_lm_restart)
     double *d_lm0 = nullptr;     // start offsets written by psc_lm_begin
     bool begun = false;
+    int slot = -1;               // the CUDA context it lives in (context_slot)
     int *d_done = nullptr;       // points at d_state->done
     int max_tab_len = 0;
     bool auto_shape = true;      // no tiling set: brick_shape() picks one from the sizes
@@ -149,12 +150,12 @@ cudaError_t dalloc(T **p, size_t n) {
 // Workspaces of the calls that make a model grid, from a pool of the library's own, one
 // a CUDA context: allocating and freeing 75 MB took 220 of the 790 us of
 // psc_model_grid_components.  Stream-ordered (safe with several threads and streams); up
-// to kPoolKeep bytes stay with the pool between calls and go back when the last psc_ctx
-// is destroyed.  Without a pool, cudaMalloc.
+// to kPoolKeep bytes stay with the pool between calls and go back when the CUDA context's
+// last psc_ctx is destroyed and by psc_release_workspace.  Without a pool, cudaMalloc.
 constexpr uint64_t kPoolKeep = (uint64_t)128 << 20;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kCtxSlots] = {};
-int g_live_ctx = 0;
+int g_live_ctx[kCtxSlots] = {};          // psc_ctx of each CUDA context
 
 struct Workspace {
     void *p = nullptr;
@@ -198,13 +199,12 @@ cudaError_t ws_free(Workspace *w, cudaStream_t s) {
     return e;
 }
 
-// One psc_ctx more or less; the last one's end returns what its CUDA context's pool holds.
-void count_ctx(int by) {
+// One psc_ctx more or less in CUDA context `slot`; the last one's end returns what the pool holds.
+void count_ctx(int slot, int by) {
+    if (slot < 0) return;
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    g_live_ctx += by;
-    if (g_live_ctx > 0) return;
-    const int slot = context_slot();
-    if (slot >= 0 && g_pool[slot]) cudaMemPoolTrimTo(g_pool[slot], 0);
+    g_live_ctx[slot] += by;
+    if (g_live_ctx[slot] == 0 && g_pool[slot]) cudaMemPoolTrimTo(g_pool[slot], 0);
 }
 
 void free_ctx(psc_ctx *c) {
@@ -225,8 +225,9 @@ void free_ctx(psc_ctx *c) {
     cudaFree(c->d_blsum); cudaFree(c->d_ev); cudaFree(c->d_cur); cudaFree(c->d_lm_trial);
     cudaFree(c->d_lm_cur); cudaFree(c->d_mat); cudaFree(c->d_mat32); cudaFree(c->d_rhs); cudaFree(c->d_state);
     cudaFree(c->d_state0); cudaFree(c->d_lm0);
+    const int slot = c->slot;
     delete c;
-    count_ctx(-1);
+    count_ctx(slot, -1);
 }
 
 // Largest visibility separation within one thread's kv time steps (cells).
@@ -667,6 +668,13 @@ psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void 
     return PSC_OK;
 }
 
+psc_status psc_release_workspace(void) {
+    const int slot = context_slot();
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    const cudaError_t e = slot >= 0 && g_pool[slot] ? cudaMemPoolTrimTo(g_pool[slot], 0) : cudaSuccess;
+    return e == cudaSuccess ? PSC_OK : cuda_fail(nullptr, e, "psc_release_workspace");
+}
+
 psc_status psc_model_grid_components(int n_comp, const double *comp_lmS, int n_grid, double cell_rad,
                                      void *grid_out, void *stream) {
     if (n_comp < 0 || n_comp > (1 << 24)) return fail(nullptr, PSC_ERR_ARG, "n_comp must be in [0, 2^24]");
@@ -842,7 +850,8 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
         if (!(obs->freq_hz[c] > 0.0) || !std::isfinite(obs->freq_hz[c])) return fail(nullptr, PSC_ERR_ARG, "frequencies must be > 0");
 
     psc_ctx *c = new psc_ctx();
-    count_ctx(1);
+    c->slot = context_slot();
+    count_ctx(c->slot, 1);
     c->stream = (cudaStream_t)stream;
     c->n_ant = obs->n_ant;
     c->n_bl = obs->n_ant * (obs->n_ant - 1) / 2;
