@@ -176,7 +176,8 @@ psc_status psc_uvw(int n_ant, const double *ant_enu_m, double lat_rad, double de
  * exp(+2 pi i ((gx-Ng/2)(col-N/2) + (gy-Ng/2)(row-N/2)) / Ng).
  * image_dev: device float [N][N]; grid_out: device complex64 [Ng][Ng];
  * stream: cudaStream_t or NULL.  Computed by FP32 FFTs in the output buffer
- * wherever the odd part of Ng is at most 512 (or, for N % 8 != 0, at most N),
+ * where Ng is a power of two or its odd part is short against N (N / 8 for N % 8 == 0,
+ * N / 2 otherwise, about),
  * with a temporary table of up to 8 Ng bytes unless Ng is a power of two.
  * Other sizes are two matrix products: for N % 8 == 0
  * on the tensor cores in split bfloat16 (each FP32 operand as three bfloat16

@@ -718,9 +718,8 @@ cudaError_t launch_model_grid(int n_img, int n_grid, const float *image, void *w
                               cudaStream_t s) {
     const size_t n = (size_t)n_img, ng = (size_t)n_grid;
     unsigned char *p = (unsigned char *)ws;
-    // FFT wherever the grid's odd part allows it (any power of two and all but
-    // grids of a large prime factor): 2048^2 -> 8192^2 in 345 us of kernels
-    // against 13.7 ms for the matrix products below, with half the error.
+    // FFT where the grid's odd part is short (2048^2 -> 8192^2 in 345 us of kernels
+    // against 13.7 ms for the matrix products below, with half the error).
     if (model_grid_fft_ok(n_img, n_grid)) {
         *err_dev = nullptr;
         return model_grid_fft(n_img, n_grid, image, ws, grid_out, s);

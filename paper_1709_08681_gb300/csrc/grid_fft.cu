@@ -44,7 +44,6 @@ namespace {
 constexpr int kE = 16;                // elements per thread
 constexpr int kMaxPass = 5;           // ceil(log2(16384) / 3)
 constexpr int kWide = 8192;           // longest transform that takes radix 16 (512 threads of up to 128 registers)
-constexpr int kMaxOdd = 512;          // longest direct DFT of any image
 
 struct FftPlan {
     int n, odd, n_pass;
@@ -324,14 +323,24 @@ size_t buf_bytes(int n) { return (size_t)(n + n / 16 + 1) * sizeof(float2); }
 
 }  // namespace
 
-// A direct DFT of the odd part costs that many complex multiply-adds per grid
-// cell (half of the cells are computed) at about 2e12 per second, the matrix
-// products N of them at about 1e13 (N % 8 == 0, tensor cores) or 4e12 (else):
-// transforms wherever the odd part is short, and up to N where the products
-// would run on the FP32 units.
+// A direct DFT of the odd part costs that many complex multiply-adds per grid cell, about
+// 3.4e-13 s each (half of the cells are computed), the matrix products N of them at
+// 0.6e-13 s (N % 8 == 0, tensor cores) or 2.4e-13 s (else), and launches and passes over
+// memory besides.  So transforms where (us as products and as transforms):
+//   the grid is a power of two (512 -> 8192: 1884 and 268);
+//   N % 8 == 0 and the odd part is at most N / 8 (128 -> 7680, 15: 514 and 654; 1024 ->
+//     8128, 127: 3998 and 3460; 512 -> 8128: 1882 and 3232; 64 -> 8176, 511: 366 and
+//     11733), 32 more up to 1024^2 grids, where launches count (512 -> 600, 75: 143 and 82),
+//     8 less beyond kWide, where a block fills an SM (64 -> 9216, 9: 451 and 1007);
+//   else, at most N / 2 (514 -> 8160, 255: 8110 and 6192; 30 -> 7680, 15: 506 and 656), 16
+//     less beyond kWide (30 -> 9216, 9: 703 and 1009), or N for images whose error on the
+//     FP32 units would reach 1e-6.
 bool model_grid_fft_ok(int n_img, int n_grid) {
     const int odd = make_plan(n_grid).odd;
-    return odd <= kMaxOdd || (n_img % 8 != 0 && odd <= n_img);
+    if (odd == 1) return true;
+    const bool wide = n_grid > kWide;
+    if (n_img % 8 == 0) return 8 * odd <= n_img + (n_grid <= 1024 ? 256 : wide ? -64 : 0);
+    return 2 * odd <= n_img - (wide ? 32 : 0) || (n_img > 512 && odd <= n_img);
 }
 
 // Tables of the sizes with an odd part, built by every call; none for powers of two.
