@@ -142,6 +142,8 @@ psc_status cuda_fail(psc_ctx *ctx, cudaError_t e, const char *what) {
         if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call); \
     } while (0)
 
+size_t al256b(size_t x) { return (x + 255) / 256 * 256; }
+
 template <class T>
 cudaError_t dalloc(T **p, size_t n) {
     return cudaMalloc((void **)p, sizeof(T) * (n ? n : 1));
@@ -657,8 +659,19 @@ psc_status psc_model_grid(const psc_grid_desc *gd, const float *image_dev, void 
     Workspace ws;
     int *err_dev = nullptr;
     int herr = 0;
-    const size_t ws_bytes = model_grid_ws_bytes(gd->n_img, gd->n_grid);
-    cudaError_t e = ws_bytes ? ws_alloc(&ws, ws_bytes, s) : cudaSuccess;
+    const size_t ws_bytes = al256b(model_grid_ws_bytes(gd->n_img, gd->n_grid));
+    // an image inside the grid's buffer is copied away first: the transforms write there
+    // while they still read it
+    const size_t img_bytes = sizeof(float) * (size_t)gd->n_img * gd->n_img;
+    const uintptr_t img0 = (uintptr_t)image_dev, out0 = (uintptr_t)grid_out;
+    const bool inside = img0 < out0 + sizeof(float2) * (size_t)gd->n_grid * gd->n_grid && out0 < img0 + img_bytes;
+    const size_t need = ws_bytes + (inside ? img_bytes : 0);
+    cudaError_t e = need ? ws_alloc(&ws, need, s) : cudaSuccess;
+    if (e == cudaSuccess && inside) {
+        float *copy = (float *)((unsigned char *)ws.p + ws_bytes);
+        e = cudaMemcpyAsync(copy, image_dev, img_bytes, cudaMemcpyDeviceToDevice, s);
+        image_dev = copy;
+    }
     if (e == cudaSuccess) e = launch_model_grid(gd->n_img, gd->n_grid, image_dev, ws.p, (float2 *)grid_out, &err_dev, s);
     if (e == cudaSuccess && err_dev) e = cudaMemcpyAsync(&herr, err_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
     const cudaError_t se = ws_free(&ws, s);
@@ -1371,7 +1384,6 @@ psc_status psc_features(psc_ctx *ctx, const void *vis_obs, const float *w, doubl
 
 namespace {
 
-size_t al256b(size_t x) { return (x + 255) / 256 * 256; }
 
 // Workspace layout of psc_features_batch: the argument tables, then per pair
 // its partials and per-baseline sums.
