@@ -741,7 +741,14 @@ psc_status psc_mlp_forward(psc_mlp *m, const float *x_dev, int batch, float *y_d
     psc_status st = check_batch(m, x_dev, batch);
     if (st != PSC_OK) return st;
     if (!y_dev) return mfail(m, PSC_ERR_ARG, "output is NULL");
-    return forward(m, x_dev, batch, y_dev);
+    const size_t y_bytes = sizeof(float) * (size_t)batch * kOut;
+    const uintptr_t x0 = (uintptr_t)x_dev, y0 = (uintptr_t)y_dev;
+    if (y0 >= x0 + sizeof(float) * (size_t)batch * kIn || x0 >= y0 + y_bytes) return forward(m, x_dev, batch, y_dev);
+    // outputs inside the input's buffer: written once every block has read its rows
+    st = forward(m, x_dev, batch, m->y);
+    if (st != PSC_OK) return st;
+    PSC_MCUDA(m, cudaMemcpyAsync(y_dev, m->y, y_bytes, cudaMemcpyDeviceToDevice, m->stream));
+    return PSC_OK;
 }
 
 psc_status psc_mlp_grad(psc_mlp *m, const float *x_dev, const float *t_dev, int batch, float *grad_host, double *loss) {
