@@ -365,6 +365,12 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * there are too few visibilities to fill the chip (the same sums bit for bit). */
 psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thread);
 
+/* The launch shape that an evaluation of ctx has now, set or picked by size, into
+ * shape_out[5]: the brick kernel's t_tile, c_group and vis_per_thread (flat bricks:
+ * items, 0, vis_per_thread), the lanes that share a visibility's rows (1: one), and the
+ * track kernel's vis_per_lane, 0 where the brick kernel runs (predictions always run it). */
+psc_status psc_get_shape(psc_ctx *ctx, int *shape_out);
+
 /* Flat bricks: the fused kernel's work items of a baseline are its (channel,
  * group of vis_per_thread consecutive time steps) pairs in channel-major
  * order, and a thread block takes `items` consecutive ones (one per thread),

@@ -30,7 +30,7 @@ EXPORTS = ("psc_solve_opts_default", "psc_model_grid", "psc_release_workspace", 
            "psc_snapshot_components", "psc_wstack_components", "psc_wstack_range", "psc_model_grid_wstack",
            "psc_set_wstack", "psc_create", "psc_destroy", "psc_last_error",
            "psc_predict", "psc_residual_grad", "psc_solve_offsets", "psc_lm_begin", "psc_lm_iterate",
-           "psc_lm_end", "psc_lm_restart", "psc_set_tiling", "psc_set_grid_precision", "psc_set_staging",
+           "psc_lm_end", "psc_lm_restart", "psc_set_tiling", "psc_get_shape", "psc_set_grid_precision", "psc_set_staging",
            "psc_set_kernel_model", "psc_set_flat_tiling", "psc_set_track_tiling", "psc_set_wait_limit",
            "psc_get_wait_limit", "psc_features_batch", "psc_features_batch_work", "psc_predict_dev", "psc_uvw", "psc_set_brick_order", "psc_fp32_fma_rate", "psc_profile", "psc_profile_read",
            "psc_residual_grad_noalloc", "psc_batch_create", "psc_batch_destroy", "psc_batch_last_error",
@@ -128,6 +128,7 @@ def lib():
             "psc_lm_iterate": (ctypes.c_int, [_V, _V, _V, ctypes.c_double, ctypes.c_int]),
             "psc_lm_end": (ctypes.c_int, [_V, _D, ctypes.POINTER(psc_solve_report)]),
             "psc_lm_restart": (ctypes.c_int, [_V]),
+            "psc_get_shape": (ctypes.c_int, [_V, ctypes.POINTER(ctypes.c_int)]),
             "psc_set_tiling": (ctypes.c_int, [_V, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
             "psc_set_grid_precision": (ctypes.c_int, [_V, ctypes.c_int]),
             "psc_set_staging": (ctypes.c_int, [_V, ctypes.c_int]),
@@ -374,6 +375,12 @@ class Context:
 
     def psc_set_tiling(self, t_tile=0, c_group=0, vis_per_thread=0):
         _check(lib().psc_set_tiling(self.h, int(t_tile), int(c_group), int(vis_per_thread)), self.h)
+
+    def psc_get_shape(self):
+        """(t_tile or items, c_group or 0, vis_per_thread, lanes per visibility, vis_per_lane or 0) of an evaluation."""
+        out = (ctypes.c_int * 5)()
+        _check(lib().psc_get_shape(self.h, out), self.h)
+        return tuple(out)
 
     def psc_set_staging(self, mode):
         _check(lib().psc_set_staging(self.h, int(mode)), self.h)

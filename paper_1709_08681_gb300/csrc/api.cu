@@ -1040,6 +1040,18 @@ psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thr
     return PSC_OK;
 }
 
+psc_status psc_get_shape(psc_ctx *ctx, int *shape_out) {
+    if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
+    if (!shape_out) return fail(ctx, PSC_ERR_ARG, "shape_out is NULL");
+    const Shape s = eval_shape(ctx);
+    shape_out[0] = s.flat > 0 ? s.flat : s.t_tile;
+    shape_out[1] = s.flat > 0 ? 0 : s.c_group;
+    shape_out[2] = s.kv;
+    shape_out[3] = s.split;
+    shape_out[4] = s.trk_kv;
+    return PSC_OK;
+}
+
 psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread) {
     if (!ctx) return fail(nullptr, PSC_ERR_ARG, "ctx is NULL");
     if (ctx->kernel_model != PSC_KERNEL_GAUSS && vis_per_thread != 1)

@@ -97,3 +97,35 @@ def test_the_kernels_of_a_batch_by_name(shapes, name):
     b = _batch([_problem(*s) for s in shapes])
     assert b.psc_batch_kernel() == name
     b.close()
+
+
+# the shapes of test_gpu_auto_shape.py, one more, and what is picked for each: (grid, dish m, antennas,
+# times, channels, hours, extent m), (t_tile or items, c_group, per thread, lanes, track)
+LARGE, SMALL = ("disk", 64, 24.0, 1024), ("disk", 512, 5.0, 1024)
+PICKED = [
+    (LARGE, 25.0, 7, 40, 5, 1.0, 300.0, (32, 4, 1, 16, 0)), (LARGE, 25.0, 9, 60, 1, 4.0, 900.0, (32, 4, 1, 8, 0)),
+    (LARGE, 25.0, 3, 1, 1, 1.0, 300.0, (32, 4, 1, 8, 0)), (LARGE, 25.0, 12, 33, 9, 1.0, 300.0, (32, 4, 1, 16, 0)),
+    (("disk", 64, 24.0, 512), 25.0, 6, 20, 6, 1.0, 300.0, (32, 4, 1, 8, 0)),
+    (("gauss", 64, 41.25, 360), 25.0, 6, 37, 3, 1.0, 300.0, (32, 4, 1, 16, 0)),
+    (LARGE, 25.0, 30, 60, 23, 0.3, 300.0, (32, 4, 1, 1, 0)),
+    (LARGE, 20.0, 30, 201, 23, 0.3, 300.0, (256, 0, 2, 1, 0)),         # the aperture inside the window
+    (LARGE, 25.0, 30, 201, 23, 0.3, 300.0, (256, 0, 1, 1, 0)), (LARGE, 25.0, 30, 201, 23, 6.0, 300.0, (256, 0, 1, 1, 0)),
+    (SMALL, 8.0, 60, 45, 26, 0.05, 300.0, (256, 0, 1, 1, 2)), (SMALL, 8.0, 64, 20, 50, 0.02, 300.0, (32, 4, 1, 1, 1)),
+]
+
+
+@pytest.mark.parametrize("spec,diam,n_ant,nt,nc,span,extent,shape", PICKED)
+def test_the_shape_that_is_picked(spec, diam, n_ant, nt, nc, span, extent, shape):
+    import cases
+    from gpu_cases import GpuProblem
+    freqs = tuple(1.2e9 + 0.1e9 * k for k in range(nc)) if nc < 20 else tuple(np.linspace(1.2e9, 1.6e9, nc))
+    m, _, _, img = cases.problem(spec, n_ant=3, n_time=1, freqs=(1.2e9,))
+    m.uvw_m, m.freq_hz = cases.geometry(n_ant, extent, nt, span, freqs)
+    m.n_ant, m.diam_m = n_ant, diam
+    ctx = GpuProblem(m, img).ctx
+    assert ctx.psc_get_shape() == shape
+    ctx.psc_set_tiling(32, 4, 1)
+    assert ctx.psc_get_shape() == (32, 4, 1, 1, 0)
+    if nt * nc >= 64:
+        ctx.psc_set_flat_tiling(64, 1)
+        assert ctx.psc_get_shape() == (64, 0, 1, 1, 0)
