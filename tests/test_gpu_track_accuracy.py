@@ -1,5 +1,5 @@
-"""Contexts without a tiling that take the track kernel by their size are as exact as
-the rectangle (32, 4, 1): both against the FP64 oracle, on data whose residuals are
+"""Contexts without a tiling that take the track kernel or flat bricks of pairs by their
+size are as exact as the rectangle (32, 4, 1): both against the FP64 oracle, on data whose residuals are
 noise of a hundredth of the visibilities, where an error of the model's phase shows in
 chi^2 most.  Boxes that the warps stage and boxes too wide for that (taps read from the
 grid), one and two visibilities per lane.
@@ -14,22 +14,26 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-# (antennas, time steps, channels, hours, array extent in m, visibilities per lane)
-@pytest.mark.parametrize("n_ant,nt,nc,span,extent,kv", [
-    (60, 45, 26, 0.05, 300.0, 2),
-    (64, 20, 50, 0.02, 300.0, 1),
-    (60, 64, 19, 0.6, 1500.0, 2),        # the longest baselines' boxes do not fit the tile
-    (201, 8, 13, 0.7, 2200.0, 1),        # several cells a step: half of the boxes do not fit
+SMALL, LARGE = ("disk", 512, 5.0, 1024), ("disk", 64, 24.0, 1024)
+
+
+# (grid, dish m, antennas, time steps, channels, hours, array extent m, shape: per thread and per lane of the track kernel)
+@pytest.mark.parametrize("spec,diam,n_ant,nt,nc,span,extent,shape", [
+    (SMALL, 25.0, 60, 45, 26, 0.05, 300.0, (1, 2)),
+    (SMALL, 25.0, 64, 20, 50, 0.02, 300.0, (1, 1)),
+    (SMALL, 25.0, 60, 64, 19, 0.6, 1500.0, (1, 2)),      # the longest baselines' boxes do not fit the tile
+    (SMALL, 25.0, 201, 8, 13, 0.7, 2200.0, (1, 1)),      # several cells a step: half of the boxes do not fit
+    (LARGE, 12.0, 30, 201, 23, 0.3, 300.0, (2, 0)),      # flat bricks of pairs
 ])
-def test_default_is_as_exact_as_the_rectangle(n_ant, nt, nc, span, extent, kv):
+def test_default_is_as_exact_as_the_rectangle(spec, diam, n_ant, nt, nc, span, extent, shape):
     import cases
     import torch
     from gpu_cases import GpuProblem
     from oracle import psc
-    from paper_1709_08681_gb300 import _abi, inputs as I
-    m, _, _, img = cases.problem(("disk", 512, 5.0, 1024), n_ant=3, n_time=1, freqs=(1.2e9,))
+    from paper_1709_08681_gb300 import inputs as I
+    m, _, _, img = cases.problem(spec, n_ant=3, n_time=1, freqs=(1.2e9,))
     m.uvw_m, m.freq_hz = cases.geometry(n_ant, extent, nt, span, tuple(np.linspace(1.2e9, 1.6e9, nc)))
-    m.n_ant, m.diam_m = n_ant, 25.0
+    m.n_ant, m.diam_m = n_ant, diam
     gp = GpuProblem(m, img)
     m.grid = gp.grid.cpu().numpy().astype(np.complex128)
     lm = np.random.default_rng(n_ant).normal(0, 1e-4, (n_ant, 2))
@@ -40,13 +44,11 @@ def test_default_is_as_exact_as_the_rectangle(n_ant, nt, nc, span, extent, kv):
     w_scale = float(np.float32(1.0 / sigma ** 2))
     exact = psc.chi2_grad_normal(m, lm, vis.astype(np.complex128), np.full(V.shape, w_scale))
     dev = gp.upload(vis)
-    b = _abi.Batch([gp.ctx], [dev], None, [w_scale])
-    assert b.psc_batch_kernel() == "track_kernel<%d>" % kv
-    b.close()
+    assert gp.ctx.psc_get_shape()[2::2] == shape
     auto = gp.ctx.psc_residual_grad(lm, dev, None, w_scale, cross=True)
     gp.ctx.psc_set_tiling(32, 4, 1)
     rect = gp.ctx.psc_residual_grad(lm, dev, None, w_scale, cross=True)
-    boxes = nc * len(m.uvw_m[0]) * -(-nt // (32 * kv))
+    boxes = nc * len(m.uvw_m[0]) * -(-nt // (32 * max(shape[1], 1)))
     ratio = scale / np.sqrt(np.mean(np.abs(vis - V) ** 2))
     ulp = 2.0 ** -23
     floors = (2 * ulp * ratio / np.sqrt(boxes), ulp * ratio / np.sqrt(2 * boxes / n_ant), ulp / np.sqrt(boxes), ulp / np.sqrt(boxes))
