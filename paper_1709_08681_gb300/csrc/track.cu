@@ -55,7 +55,6 @@ using namespace tap;
 constexpr int kTrkWarps = kTrkThreads / 32;
 constexpr int kBoxRows = 8;                 // rows of one TMA copy
 constexpr int kMaxBoxW = 32;                // widest staged box (cells)
-constexpr int kMaxBoxRows = 64;             // tallest: the tile in rows of 8
 constexpr unsigned kFull = 0xffffffffu;
 constexpr long long kDrainPolls = 1LL << 26;
 
@@ -280,8 +279,8 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
     __shared__ EvalArgs s_args[kTrkWarps];
     __shared__ __align__(8) unsigned long long s_mbar[kTrkWarps][2];
     __shared__ float s_mom[kTrkWarps][14][32];      // the lanes' running channel moments
-    __shared__ float4 s_q[kTrkWarps][2][32];         // per lane: first (u, v) split; (du1, dv1, wv0, wv1)
-    __shared__ float2 s_ph[kTrkWarps][kMaxBoxW + kMaxBoxRows];   // per item: phasors of columns, then of rows
+    __shared__ float4 s_q[kTrkWarps][kV][32];        // per lane: first (u, v) split; kV = 2: (du1, dv1, wv0, wv1)
+    __shared__ float2 s_ph[kTrkWarps][65];           // per item: phasors of columns 0 .. 31 and rows 0 .. 32
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool persistent = queue != nullptr;
     EvalArgs &a = s_args[warp];
@@ -304,7 +303,7 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
     long long first = 0;
     long long gi_static = (long long)blockIdx.x * kTrkWarps + warp;
     const float pi_f = 3.14159265358979f;
-    float2 *const col_ph = s_ph[warp], *const row_ph = col_ph + kMaxBoxW;
+    float2 *const col_ph = s_ph[warp], *const row_ph = col_ph + 32;
     // exp(i pi x), as the brick kernel forms its phasors
     auto phasor = [](float x) {
         float sn, cs;
@@ -355,11 +354,14 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
         // an origin, as a column's phasor times a row's, the same for every channel, like
         // the brick kernel's.  Hardware sines and a step's phasor multiplied along the rows
         // had an error common to a box, up to 8 times the brick kernel's in chi^2; exact
-        // ones take 17.83 ms where those took 17.42 (two LM iterations of 2 x 197
-        // antennas, 60 x 128; per channel instead of per item: 18.18)
+        // ones cost 2-3 % (197 antennas, 60 x 128, two per lane: 4.57 and 4.65 ms; formed
+        // per channel 4.2 %).  The table is no longer than this: with all 64 rows, and the
+        // weight kept for one visibility a lane, a block left the SM at apertures of 6.7
+        // cells (64 antennas, 200 x 16: 1722 us, 1764 now, 1907).
         __syncwarp();
         col_ph[lane] = phasor(-du * ((float)lane * L));
-        for (int r = lane; r < kMaxBoxRows; r += 32) row_ph[r] = phasor(-du * ((float)r * M));
+        row_ph[lane] = phasor(-du * ((float)lane * M));
+        if (lane == 0) row_ph[32] = phasor(-du * (32.f * M));
         __syncwarp();
         const int tb = chunk * 32 * kV + lane * kV;
         // rows of the lane's visibilities in uvs (past the interval's end: the
@@ -378,6 +380,7 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
             du1 = __fadd_rn(__fsub_rn(q1.x, q0.x), __fsub_rn(q1.y, q0.y));
             dv1 = __fadd_rn(__fsub_rn(q1.z, q0.z), __fsub_rn(q1.w, q0.w));
         }
+        const int left = nt - chunk * 32 * kV;         // time steps from the item's first on
         const float wv0 = tb < nt ? a.w_scale : 0.f;
         const float wv1 = tb + 1 < nt ? a.w_scale : 0.f;
         // the lane's running sums (see the epilogue): chi^2 and the gradient
@@ -394,11 +397,11 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
         ChanConst ch = a.chan[0];
         // per-lane item constants live in shared memory, not registers (the tap
         // loops need every register): the first visibility's (u, v) split,
-        // read for every channel's box, and (du1, dv1, weight 0, weight 1)
+        // read for every channel's box, and (du1, dv1, weight 0, weight 1) of two
         const float4 &q00 = s_q[warp][0][lane];
-        const float4 &qd = s_q[warp][1][lane];
+        const float4 &qd = s_q[warp][kV - 1][lane];
         s_q[warp][0][lane] = uvs0[0];
-        s_q[warp][1][lane] = make_float4(du1, dv1, wv0, wv1);
+        if constexpr (kV == 2) s_q[warp][1][lane] = make_float4(du1, dv1, wv0, wv1);
         Box box = chan_box(q00, ch.sc_hi, ch.sc_lo, half, ch.rho_max + fmaf(sp_m, ch.sc_hi, 1e-3f));
         bool ok = true;
         // issues the copies of channel cc (box bx, table length tl) into buffer bb
@@ -466,7 +469,8 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
             for (int v = 0; v < kV; ++v) {
                 const size_t k = kb0 + (size_t)v * kstep + c;
                 vo[v] = a.vis_obs[k];
-                wk[v] = (v == 0 ? qd.z : qd.w) * (a.w != nullptr ? a.w[k] : 1.f);
+                const float wv = kV == 2 ? (v == 0 ? qd.z : qd.w) : lane < left ? a.w_scale : 0.f;
+                wk[v] = wv * (a.w != nullptr ? a.w[k] : 1.f);
             }
             const float rmax = ch.rho_max, rmax2 = rmax * rmax;
             const int W = box_width(box);
@@ -489,8 +493,13 @@ track_kernel(const EvalArgs a0, const EvalArgs *__restrict__ args, const long lo
                     const float2 zcol = col_ph[col];
                     uint32_t cell = tile + (uint32_t)(r * W + col) * 8u;
                     const uint32_t cstep = (uint32_t)(rstep * W) * 8u;
-                    for (; r < rows; r += rstep, cell += cstep)
+                    for (; r < min(rows, 32); r += rstep, cell += cstep)
                         sts_f2(cell, cmul(lds_f2(cell), cmul(zcol, row_ph[r])));
+                    if (r < rows) {                    // boxes of 8 columns, up to 64 rows
+                        const float2 z = cmul(zcol, row_ph[32]);
+                        for (; r < rows; r += rstep, cell += cstep)
+                            sts_f2(cell, cmul(lds_f2(cell), cmul(z, row_ph[r - 32])));
+                    }
                 }
                 __syncwarp();
 #pragma unroll
