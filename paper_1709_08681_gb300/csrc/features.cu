@@ -40,6 +40,7 @@ constexpr int kTabPad = 2;
 constexpr int kSRed = 56;                 // X[25], Y[25], Z, g_l, g_m, H_ll, H_lm, H_mm
 constexpr int kRingMax = 34;              // widest ring row (cells): wider apertures read the grid per tap
 constexpr size_t kRingSmem = 200 * 1024;  // most dynamic shared memory of a block with rings
+constexpr size_t kRingStaged = 52 * 1024; // the same where bricks may be staged: four blocks an SM
 
 // Bytes of one lane's row: 16 more than the cells, which spreads the lanes over the banks.
 __host__ __device__ inline int ring_pitch(int cells) { return cells * 8 + 16; }
@@ -451,11 +452,15 @@ __global__ void features_batch_kernel(const FeatPair *__restrict__ pairs, float 
 }  // namespace
 
 // Cells of a ring row: an aperture's width, rounded out to 16-byte chunks; no ring
-// for apertures beyond 16 cells, grids that are not 16-byte aligned, or where the
-// rings would not fit beside the channel tables.
+// for apertures beyond 16 cells, grids that are not 16-byte aligned, where the rings
+// would not fit beside the channel tables, or where bricks may be staged and rings would
+// keep the registers' four blocks from an SM: staged bricks do without rings but have
+// their memory (27 antennas, 60 x 64, 13 cells: 1236 us, 1382 with rings; 64 antennas,
+// 60 x 16, 7 cells: 980, 1059 without).
 int stencil_ring(const StencilArgs &a, int threads) {
     const int w = (2 * (a.max_tab_len - 1) / a.ov + 3) & ~1;
     const size_t need = stencil_tab_bytes(a.c_group, a.max_tab_len) + 2 * (size_t)threads * ring_pitch(w);
+    if (a.stage && need > kRingStaged) return 0;
     return w <= kRingMax && ((uintptr_t)a.grid & 15) == 0 && need <= kRingSmem ? w : 0;
 }
 
