@@ -202,10 +202,11 @@ psc_status psc_release_workspace(void);
  * exp(+2 pi i ((gx-Ng/2) du l_k + (gy-Ng/2) du m_k)), du = 1 / (n_grid
  * cell_rad) -- for sources at pixel centres the same grid as psc_model_grid
  * of their image.  One complex matrix product on the tensor cores (split
- * bfloat16 as psc_model_grid; operands from FP64 sincospi; the component
- * count padded to a multiple of 32 with zero flux).  grid_out: device
- * complex64 [n_grid][n_grid].  Temporary workspace of 24 n_grid K bytes, K
- * the padded count.  Synchronises.  Errors: PSC_ERR_ARG (sizes, NULL or
+ * bfloat16 as psc_model_grid; operands as products of phasors from FP64 sincospi,
+ * held as pairs of FP32; the component count padded to a multiple of 32 with zero
+ * flux) over the rows v < 0, whose mirror images are the others (the fluxes are real).
+ * grid_out: device complex64 [n_grid][n_grid].  Temporary workspace of 18 n_grid K
+ * bytes, K the padded count.  Synchronises.  Errors: PSC_ERR_ARG (sizes, NULL or
  * non-finite input), PSC_ERR_CUDA / PSC_ERR_OOM, PSC_ERR_TIMEOUT (a
  * tensor-core wait ran out). */
 psc_status psc_model_grid_components(int n_comp, const double *comp_lmS, int n_grid, double cell_rad,
@@ -257,7 +258,7 @@ psc_status psc_snapshot_components(int n_comp, const double *comp_in, double a, 
  * psc_model_grid_wstack: the n_planes (>= 2) grids, each as
  * psc_model_grid_components with the plane's complex fluxes, into grids_out
  * (device complex64 [n_planes][n_grid][n_grid], caller-owned).  Temporary
- * workspace as psc_model_grid_components.  Synchronises.  Errors as
+ * workspace of 24 n_grid K bytes (complex fluxes: all rows).  Synchronises.  Errors as
  * psc_model_grid_components, plus PSC_ERR_ARG for n_planes or dw.
  * psc_set_wstack: the context degrids from the stack (borrowed like the grid of
  * psc_create, planes [n_planes][Ng][Ng] of the context's grid size) instead of
@@ -270,7 +271,7 @@ psc_status psc_snapshot_components(int n_comp, const double *comp_in, double a, 
  * Gaussian kernel model and FP32 grid only: this call refuses a
  * context with the exact kernel or the BF16 grid copy, psc_set_kernel_model
  * and psc_set_grid_precision refuse those while a stack is set.  A batch
- * takes either only stacked contexts (its persistent launch then runs the
+ * takes either only stacked contexts (its brick launch then runs the
  * stacked kernel) or none.  psc_features reads the context's own grid.
  * Synchronises. */
 psc_status psc_wstack_components(int n_comp, const double *comp_in, double a, double b, const psc_aperture *ap,
@@ -635,9 +636,9 @@ psc_status psc_batch_restart(psc_batch *b);
 psc_status psc_batch_iterate(psc_batch *b, int n_iter);
 psc_status psc_batch_end(psc_batch *b, double *lm_out, psc_solve_report *reps);
 
-/* Timing of the batch's persistent fused launch: while enabled,
+/* Timing of the batch's persistent fused launches: while enabled,
  * psc_batch_iterate launches each iteration directly (not through the graph)
- * with a pair of CUDA events around the fused launch; psc_batch_profile_read
+ * with a pair of CUDA events around them; psc_batch_profile_read
  * synchronises, returns the summed duration (ms) and count, and clears them. */
 psc_status psc_batch_profile(psc_batch *b, int enable);
 psc_status psc_batch_profile_read(psc_batch *b, double *total_ms, int *n_launches);

@@ -287,10 +287,14 @@ int flat_span(const psc_ctx *c, int flat, int kv) {
 //     move less than half a cell a step: 27 antennas, 150 x 64: 731 against 997 for
 //     rectangles of 32 x 4 (one visibility each: 843); 64 antennas at 1.8 cells a
 //     step, 173 x 16: 1413 (two: 1499) against 1734;
-//   below, the rectangles, in whose sums a solve's stop rule and so its last digits
-//     depend on every bit, with the rows of a visibility shared among up to 16 lanes
+//   below, the rectangles, with the rows of a visibility shared among up to 16 lanes
 //     while the chip would not be full otherwise (at most one lane per two rows, at
 //     least 4): the same sums, see eval.cu.
+// The line is a choice, not where the flat bricks begin to win (27 antennas: 659 us for
+// 89 x 64 as rectangles, 516 for 90 x 64 as flat bricks).  A solve ends once a step is
+// within its tolerance, so where it ends, by up to that tolerance (1e-6 to 1e-4 of the
+// offsets), follows from every bit of its sums: below the line they are the rectangle's,
+// whatever the sizes; above it another order of them, as exact, is worth its time.
 // Stacks of grids take flat bricks of 128 from the same size on.  A brick spans at most
 // 8 channels (its tables' shared memory), else the rectangle.
 constexpr double kLargeVis = 2e6;

@@ -57,7 +57,7 @@ struct EvalArgs {
     // holds items [b flat, (b + 1) flat), so bpb bricks per baseline, each
     // spanning at most ch_span channels.
     int flat, n_tp, bpb, ch_span;
-    int split;                 // rectangular bricks: lanes that share a visibility's rows (1, or 4 .. 32, a power of two)
+    int split;                 // rectangular bricks: lanes that share a visibility's rows (1, 4, 8 or 16)
     // nullptr, or [n_bl]: the baseline of each group of bpb consecutive bricks in
     // launch order (partials stay indexed by baseline: brick = bl * bpb + j)
     const int *bl_order;
