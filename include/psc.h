@@ -354,7 +354,8 @@ psc_status psc_lm_restart(psc_ctx *ctx);
  * rounded up to a multiple of 32).  t_tile in [1, 256], c_group in [1, 8],
  * t_tile * c_group <= 256, vis_per_thread in {1, 2}.  vis_per_thread = 2
  * shares each staged grid cell between the thread's two visibilities; it is
- * refused (PSC_ERR_ARG) unless every channel's aperture lies inside the
+ * refused (PSC_ERR_ARG) unless every u and v was finite (and below 2^22 grid
+ * cells) when psc_create read it, every channel's aperture lies inside the
  * S x S tap window and consecutive time steps move a baseline by at most 4
  * grid cells at the highest frequency.  Results do not depend on the shape
  * beyond FP32 rounding.
@@ -405,7 +406,8 @@ psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread);
  * it picks this kernel by size) or the first call with vis_per_lane > 0 builds the tensor maps of the grid and per-channel
  * tables (a few KB; synchronises the stream).  Errors: PSC_ERR_ARG when the
  * context uses the exact kernel, a residual-w stack or the BF16 grid copy, a
- * grid not 16-byte aligned, an aperture reaching outside the S x S window,
+ * grid not 16-byte aligned, a baseline that is not finite (or 2^22 cells or
+ * longer), an aperture reaching outside the S x S window,
  * or (vis_per_lane 2) consecutive time steps more than 4 cells apart.
  * Results equal the brick kernel's up to FP32 rounding (positions, taps and sums
  * are ordered differently; the phases are formed alike). */

@@ -73,7 +73,7 @@ struct psc_ctx {
     std::vector<int> h_tab_off, h_tab_len;   // radial table layout per channel
     double rho_top = 0.0;        // aperture radius at the top channel (cells)
     double step_cells = 0.0;     // largest move of a baseline between time steps (cells, top channel)
-    bool multi_ok = false;       // kv > 1 allowed: every channel's aperture fits inside the S x S window
+    bool multi_ok = false;       // kv > 1 and the track kernel allowed: the aperture inside the S x S window, baselines finite
     LMState h_state{};
     std::vector<double> h_ev;
     std::string err;
@@ -232,6 +232,9 @@ void free_ctx(psc_ctx *c) {
     count_ctx(slot, -1);
 }
 
+// Baselines of multi_ok contexts end here (cells): their positions' fractions are exact far beyond any grid.
+constexpr double kFarCells = 1 << 22;
+
 // Largest visibility separation within one thread's kv time steps (cells).
 double kv_spread(const psc_ctx *c, int kv) { return (kv - 1) * c->step_cells; }
 
@@ -265,7 +268,7 @@ std::string trk_refusal(const psc_ctx *c, int kv) {
     if (c->wp_n > 0) return "the track kernel does not read a residual-w stack";
     if (c->d_grid_bf16) return "the track kernel reads the FP32 grid";
     if ((uintptr_t)c->grid % 16) return "the track kernel needs a 16-byte aligned grid";
-    if (!c->multi_ok) return "the track kernel needs every channel's aperture inside the S x S window";
+    if (!c->multi_ok) return "the track kernel needs finite baselines and every channel's aperture inside the S x S window";
     if (!kv_allowed(c, kv)) return "vis_per_lane 2 needs consecutive time steps within 4 cells";
     return "";
 }
@@ -915,7 +918,7 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
     double *d_freq = nullptr;
     int *d_off = nullptr, *d_len = nullptr;
     unsigned *d_step = nullptr;
-    unsigned h_step = 0;
+    unsigned h_step[2] = {0, 0};
     const size_t evn = ev_len(c->n_ant, c->n_bl);
     const int n2 = 2 * c->n_ant;
     cudaError_t e = cudaSuccess;
@@ -938,12 +941,12 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
     if (e == cudaSuccess) e = dalloc(&d_freq, c->nc);
     if (e == cudaSuccess) e = dalloc(&d_off, c->nc);
     if (e == cudaSuccess) e = dalloc(&d_len, c->nc);
-    if (e == cudaSuccess) e = dalloc(&d_step, 1);
+    if (e == cudaSuccess) e = dalloc(&d_step, 2);
     if (e == cudaSuccess) e = dalloc(&c->d_uvs, (size_t)c->nt * c->n_bl);
     if (e == cudaSuccess) e = launch_split_uv(c->uvw, (size_t)c->nt * c->n_bl, c->d_uvs, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_step, 0, sizeof(unsigned), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_step, 0, sizeof(h_step), c->stream);
     if (e == cudaSuccess) e = launch_step_max(c->uvw, c->nt, c->n_bl, d_step, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_step, d_step, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h_step, d_step, sizeof(h_step), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_chan, ch.data(), sizeof(ChanConst) * c->nc, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_pairs, pairs.data(), sizeof(int2) * c->n_bl, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_freq, obs->freq_hz, sizeof(double) * c->nc, cudaMemcpyHostToDevice, c->stream);
@@ -996,8 +999,9 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
     c->d_done = &c->d_state->done;
     c->h_ev.resize(evn);
     {
-        float step_m = 0.f;
-        std::memcpy(&step_m, &h_step, sizeof(float));
+        float step_m = 0.f, far_m = 0.f;
+        std::memcpy(&step_m, &h_step[0], sizeof(float));
+        std::memcpy(&far_m, &h_step[1], sizeof(float));
         double sc_max = 0.0, rho_top = 0.0;
         for (int k = 0; k < c->nc; ++k) {
             sc_max = std::max(sc_max, ch[k].uv_scale);
@@ -1005,7 +1009,9 @@ psc_status psc_create(psc_ctx **out, const psc_obs *obs, const psc_aperture *ap,
         }
         c->step_cells = (double)step_m * sc_max;
         c->rho_top = rho_top;
-        c->multi_ok = std::isfinite(c->step_cells) && rho_top <= 0.5 * gd->support - 1.0;
+        // a position that is not finite, or has no fraction left in FP32, would give the taps
+        // that its neighbours share an address outside the tables
+        c->multi_ok = std::isfinite(c->step_cells) && far_m * sc_max < kFarCells && rho_top <= 0.5 * gd->support - 1.0;
     }
     // room for the tables of the widest channel group, and the LM layouts
     int stride_max = tab_stride(c, 1);
@@ -1029,7 +1035,7 @@ psc_status psc_set_tiling(psc_ctx *ctx, int t_tile, int c_group, int vis_per_thr
     if (kv != 1 && ctx->kernel_model == PSC_KERNEL_EXACT_DISK)
         return fail(ctx, PSC_ERR_ARG, "the exact disk kernel takes one visibility per thread");
     if (!kv_allowed(ctx, kv))
-        return fail(ctx, PSC_ERR_ARG, "vis_per_thread 2 needs the aperture inside the S x S window and "
+        return fail(ctx, PSC_ERR_ARG, "vis_per_thread 2 needs finite baselines, the aperture inside the S x S window and "
                                       "consecutive time steps within 4 cells");
     if (tt < 1 || tt > kMaxThreads) return fail(ctx, PSC_ERR_ARG, "t_tile must be in [1, 256]");
     if (cg < 1 || cg > 8) return fail(ctx, PSC_ERR_ARG, "c_group must be in [1, 8]");
@@ -1063,7 +1069,7 @@ psc_status psc_set_flat_tiling(psc_ctx *ctx, int items, int vis_per_thread) {
     if (items < 32 || items > kMaxThreads || items % 32) return fail(ctx, PSC_ERR_ARG, "items must be 32, 64, ..., 256");
     if (!(vis_per_thread == 1 || vis_per_thread == 2)) return fail(ctx, PSC_ERR_ARG, "vis_per_thread must be 1 or 2");
     if (!kv_allowed(ctx, vis_per_thread))
-        return fail(ctx, PSC_ERR_ARG, "vis_per_thread 2 needs the aperture inside the S x S window and "
+        return fail(ctx, PSC_ERR_ARG, "vis_per_thread 2 needs finite baselines, the aperture inside the S x S window and "
                                       "consecutive time steps within 4 cells");
     if (flat_span(ctx, items, vis_per_thread) > 8)
         return fail(ctx, PSC_ERR_ARG, "a brick would span more than 8 channels (too few time steps per channel)");

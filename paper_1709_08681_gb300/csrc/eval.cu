@@ -909,18 +909,28 @@ __global__ void __launch_bounds__(32 * kEvWarps) ev_kernel(const RedArgs r0, con
     }
 }
 
-// Largest |uv(t+1) - uv(t)| over consecutive time steps and baselines.
+// Largest |uv(t+1) - uv(t)| over consecutive time steps and baselines (out_bits[0]) and
+// largest |u| or |v| (out_bits[1]; infinity if any is not finite).
 __global__ void step_max_kernel(const double *__restrict__ uvw, int nt, int n_bl, unsigned *out_bits) {
-    float m = 0.f;
-    const long long n = (long long)(nt - 1) * n_bl;
+    float m = 0.f, far = 0.f;
+    const long long n = (long long)nt * n_bl;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const double *p = uvw + 3 * k;
+        const float a = (float)fmax(fabs(p[0]), fabs(p[1]));
+        far = isfinite(p[0] + p[1]) ? fmaxf(far, a) : INFINITY;
+        if (k + n_bl >= n) continue;
         const double *q = p + 3 * (size_t)n_bl;
         const double du = q[0] - p[0], dv = q[1] - p[1];
         m = fmaxf(m, (float)sqrt(du * du + dv * dv));
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out_bits, __float_as_uint(m));   // m >= 0: bits order as values
+    for (int o = 16; o > 0; o >>= 1) {
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, o));
+    }
+    if ((threadIdx.x & 31) == 0) {                    // both >= 0: bits order as values
+        atomicMax(out_bits, __float_as_uint(m));
+        atomicMax(out_bits + 1, __float_as_uint(far));
+    }
 }
 
 __global__ void grid_to_bf16_kernel(const float2 *__restrict__ g, size_t n, unsigned *__restrict__ out) {
@@ -954,8 +964,7 @@ cudaError_t launch_grid_to_bf16(const float2 *grid, size_t n, unsigned *out, cud
 }
 
 cudaError_t launch_step_max(const double *uvw, int nt, int n_bl, unsigned *out_bits, cudaStream_t s) {
-    if (nt < 2) return cudaSuccess;
-    const long long n = (long long)(nt - 1) * n_bl;
+    const long long n = (long long)nt * n_bl;
     const int blocks = (int)std::min<long long>((n + 255) / 256, 1024);
     step_max_kernel<<<blocks, 256, 0, s>>>(uvw, nt, n_bl, out_bits);
     return cudaGetLastError();
